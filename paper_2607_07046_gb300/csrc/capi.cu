@@ -186,8 +186,6 @@ struct vt_partition {
     bool counted = false;      // counted in the model's n_partitions
     mutable int n_kv = 0;      // live KV caches of the partition (precisions are fixed while any exists)
     std::vector<int> comm_bits;   // per device: precision of its partials on the way to the combine (16: fp32)
-    uint8_t* pcodes = nullptr;    // [n_dev][D] quantized partials of the whole-token path
-    __half* pscales = nullptr;    // [n_dev][ceil(D / 32)]
     uint32_t* status = nullptr;
     // whole-stack buffers
     float* dpart = nullptr;     // [n_dev][D] decode partials (kept zero between blocks)
@@ -1060,16 +1058,7 @@ static vt_status partition_create(vt_model* m, int32_t n, const vt_range* heads,
         p->p_u = b.take<__half>((size_t)n * p->u_slot);
         VT_CUDA(cudaMemsetAsync(q, 0, bytes, st));
     }
-    // ------------------------------------------------------------------ quantized partials (communication scaling)
-    {
-        p->comm_bits.assign(n, 16);
-        const size_t nbq = (size_t)(D + kQBlock - 1) / kQBlock;
-        void* q;
-        if ((r = owned_alloc(p, align256((size_t)n * D) + align256((size_t)n * nbq * 2), &q)) != VT_OK) return bail(r);
-        Bump b{static_cast<uint8_t*>(q)};
-        p->pcodes = b.take<uint8_t>((size_t)n * D);
-        p->pscales = b.take<__half>((size_t)n * nbq);
-    }
+    p->comm_bits.assign(n, 16);
     // ------------------------------------------------------------------ decode-token kernel
     {
         TokArgs& t = p->tok_base;
@@ -2003,8 +1992,8 @@ extern "C" vt_status vt_decode_token(const vt_partition* p, vt_kv* kv, const voi
 }
 
 // The combine of one block of the whole-token path: the plain fp32 combine, or, when some
-// device's partials travel quantized (communication scaling), each such partial quantized as it
-// leaves its shard and the combine of the dequantized values (both clear the fp32 partials).
+// device's partials travel quantized (communication scaling), the combine that quantizes each such
+// partial on its way (both clear the fp32 partials).
 static vt_status combine_block(const vt_partition* p, int l, vt_block block, const CombineArgs& c, cudaStream_t st) {
     bool any = false;
     for (int b : p->comm_bits) any |= b != 16;
@@ -2012,23 +2001,17 @@ static vt_status combine_block(const vt_partition* p, int l, vt_block block, con
         VT_CUDA(launch_combine(c, st));
         return VT_OK;
     }
-    const int D = p->m->s.d_model, nbq = (D + kQBlock - 1) / kQBlock;
-    CombineQArgs q{};
+    CombineTokenQArgs q{};
     q.n = p->n_dev;
-    q.clear = 1;
-    q.count = D;
+    q.count = p->m->s.d_model;
     q.residual = c.residual;
     q.out = c.out;
     for (int d = 0; d < p->n_dev; ++d) {
         const bool empty = block == VT_BLOCK_ATTN ? p->a(l, d).h1 == p->a(l, d).h0 : p->f(l, d).c1 == p->f(l, d).c0;
         q.bits[d] = empty ? 16 : p->comm_bits[d];
-        q.fparts[d] = c.parts[d];
-        q.codes[d] = p->pcodes + (size_t)d * D;
-        q.scales[d] = p->pscales + (size_t)d * nbq;
-        if (q.bits[d] != 16)
-            VT_CUDA(launch_quantize_vec(c.parts[d], D, q.bits[d], p->pcodes + (size_t)d * D, p->pscales + (size_t)d * nbq, 1, st));
+        q.parts[d] = c.parts[d];
     }
-    VT_CUDA(launch_combine_q(q, st));
+    VT_CUDA(launch_combine_token_q(q, st));
     return VT_OK;
 }
 
@@ -2051,8 +2034,8 @@ extern "C" vt_status vt_quantize_partial(const float* partial, int64_t count, in
                                          vt_stream stream) {
     if (count < 0 || (bits != 8 && bits != 4)) return fail(VT_ERR_INVALID_ARG, "count %lld, bits %d", (long long)count, bits);
     if (count > 0 && (!partial || !codes || !scales)) return fail(VT_ERR_INVALID_ARG, "NULL pointer");
-    VT_CUDA(launch_quantize_vec(const_cast<float*>(partial), count, bits, static_cast<uint8_t*>(codes),
-                                static_cast<__half*>(scales), 0, (cudaStream_t)stream));
+    VT_CUDA(launch_quantize_vec(partial, count, bits, static_cast<uint8_t*>(codes), static_cast<__half*>(scales),
+                                (cudaStream_t)stream));
     return ok();
 }
 
@@ -2062,12 +2045,12 @@ extern "C" vt_status vt_combine_q(const void* const* codes, const void* const* s
         return fail(VT_ERR_INVALID_ARG, "bad vt_combine_q arguments");
     CombineQArgs q{};
     q.n = n;
+    q.bits = bits;
     q.count = count;
     q.residual = static_cast<const __half*>(residual);
     q.out = static_cast<__half*>(out);
     for (int s = 0; s < n; ++s) {
         if (!codes[s] || !scales[s]) return fail(VT_ERR_INVALID_ARG, "codes or scales of partial %d are NULL", s);
-        q.bits[s] = bits;
         q.codes[s] = static_cast<const uint8_t*>(codes[s]);
         q.scales[s] = static_cast<const __half*>(scales[s]);
     }

@@ -453,85 +453,69 @@ cudaError_t launch_gemv_q(int epi, const QGemvArgs& a, cudaStream_t st) {
 // stored as one int8 per value (8 bits) or two per byte (4 bits: value 2 i in the low nibble and
 // 2 i + 1 in the high nibble, each as q + 8).
 
-// One thread per block of 32 values.  clear: zero the partial after reading it (the partials of the
-// whole-token path are accumulated into zeroed buffers).
+// The scale and this lane's code of a block of 32 values, one value per lane of the warp (0 past
+// the end of the vector): every decision is the oracle's, in fp32.  A NaN takes no part in the
+// maximum and has the code 0.
+template <int QMAX>
+__device__ __forceinline__ int block_code(float v, __half& d16, float& d) {
+    const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fabsf(v), 0.f))));
+    d16 = __float2half_rn(amax / (float)QMAX);
+    d = __half2float(d16);
+    if (d == 0.f) return 0;
+    const float r = rintf(v / d);
+    return r > (float)QMAX ? QMAX : (r < (float)-QMAX ? -QMAX : (int)r);
+}
+
+// One warp per block of 32 values, one value per lane: the loads, the codes' stores and the 32
+// divisions of a block run side by side.  It is latency bound (a few KB); a thread per block, with
+// its 32 loads and divisions in a row on one CTA, took 10.5 us for a 4096-value partial.
 template <int BITS>
-__global__ void k_quantize_vec(float* __restrict__ x, int64_t n, uint8_t* __restrict__ codes, __half* __restrict__ scales,
-                               int clear) {
+__global__ void __launch_bounds__(256) k_quantize_vec(const float* __restrict__ x, int64_t n, uint8_t* __restrict__ codes,
+                                                      __half* __restrict__ scales) {
     constexpr int QMAX = BITS == 8 ? 127 : 7;
     pdl_wait();
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nb = (n + kQBlock - 1) / kQBlock;
-    if (b < nb) {
-        const int64_t e0 = b * kQBlock;
-        const int m = (int)(n - e0 < (int64_t)kQBlock ? n - e0 : (int64_t)kQBlock);
-        float v[kQBlock];
-        float amax = 0.f;
-#pragma unroll
-        for (int e = 0; e < kQBlock; ++e) {
-            v[e] = e < m ? x[e0 + e] : 0.f;
-            amax = fmaxf(amax, fabsf(v[e]));
-        }
-        const __half d16 = __float2half_rn(amax / (float)QMAX);
-        const float d = __half2float(d16);
-        scales[b] = d16;
-        int q[kQBlock];
-#pragma unroll
-        for (int e = 0; e < kQBlock; ++e) {
-            int c = 0;
-            if (d != 0.f) {
-                const float r = rintf(v[e] / d);
-                c = r > (float)QMAX ? QMAX : (r < (float)-QMAX ? -QMAX : (int)r);
-            }
-            q[e] = c;
-        }
+    const int lane = threadIdx.x & 31;
+    const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), e = b * kQBlock + lane;
+    if (b * kQBlock < n) {
+        __half d16;
+        float d;
+        const int q = block_code<QMAX>(e < n ? x[e] : 0.f, d16, d);
+        if (lane == 0) scales[b] = d16;
         if constexpr (BITS == 8) {
-            for (int e = 0; e < m; ++e) codes[e0 + e] = (uint8_t)(int8_t)q[e];
+            if (e < n) codes[e] = (uint8_t)(int8_t)q;
         } else {
-            for (int e = 0; e < m; e += 2) {
-                const uint32_t lo = (uint32_t)(q[e] + 8), hi = e + 1 < m ? (uint32_t)(q[e + 1] + 8) : 8u;
-                codes[(e0 + e) >> 1] = (uint8_t)(lo | (hi << 4));
-            }
+            const int hi = __shfl_down_sync(0xffffffffu, q, 1);  // (the code of 0 past the end)
+            if ((lane & 1) == 0 && e < n) codes[e >> 1] = (uint8_t)((uint32_t)(q + 8) | ((uint32_t)(hi + 8) << 4));
         }
-        if (clear)
-            for (int e = 0; e < m; ++e) x[e0 + e] = 0.f;
     }
     pdl_launch_dependents();
 }
 
-cudaError_t launch_quantize_vec(float* x, int64_t n, int bits, uint8_t* codes, __half* scales, int clear,
-                                cudaStream_t st) {
+cudaError_t launch_quantize_vec(const float* x, int64_t n, int bits, uint8_t* codes, __half* scales, cudaStream_t st) {
     const int64_t nb = (n + kQBlock - 1) / kQBlock;
     if (nb <= 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((nb + 127) / 128);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(128);
+    cfg.gridDim = dim3((unsigned)((nb + 7) / 8));
+    cfg.blockDim = dim3(256);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_use_pdl ? 1 : 0;
-    if (bits == 8) return cudaLaunchKernelEx(&cfg, k_quantize_vec<8>, x, n, codes, scales, clear);
-    if (bits == 4) return cudaLaunchKernelEx(&cfg, k_quantize_vec<4>, x, n, codes, scales, clear);
+    if (bits == 8) return cudaLaunchKernelEx(&cfg, k_quantize_vec<8>, x, n, codes, scales);
+    if (bits == 4) return cudaLaunchKernelEx(&cfg, k_quantize_vec<4>, x, n, codes, scales);
     return cudaErrorInvalidValue;
 }
 
-// out[e] = fp16(residual[e] + sum_s p_s[e]) with shards in order, fp32: p_s is the fp32 partial
-// (bits 16; zeroed after reading when clear is set) or the dequantized code q_s[e] d_s[e / 32].
+// out[e] = fp16(residual[e] + sum_s q_s[e] d_s[e / 32]), shards in order, fp32.
 __global__ void k_combine_q(const __grid_constant__ CombineQArgs a) {
     pdl_wait();
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.count; e += (int64_t)gridDim.x * blockDim.x) {
         float acc = a.residual ? __half2float(a.residual[e]) : 0.f;
         for (int s = 0; s < a.n; ++s) {
-            const int bits = a.bits[s];
-            if (bits == 16) {
-                acc += __ldcg(a.fparts[s] + e);
-                if (a.clear) a.fparts[s][e] = 0.f;
-                continue;
-            }
             int q;
-            if (bits == 8) {
+            if (a.bits == 8) {
                 q = (int)(int8_t)a.codes[s][e];
             } else {
                 const uint8_t byte = a.codes[s][e >> 1];
@@ -557,6 +541,55 @@ cudaError_t launch_combine_q(const CombineQArgs& a, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = g_use_pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k_combine_q, a);
+}
+
+// The combine of one decode token whose partials travel at bits[s] (16: fp32): out = fp16(residual
+// + sum_s p_s), shards in order, p_s the partial or, at 8 or 4 bits, its codes times their scale.
+// One warp per block of 32 elements quantizes each shard's block as it leaves that shard and adds
+// it at once (the same codes, scales and sums as k_quantize_vec followed by k_combine_q, which the
+// tests compare with the oracle), so a block of the layer has one launch instead of one per shard
+// and the codes need no memory.  Latency bound (n * 16 KB): the launches were what it cost (four
+// launches of 10.5 + 3.3 us per block of the layer before, COMBT_US now).  The partials are
+// cleared after reading (they are accumulated into zeroed buffers).
+__global__ void __launch_bounds__(256) k_combine_token_q(const __grid_constant__ CombineTokenQArgs a) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31;
+    const int e = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kQBlock + lane;
+    if (e - lane >= a.count) return;
+    const bool on = e < a.count;
+    float v[VT_MAX_DEVICES];
+#pragma unroll
+    for (int s = 0; s < VT_MAX_DEVICES; ++s) v[s] = on && s < a.n ? __ldcg(a.parts[s] + e) : 0.f;
+    float acc = on ? __half2float(a.residual[e]) : 0.f;
+#pragma unroll
+    for (int s = 0; s < VT_MAX_DEVICES; ++s) {
+        if (s >= a.n) break;
+        if (a.bits[s] == 16) {
+            acc += v[s];
+        } else {
+            __half d16;
+            float d;
+            const int q = a.bits[s] == 8 ? block_code<127>(v[s], d16, d) : block_code<7>(v[s], d16, d);
+            acc = fmaf((float)q, d, acc);
+        }
+        if (on) a.parts[s][e] = 0.f;
+    }
+    if (on) a.out[e] = __float2half_rn(acc);
+}
+
+cudaError_t launch_combine_token_q(const CombineTokenQArgs& a, cudaStream_t st) {
+    if (a.count <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((a.count + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g_use_pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_combine_token_q, a);
 }
 
 cudaError_t init_quant_kernels() {

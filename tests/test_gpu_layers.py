@@ -41,10 +41,11 @@ PRUNED = ([[(0, 2), (4, 6), (6, 8)], [(0, 2), (2, 2), (6, 8)], [(0, 4), (4, 6), 
           [[(0, 100), (300, 1000), (1000, 1408)], [(0, 701), (701, 701), (1000, 1408)], [(0, 700), (700, 1000), (1000, 1400)]])
 
 
-def _stack(vt, wl, cap, layer_ranges=None):
+def _stack(vt, wl, cap, layer_ranges=None, precision=None):
     from paper_2607_07046_gb300.stack import Stack
     shapes = shapes_of(vt, wl, max_seq=max(wl.max_seq, cap))
-    return Stack(shapes, wl.layer_weights, wl.head_ranges, wl.ffn_ranges, cap, layer_ranges=layer_ranges)
+    return Stack(shapes, wl.layer_weights, wl.head_ranges, wl.ffn_ranges, cap, precision=precision,
+                 layer_ranges=layer_ranges)
 
 
 def _reference_tokens(wl, heads, cols, L0, xs, caches):
@@ -173,3 +174,54 @@ def test_whole_token_with_quantized_partials(vtlib, bits):
         # back to fp32 partials: the fused kernel is available again
         vt.vt_partition_set_comm_bits(st.part, -1, 16)
         assert vt.vt_decode_token_fused_available(st.part)[0]
+
+
+@pytest.mark.parametrize("d_model,bits", [(64, (8,)), (192, (16, 4, 8)), (320, (4, 8, 16, 4)), (512, (8, 4))])
+def test_token_combine_quantizes_each_partial_on_its_way(vtlib, d_model, bits):
+    """The token's combine with a different precision per device (some fp32, the last device empty),
+    at widths that are no multiple of its 256-element CTAs: h and x_next equal, bit for bit, the
+    sums of the devices' own partials through vt_quantize_partial (FFN shards block-quantized, so
+    that every partial repeats exactly)."""
+    vt = vtlib
+    n = len(bits)
+    H, F = 2 * n, 64 * n
+    wl = synthetic.small("mixed", n_layers=1, d_model=d_model, n_heads=H, n_kv_heads=H, d_head=64, d_ffn=F,
+                         head_ranges=tuple((2 * d, 2 * d + 2) for d in range(n)) + ((H, H),),
+                         ffn_ranges=tuple((64 * d, 64 * d + 64) for d in range(n)) + ((F, F),),
+                         kv_len=9, decode_steps=1, prompt_len=0, model_id=143)
+    L0, cap = 9, 16
+    kc, vc = wl.kv_fill(0, L0, cap)
+    x = wl.hidden(1, stream=421)
+
+    def combined(residual, parts):
+        acc = residual.astype(np.float32)
+        for d, p in enumerate(parts):
+            if d >= n or bits[d] == 16:
+                acc = acc + host(p)
+                continue
+            codes = torch.empty(vt.vt_partial_code_bytes(d_model, bits[d]), dtype=torch.uint8, device="cuda")
+            scales = torch.empty((d_model + 31) // 32, dtype=torch.float16, device="cuda")
+            vt.vt_quantize_partial(p, bits[d], codes, scales)
+            raw = host(codes)
+            q = raw.view(np.int8) if bits[d] == 8 else np.stack([(raw & 15).astype(np.int8) - 8, (raw >> 4).astype(np.int8) - 8], 1).reshape(-1)
+            # code times scale is exact in fp32 (at most 7 + 11 bits), so this is the fused multiply-add
+            acc = acc + q.astype(np.float32) * np.repeat(host(scales), 32)[:d_model].astype(np.float32)
+        return acc.astype(np.float16)
+
+    with _stack(vt, wl, cap, precision=lambda l, d, b: 8 if b == vt.VT_BLOCK_FFN and d < n else 16) as st:
+        for d in range(n):
+            vt.vt_partition_set_comm_bits(st.part, d, bits[d])
+            h0, h1 = wl.head_ranges[d]
+            vt.vt_kv_write_raw(st.kv, 0, d, kc[h0:h1, :L0], vc[h0:h1, :L0])
+        vt.vt_kv_set_length(st.kv, -1, L0)
+
+        def step(block, inp, d):
+            out = torch.empty(d_model, dtype=torch.float32, device="cuda")
+            vt.vt_decode_step(st.part, (0, d, block), dev(inp), st.kv, out)
+            return out
+
+        h = combined(x.reshape(-1), [step(vt.VT_BLOCK_ATTN, x.reshape(-1), d) for d in range(n + 1)])
+        want = combined(h, [step(vt.VT_BLOCK_FFN, h, d) for d in range(n + 1)])
+        got = torch.empty(d_model, dtype=torch.float16, device="cuda")
+        vt.vt_decode_token(st.part, st.kv, dev(x.reshape(-1)), got)
+        assert np.array_equal(host(got).view(np.uint16), want.view(np.uint16))
