@@ -427,9 +427,7 @@ VT_API vt_status vt_decode_step(const vt_partition* part, vt_shard shard, const 
  *   every intermediate in one file-scope __device__ array of 1 MiB (1048576 bytes) that is part
  *   of the library's device image.  It calls no cudaMalloc, cudaFree or other allocating routine.
  *   It does not use the partition's decode scratch.
- *   Computation: as vt_decode_step for the ATTN shard.  Attention runs as split-K over 16 slices
- *   per KV head.  The slices are merged by the last one to finish, so results match
- *   vt_decode_step to rounding, not bit for bit.
+ *   Computation: the kernels of vt_decode_step for the ATTN shard, so results match its bits.
  *   Arguments, layouts, ownership: as vt_decode_step.  kv is required.  Does not advance the KV
  *   length.
  *   Limits: the shard needs 256 + 8*h_s*dh + 64*hk_s*G*(dh+2) bytes (each region rounded up to
@@ -441,8 +439,7 @@ VT_API vt_status vt_decode_step(const vt_partition* part, vt_shard shard, const 
  *   any stream capture on that device begins.  The kept address is the array's for the life of
  *   the device's primary context: do not use the library across a cudaDeviceReset (the module
  *   would load again and the array could move).
- *   Must start at zero: only the 64 per-KV-head arrival counters at the start of the array.  The
- *   module loader zeroes them, and every call leaves them at zero.
+ *   Must start at zero: nothing; every region is written before it is read within a call.
  *   Races: the array is shared by every call in the process on that device.  Two calls in flight
  *   at once, on different streams or host threads, corrupt each other.  Order them. */
 VT_API vt_status vt_decode_step_static(const vt_partition* part, vt_shard shard, const void* x, vt_kv* kv,

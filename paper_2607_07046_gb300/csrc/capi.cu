@@ -1594,6 +1594,28 @@ static cudaError_t attn_qkv(const vt_partition* p, int l, int d, const __half* x
     return launch_gemv(kEpiQkvRope, g, st);
 }
 
+// Attention of ATTN shard (l, d) over the cache: q [hq][dh] rotated queries -> attn [hq][dh].
+static cudaError_t attn_slices(const vt_partition* p, int l, int d, const float* q, vt_kv* kv, float* attn,
+                               cudaStream_t st) {
+    const vt_shapes& s = p->m->s;
+    const AttnShard& a = p->a(l, d);
+    AttnDecodeArgs t{};
+    t.q = q;
+    t.kcache = kv->k(l, d);
+    t.vcache = kv->v(l, d);
+    t.len = kv->len + l;
+    t.cap = kv->cap;
+    t.hk = a.kv1 - a.kv0;
+    t.group = s.n_heads / s.n_kv_heads;
+    t.dh = s.d_head;
+    t.stages = attn_stages(kv->cap, attn_cluster_size(t.hk));
+    t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)s.d_head));
+    t.window = p->m->window[l];
+    t.out = attn;
+    t.status = kv->status;
+    return launch_attn_decode(t, st);
+}
+
 // O projection of ATTN shard (l, d): out [D] = Wo_s . attn (fp32), fp16 or block-quantized.
 static cudaError_t attn_o(const vt_partition* p, int l, int d, const float* attn, float* out, uint32_t* status,
                           cudaStream_t st) {
@@ -1626,28 +1648,14 @@ static vt_status decode_attn(const vt_partition* p, int l, int d, const __half* 
     const vt_shapes& s = p->m->s;
     const AttnShard& a = p->a(l, d);
     const DecodeScratch& ds = p->dec[d];
-    const int hq = a.h1 - a.h0, hk = a.kv1 - a.kv0, dh = s.d_head, D = s.d_model;
+    const int hq = a.h1 - a.h0, D = s.d_model;
     if (hq == 0) {
         VT_CUDA(launch_fill_zero_f32(out, D, st));
         return VT_OK;
     }
     VT_CUDA(attn_qkv(p, l, d, x, kv, ds.q, st, indep));
 
-    AttnDecodeArgs t{};
-    t.q = ds.q;
-    t.kcache = kv->k(l, d);
-    t.vcache = kv->v(l, d);
-    t.len = kv->len + l;
-    t.cap = kv->cap;
-    t.hk = hk;
-    t.group = s.n_heads / s.n_kv_heads;
-    t.dh = dh;
-    t.stages = attn_stages(kv->cap, attn_cluster_size(hk));
-    t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)dh));
-    t.window = p->m->window[l];
-    t.out = ds.attn;
-    t.status = kv->status;
-    VT_CUDA(launch_attn_decode(t, st));
+    VT_CUDA(attn_slices(p, l, d, ds.q, kv, ds.attn, st));
     VT_CUDA(attn_o(p, l, d, ds.attn, out, kv->status, st));
     return VT_OK;
 }
@@ -1713,9 +1721,8 @@ extern "C" vt_status vt_decode_step(const vt_partition* p, vt_shard sh, const vo
     return ok();
 }
 
-// ATTN shard step with every intermediate in the module's static scratch array: the same QKV and
-// O kernels as decode_attn, with the split-K attention kernel of static_scratch.cu between them.
-// Touches neither the partition's decode scratch nor any allocator.
+// ATTN shard step with every intermediate in the module's static scratch array: the kernels of
+// decode_attn.  Touches neither the partition's decode scratch nor any allocator.
 extern "C" vt_status vt_decode_step_static(const vt_partition* p, vt_shard sh, const void* x, vt_kv* kv,
                                            float* out, vt_stream stream) {
     VT_TRY(check_shard(p, sh));
@@ -1750,23 +1757,7 @@ extern "C" vt_status vt_decode_step_static(const vt_partition* p, vt_shard sh, c
 
     VT_CUDA(attn_qkv(p, l, d, static_cast<const __half*>(x), kv, q, st, 0));
 
-    StaticAttnArgs t{};
-    t.q = q;
-    t.kcache = kv->k(l, d);
-    t.vcache = kv->v(l, d);
-    t.len = kv->len + l;
-    t.cap = kv->cap;
-    t.hk = hk;
-    t.group = s.n_heads / s.n_kv_heads;
-    t.dh = dh;
-    t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)dh));
-    t.window = p->m->window[l];
-    t.part_ml = reinterpret_cast<float*>(b + lay.part_ml);
-    t.part_o = reinterpret_cast<float*>(b + lay.part_o);
-    t.counters = reinterpret_cast<uint32_t*>(b + lay.counters);
-    t.out = attn;
-    VT_CUDA(launch_attn_decode_static(t, st));
-
+    VT_CUDA(attn_slices(p, l, d, q, kv, attn, st));
     VT_CUDA(attn_o(p, l, d, attn, out, kv->status, st));
     return ok();
 }

@@ -262,33 +262,19 @@ struct CombineTokenQArgs {               // a token's combine, partials travelli
 };
 cudaError_t launch_combine_token_q(const CombineTokenQArgs& a, cudaStream_t st);
 
-// ------------------------------------------------------------------ static-scratch decode attention
-// (static_scratch.cu) split-K decode attention whose scratch is one file-scope __device__ array.
+// ------------------------------------------------------------------ static scratch
+// (static_scratch.cu) the decode step whose intermediates are in one file-scope __device__ array.
 constexpr size_t kStaticScratchBytes = (size_t)1 << 20;  // 1 MiB
-constexpr int kStaticSplits = 16;                        // position slices per KV head
-constexpr int kStaticMaxKvHeads = 64;                    // arrival counters
+constexpr int kStaticSplits = 16;                        // slice states per KV head that the size limit counts
+constexpr int kStaticMaxKvHeads = 64;                    // KV heads of a shard that the call takes
 constexpr int kStaticMaxDevices = 64;                    // cached symbol addresses
 
-struct StaticAttnLayout {  // byte offsets of the regions in the array
-    size_t counters, q, attn, part_ml, part_o, bytes;
+struct StaticAttnLayout {  // byte offsets of the vectors in the array; bytes: what the limit counts
+    size_t q, attn, bytes;
 };
 StaticAttnLayout static_attn_layout(int hq, int hk, int dh);
 cudaError_t static_scratch_base(void** out);
 
-struct StaticAttnArgs {
-    const float* q;        // [hq][dh] rotated queries
-    const __half* kcache;  // [hk][cap][dh]
-    const __half* vcache;
-    const int32_t* len;
-    int cap, hk, group, dh;
-    float scale_log2;
-    int window;            // > 0: sliding window over the last `window` positions
-    float* part_ml;        // [hk][kStaticSplits][group][2] (max, sum) of each slice
-    float* part_o;         // [hk][kStaticSplits][group][dh] weighted V of each slice
-    uint32_t* counters;    // [hk] slices finished; zero between calls
-    float* out;            // [hq][dh]
-};
-cudaError_t launch_attn_decode_static(const StaticAttnArgs& a, cudaStream_t st);
 vt_status prefill_ffn_shard(const PrefillFfnArgs& a, cudaStream_t st, std::string* err);
 
 
