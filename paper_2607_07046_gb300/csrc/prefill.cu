@@ -249,40 +249,68 @@ __device__ __forceinline__ void store_hl8(__half* row, int d, int c, const float
     if (split) *reinterpret_cast<uint4*>(row + d + (size_t)c * 8) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
-__global__ void __launch_bounds__(256) k_rmsnorm_rows(const __half* __restrict__ x, const __half* __restrict__ gain,
-                                                      float eps, int d, __half* __restrict__ y, int split) {
-    __shared__ float red[8];
-    pdl_wait();
-    const __half* xr = x + (size_t)blockIdx.x * d;
-    __half* yr = y + (size_t)blockIdx.x * d * (split ? 2 : 1);
-    float ss = 0.f;
-    for (int c = threadIdx.x; c < d / 8; c += blockDim.x) {
-        const uint4 v = *reinterpret_cast<const uint4*>(xr + c * 8);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 f = h2_to_f2(w[e]);
-            ss = fmaf(f.x, f.x, ss);
-            ss = fmaf(f.y, f.y, ss);
-        }
-    }
+// Rows kernels: one CTA per row, MC 16-byte chunks of the row per thread, its values in registers
+// between the two passes of the norm.  With few rows the time is one row's latency and a thread
+// takes one chunk, so that the row's loads are all in flight at once (77 rows of 4096, four
+// partials: 6.1 -> 4.5 us); from two rows an SM on it is the memory rate, and two chunks leave
+// room for more CTAs (512 rows: 8.35 -> 7.9 us; one chunk a thread made the prompt 0.3% slower).
+static int row_mc(int rows, int d) { return d / 8 > 1024 || rows >= 2 * (g_num_sms > 0 ? g_num_sms : 148) ? 2 : 1; }
+static int row_threads(int mc, int d) { return ((d / 8 + mc - 1) / mc + 31) / 32 * 32; }
+
+// Sum of `ss` over the CTA (at most 32 warps), in warp order.
+__device__ __forceinline__ float block_sum(float ss, float* red) {
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
     __syncthreads();
     float tot = 0.f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-    const float r = 1.0f / sqrtf(tot / (float)d + eps);
-    for (int c = threadIdx.x; c < d / 8; c += blockDim.x) {
-        const uint4 v = *reinterpret_cast<const uint4*>(xr + c * 8);
-        const uint4 g = *reinterpret_cast<const uint4*>(gain + c * 8);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w}, gw[4] = {g.x, g.y, g.z, g.w};
-        float o[8];
+    return tot;
+}
+
+// y = v * r * gain of one chunk
+__device__ __forceinline__ void norm_chunk(const float (&v)[8], float r, uint4 g, float (&o)[8]) {
+    const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 gg = h2_to_f2(gw[e]);
+        o[2 * e] = v[2 * e] * r * gg.x;
+        o[2 * e + 1] = v[2 * e + 1] * r * gg.y;
+    }
+}
+
+template <int MC>
+__global__ void __launch_bounds__(1024) k_rmsnorm_rows(const __half* __restrict__ x, const __half* __restrict__ gain,
+                                                       float eps, int d, __half* __restrict__ y, int split) {
+    __shared__ float red[32];
+    pdl_wait();
+    const __half* xr = x + (size_t)blockIdx.x * d;
+    __half* yr = y + (size_t)blockIdx.x * d * (split ? 2 : 1);
+    float v[MC][8];
+    uint4 g[MC];
+    float ss = 0.f;
+#pragma unroll
+    for (int m = 0; m < MC; ++m) {
+        const int c = threadIdx.x + m * blockDim.x;
+        const bool on = c < d / 8;
+        const uint4 u = on ? *reinterpret_cast<const uint4*>(xr + c * 8) : make_uint4(0u, 0u, 0u, 0u);
+        g[m] = on ? *reinterpret_cast<const uint4*>(gain + c * 8) : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const float2 f = h2_to_f2(w[e]), gg = h2_to_f2(gw[e]);
-            o[2 * e] = f.x * r * gg.x;
-            o[2 * e + 1] = f.y * r * gg.y;
+            const float2 f = h2_to_f2(w[e]);
+            v[m][2 * e] = f.x;
+            v[m][2 * e + 1] = f.y;
+            ss = fmaf(f.x, f.x, ss);
+            ss = fmaf(f.y, f.y, ss);
         }
+    }
+    const float r = 1.0f / sqrtf(block_sum(ss, red) / (float)d + eps);
+#pragma unroll
+    for (int m = 0; m < MC; ++m) {
+        const int c = threadIdx.x + m * blockDim.x;
+        if (c >= d / 8) break;
+        float o[8];
+        norm_chunk(v[m], r, g[m], o);
         store_hl8(yr, d, c, o, split != 0);
     }
 }
@@ -291,67 +319,71 @@ __global__ void __launch_bounds__(256) k_rmsnorm_rows(const __half* __restrict__
 
 // One CTA per row: out = fp16(residual + sum_s parts[s]) (fp32, shards in order, as k_combine),
 // and, when gain is set, xhat = fp16(RMSNorm(out) * gain) computed from the rounded row: the input
-// every shard of the next block would normalise for itself.
-__global__ void __launch_bounds__(256) k_combine_norm(const __grid_constant__ CombineArgs a, int d,
-                                                      const __half* __restrict__ gain, float eps,
-                                                      __half* __restrict__ xhat, int split) {
-    __shared__ float red[8];
+// every shard of the next block would normalise for itself.  Bound by the partials' bytes (four
+// shards, 512 rows of 4096: 50 MB); the loads of four shards are issued before their additions.
+template <int MC>
+__global__ void __launch_bounds__(1024) k_combine_norm(const __grid_constant__ CombineArgs a, int d,
+                                                       const __half* __restrict__ gain, float eps,
+                                                       __half* __restrict__ xhat, int split) {
+    __shared__ float red[32];
     pdl_wait();
     const size_t row = blockIdx.x;
+    float v[MC][8];
     float ss = 0.f;
-    for (int c = threadIdx.x; c < d / 8; c += blockDim.x) {
+#pragma unroll
+    for (int m = 0; m < MC; ++m) {
+        const int c = threadIdx.x + m * blockDim.x;
+        if (c >= d / 8) break;
         const size_t e0 = row * d + (size_t)c * 8;
-        float acc[8];
-        if (a.residual) {
-            const uint4 r = *reinterpret_cast<const uint4*>(a.residual + e0);
-            const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+        const uint4 r = a.residual ? *reinterpret_cast<const uint4*>(a.residual + e0) : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = h2_to_f2(w[j]);
-                acc[2 * j] = f.x;
-                acc[2 * j + 1] = f.y;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+        for (int j = 0; j < 4; ++j) {
+            const float2 f = h2_to_f2(w[j]);
+            v[m][2 * j] = f.x;
+            v[m][2 * j + 1] = f.y;
         }
-        for (int sh = 0; sh < a.n; ++sh) {
-            if (!a.parts[sh]) continue;
-            const float4 p0 = __ldcg(reinterpret_cast<const float4*>(a.parts[sh] + e0));
-            const float4 p1 = __ldcg(reinterpret_cast<const float4*>(a.parts[sh] + e0 + 4));
-            acc[0] += p0.x; acc[1] += p0.y; acc[2] += p0.z; acc[3] += p0.w;
-            acc[4] += p1.x; acc[5] += p1.y; acc[6] += p1.z; acc[7] += p1.w;
+        for (int s0 = 0; s0 < a.n; s0 += 4) {
+            float4 p[4][2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float* src = s0 + i < a.n ? a.parts[s0 + i] : nullptr;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    p[i][h] = src ? __ldcg(reinterpret_cast<const float4*>(src + e0) + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (s0 + i < a.n)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        v[m][4 * h] += p[i][h].x;
+                        v[m][4 * h + 1] += p[i][h].y;
+                        v[m][4 * h + 2] += p[i][h].z;
+                        v[m][4 * h + 3] += p[i][h].w;
+                    }
         }
         uint32_t o[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const __half2 h = __floats2half2_rn(acc[2 * j], acc[2 * j + 1]);
+            const __half2 h = __floats2half2_rn(v[m][2 * j], v[m][2 * j + 1]);
             o[j] = *reinterpret_cast<const uint32_t*>(&h);
             const float2 f = __half22float2(h);
+            v[m][2 * j] = f.x;
+            v[m][2 * j + 1] = f.y;
             ss = fmaf(f.x, f.x, ss);
             ss = fmaf(f.y, f.y, ss);
         }
         *reinterpret_cast<uint4*>(a.out + e0) = make_uint4(o[0], o[1], o[2], o[3]);
     }
     if (!gain) return;
-    ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    float tot = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-    const float r = 1.0f / sqrtf(tot / (float)d + eps);
-    for (int c = threadIdx.x; c < d / 8; c += blockDim.x) {
-        // this thread's own row elements, written above
-        const uint4 hv = *reinterpret_cast<const uint4*>(a.out + row * d + (size_t)c * 8);
-        const uint4 g = *reinterpret_cast<const uint4*>(gain + c * 8);
-        const uint32_t w[4] = {hv.x, hv.y, hv.z, hv.w}, gw[4] = {g.x, g.y, g.z, g.w};
-        float o[8];
+    const float r = 1.0f / sqrtf(block_sum(ss, red) / (float)d + eps);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = h2_to_f2(w[j]), gg = h2_to_f2(gw[j]);
-            o[2 * j] = f.x * r * gg.x;
-            o[2 * j + 1] = f.y * r * gg.y;
-        }
+    for (int m = 0; m < MC; ++m) {
+        const int c = threadIdx.x + m * blockDim.x;
+        if (c >= d / 8) break;
+        float o[8];
+        norm_chunk(v[m], r, *reinterpret_cast<const uint4*>(gain + c * 8), o);
         store_hl8(xhat + row * d * (split ? 2 : 1), d, c, o, split != 0);
     }
 }
@@ -360,7 +392,9 @@ cudaError_t launch_combine_norm(const CombineArgs& a, int rows, int d, const __h
                                 int split, cudaStream_t st) {
     if (rows <= 0) return cudaSuccess;
     if (d % 8 != 0 || d > 16384) return cudaErrorInvalidValue;
-    k_combine_norm<<<rows, 256, 0, st>>>(a, d, gain, eps, xhat, split);
+    const int mc = row_mc(rows, d), t = row_threads(mc, d);
+    if (mc == 1) k_combine_norm<1><<<rows, t, 0, st>>>(a, d, gain, eps, xhat, split);
+    else k_combine_norm<2><<<rows, t, 0, st>>>(a, d, gain, eps, xhat, split);
     return cudaGetLastError();
 }
 
@@ -1814,8 +1848,10 @@ static vt_status run_gemm(const void* A, int64_t lda, const void* B, int64_t ldb
 cudaError_t launch_rmsnorm_rows(const __half* x, const __half* gain, float eps, int rows, int d, __half* y,
                                 int split, cudaStream_t st) {
     if (rows <= 0) return cudaSuccess;
-    if (d % 8 != 0) return cudaErrorInvalidValue;
-    k_rmsnorm_rows<<<rows, 256, 0, st>>>(x, gain, eps, d, y, split);
+    if (d % 8 != 0 || d > 16384) return cudaErrorInvalidValue;
+    const int mc = row_mc(rows, d), t = row_threads(mc, d);
+    if (mc == 1) k_rmsnorm_rows<1><<<rows, t, 0, st>>>(x, gain, eps, d, y, split);
+    else k_rmsnorm_rows<2><<<rows, t, 0, st>>>(x, gain, eps, d, y, split);
     return cudaGetLastError();
 }
 
