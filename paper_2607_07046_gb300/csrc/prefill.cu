@@ -197,15 +197,12 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // Shared-memory matrix descriptor of a K-major operand tile written by TMA with the 128-byte
 // swizzle: rows of 64 fp16 (128 bytes), 8-row groups 1024 bytes apart.  The tile base is 1024-byte
 // aligned; stepping K by 16 elements inside the 128-byte row advances the start address by 32 bytes.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);  // start address
-    d |= (uint64_t)1 << 16;                    // leading-dimension offset (unused with this swizzle)
-    d |= (uint64_t)(1024 >> 4) << 32;          // stride between 8-row groups
-    d |= (uint64_t)1 << 46;                    // descriptor version
-    d |= (uint64_t)2 << 61;                    // 128-byte swizzle
-    return d;
-}
+// In two halves: the constant upper word (stride between 8-row groups, descriptor version, 128-byte
+// swizzle) and the lower word of the tile at `saddr` (start address in units of 16 bytes, so that
+// stepping inside shared memory adds to it; the leading-dimension offset is unused).
+constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_sw128_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ uint64_t desc_of(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
 
 // Descriptor of an MN-major operand (the N index contiguous) written by TMA with the 128-byte
 // swizzle: each K index is one 128-byte row of 64 consecutive N elements, 8-row groups are 1024
@@ -548,10 +545,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     // and the L2 prefetch of the CTA's remaining B tiles are issued before griddepcontrol.wait, so
     // they stream while the preceding kernel finishes; A, which it wrote, is loaded after the wait.
     const int pre = nk < kStages ? nk : kStages;
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         for (int i = 0; i < pre; ++i) {
-            mbar_arrive_expect_tx(&full[i], kStageBytes);
-            tc::tma_load_2d(smem + i * kStageBytes + kABytes, &tb, bk_tile(a, kt0 + i) * kBK, n0, &full[i]);
+            if (elect_one()) {
+                mbar_arrive_expect_tx(&full[i], kStageBytes);
+                tc::tma_load_2d(smem + i * kStageBytes + kABytes, &tb, bk_tile(a, kt0 + i) * kBK, n0, &full[i]);
+            }
+            __syncwarp();
         }
     } else if (warp >= 2) {
         const int t = threadIdx.x - 64;
@@ -566,53 +566,56 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
 
     bool ok = true;
     if (warp == 0) {
-        if (lane == 0) {
-            int issued = 0;
-            for (int i = 0; i < nk; ++i) {
-                const int s = i % kStages;
-                if (i >= kStages && !mbar_wait(&empty[s], ((i / kStages) - 1) & 1)) {
-                    s_err = 1;
-                    set_status(a.status, VT_DEV_WAIT_TIMEOUT);
-                    break;
-                }
-                if (*(volatile int*)&s_err) break;
-                uint8_t* st = smem + s * kStageBytes;
-                if (i < pre) {  // B of this stage is already on its way
-                    tc::tma_load_2d(st, &ta, (kt0 + i) * kBK, m0, &full[s]);
-                } else {
+        int issued = 0;
+        for (int i = 0; i < nk; ++i) {
+            const int s = i % kStages;
+            ok = __all_sync(0xffffffffu, (i < kStages || mbar_wait(&empty[s], ((i / kStages) - 1) & 1)) && !*(volatile int*)&s_err);
+            if (!ok) break;
+            uint8_t* st = smem + s * kStageBytes;
+            if (elect_one()) {
+                if (i >= pre) {  // (before that, B of the stage is already on its way)
                     mbar_arrive_expect_tx(&full[s], kStageBytes);
-                    tc::tma_load_2d(st, &ta, (kt0 + i) * kBK, m0, &full[s]);
                     tc::tma_load_2d(st + kABytes, &tb, bk_tile(a, kt0 + i) * kBK, n0, &full[s]);
                 }
-                issued = i + 1;
+                tc::tma_load_2d(st, &ta, (kt0 + i) * kBK, m0, &full[s]);
             }
-            // no copy may still be in flight when the stage memory is reused or the CTA ends (after an
-            // early stop this includes the B halves issued before griddepcontrol.wait: their stages
-            // never complete, and the bounded wait outlasts the copies)
-            if (issued < pre) issued = pre;
-            for (int i = issued > kStages ? issued - kStages : 0; i < issued; ++i)
-                if (!mbar_wait(&full[i % kStages], (i / kStages) & 1)) set_status(a.status, VT_DEV_WAIT_TIMEOUT);
+            __syncwarp();
+            issued = i + 1;
         }
+        if (!ok && lane == 0) {
+            s_err = 1;
+            set_status(a.status, VT_DEV_WAIT_TIMEOUT);
+        }
+        // no copy may still be in flight when the stage memory is reused or the CTA ends (after an
+        // early stop this includes the B halves issued before griddepcontrol.wait: their stages
+        // never complete, and the bounded wait outlasts the copies)
+        if (issued < pre) issued = pre;
+        for (int i = issued > kStages ? issued - kStages : 0; i < issued; ++i)
+            if (!mbar_wait_warp(&full[i % kStages], (i / kStages) & 1) && lane == 0) set_status(a.status, VT_DEV_WAIT_TIMEOUT);
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_f16(kBM, kBN);
-            for (int i = 0; i < nk; ++i) {
-                const int s = i % kStages;
-                if (!mbar_wait(&full[s], (i / kStages) & 1)) {
-                    s_err = 1;
-                    set_status(a.status, VT_DEV_WAIT_TIMEOUT);
-                    break;
-                }
-                tc::fence_after();
-                const uint32_t sa = smem_u32(smem + s * kStageBytes), sb = sa + kABytes;
+        constexpr uint32_t idesc = tc::idesc_f16(kBM, kBN);
+        for (int i = 0; i < nk; ++i) {
+            const int s = i % kStages;
+            ok = mbar_wait_warp(&full[s], (i / kStages) & 1);
+            if (!ok) break;
+            tc::fence_after();
+            const uint32_t sa = smem_u32(smem) + s * kStageBytes;
+            const uint32_t da = tc::desc_sw128_lo(sa), db = tc::desc_sw128_lo(sa + kABytes);
+            if (elect_one()) {
 #pragma unroll
                 for (int k = 0; k < kBK / 16; ++k)
-                    tc::mma_f16(tmem, tc::desc_sw128(sa + k * 32), tc::desc_sw128(sb + k * 32), idesc,
+                    tc::mma_f16(tmem, tc::desc_of(tc::kDescSw128Hi, da + k * 2), tc::desc_of(tc::kDescSw128Hi, db + k * 2), idesc,
                                 (i | k) != 0);
                 tc::mma_commit(&empty[s]);
             }
-            tc::mma_commit(done);
+            __syncwarp();
         }
+        if (!ok && lane == 0) {
+            s_err = 1;
+            set_status(a.status, VT_DEV_WAIT_TIMEOUT);
+        }
+        if (elect_one()) tc::mma_commit(done);
+        __syncwarp();
     } else {
         // one lane per warp polls the barrier (128 pollers would compete with the TMA and MMA
         // threads for issue slots and shared-memory bandwidth during the whole main loop)
@@ -904,105 +907,116 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
     const uint32_t tempty0 = CG == 2 ? dsmem_addr(tempty, 0) : smem_u32(tempty);
 
     if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            pdl_wait();  // A was written by the preceding kernel
-            uint32_t k = 0;  // stages filled so far
-            for (int t = cid; t < G.total_tiles && !*(volatile int*)&s_err; t += nctas) {
-                int g, m0, n0;
-                ptile(G, t, g, m0, n0);
-                const GemmArgs& a = G.a[g];
-                for (int kt = 0; kt < a.k_tiles; kt += T, ++k) {
-                    const int s = (int)(k % (uint32_t)S);
-                    if (k >= (uint32_t)S && !mbar_wait(&empty[s], ((k / S) - 1) & 1)) {
-                        abort_cta();
-                        break;
-                    }
-                    if (*(volatile int*)&s_err) break;
-                    uint8_t* st = smem + (size_t)s * stage_bytes;
-                    // a 3-D box past the last k-tile is filled with zeros and still counts its bytes
-                    const uint32_t fb = full0 + (uint32_t)s * 8;
-                    const int ya = m0 + rank * kBM, yb = n0 + rank * BNc, kb = bk_tile(a, kt);
+        // ------------------------------------------------------------ TMA producer (the whole warp)
+        pdl_wait();  // A was written by the preceding kernel
+        uint32_t slot = 0, phase = 0, filled = 0;  // ring position; stages filled so far
+        bool ok = true;
+        for (int t = cid; t < G.total_tiles && ok; t += nctas) {
+            int g, m0, n0;
+            ptile(G, t, g, m0, n0);
+            const int ya = m0 + rank * kBM, yb = n0 + rank * BNc, k_tiles = G.a[g].k_tiles, wrap = G.a[g].kb_wrap;
+            const CUtensorMap *ta = &G.ta[g], *tb = &G.tb[g];
+            for (int kt = 0; kt < k_tiles; kt += T) {
+                // (the first round of the ring passes at once: the phase before a barrier's first is complete)
+                ok = __all_sync(0xffffffffu, mbar_wait(&empty[slot], phase ^ 1u) && !*(volatile int*)&s_err);
+                if (!ok) break;
+                uint8_t* st = smem + (size_t)slot * stage_bytes;
+                // a 3-D box past the last k-tile is filled with zeros and still counts its bytes
+                const uint32_t fb = full0 + slot * 8;
+                const int kb = wrap > 0 && kt >= wrap ? kt - wrap : kt;  // B's k-tile
+                if (elect_one()) {
                     if constexpr (CG == 2) {
                         // rank 0 expects both CTAs' bytes; each CTA loads its own A rows and B half
-                        if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * stage_bytes);
+                        if (rank == 0) mbar_arrive_expect_tx(&full[slot], 2 * stage_bytes);
                         if (T == 2) {
-                            tc::tma_load_3d_pair(st, &G.ta[g], ya, kt, fb);
-                            tc::tma_load_3d_pair(st + a_bytes, &G.tb[g], yb, kb, fb);
+                            tc::tma_load_3d_pair(st, ta, ya, kt, fb);
+                            tc::tma_load_3d_pair(st + a_bytes, tb, yb, kb, fb);
                         } else {
-                            tc::tma_load_2d_pair(st, &G.ta[g], kt * kBK, ya, fb);
-                            tc::tma_load_2d_pair(st + a_bytes, &G.tb[g], kb * kBK, yb, fb);
+                            tc::tma_load_2d_pair(st, ta, kt * kBK, ya, fb);
+                            tc::tma_load_2d_pair(st + a_bytes, tb, kb * kBK, yb, fb);
                         }
                     } else {
-                        mbar_arrive_expect_tx(&full[s], stage_bytes);
+                        mbar_arrive_expect_tx(&full[slot], stage_bytes);
                         if (T == 2) {
-                            tc::tma_load_3d(st, &G.ta[g], ya, kt, fb);
-                            tc::tma_load_3d(st + a_bytes, &G.tb[g], yb, kb, fb);
+                            tc::tma_load_3d(st, ta, ya, kt, fb);
+                            tc::tma_load_3d(st + a_bytes, tb, yb, kb, fb);
                         } else {
-                            tc::tma_load_2d(st, &G.ta[g], kt * kBK, ya, &full[s]);
-                            tc::tma_load_2d(st + a_bytes, &G.tb[g], kb * kBK, yb, &full[s]);
+                            tc::tma_load_2d(st, ta, kt * kBK, ya, &full[slot]);
+                            tc::tma_load_2d(st + a_bytes, tb, kb * kBK, yb, &full[slot]);
                         }
                     }
                 }
+                __syncwarp();
+                ++filled;
+                if (++slot == (uint32_t)S) {
+                    slot = 0;
+                    phase ^= 1u;
+                }
             }
-            // no copy may be in flight when the CTA ends (rank 0's barriers count both CTAs' copies;
-            // the final cluster barrier keeps the peer until then)
-            if (rank == 0)
-                for (uint32_t i = k > (uint32_t)S ? k - S : 0; i < k; ++i)
-                    if (!mbar_wait(&full[i % S], (i / S) & 1)) set_status(status, VT_DEV_WAIT_TIMEOUT);
         }
+        if (!ok && lane == 0) abort_cta();
+        // no copy may be in flight when the CTA ends (rank 0's barriers count both CTAs' copies;
+        // the final cluster barrier keeps the peer until then)
+        if (rank == 0)
+            for (uint32_t i = filled > (uint32_t)S ? filled - S : 0; i < filled; ++i)
+                if (!mbar_wait_warp(&full[i % S], (i / S) & 1) && lane == 0) set_status(status, VT_DEV_WAIT_TIMEOUT);
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (rank 0)
-        if (lane == 0 && rank == 0) {
-            uint32_t k = 0;
+        // ------------------------------------------------------------ MMA issuer (rank 0, the whole warp)
+        if (rank == 0) {
+            uint32_t slot = 0, phase = 0;
             int it = 0;
-            for (int t = cid; t < G.total_tiles && !*(volatile int*)&s_err; t += nctas, ++it) {
+            bool ok = true;
+            const uint32_t idesc = tc::idesc_f16(kBM * CG, BN);
+            for (int t = cid; t < G.total_tiles && ok; t += nctas, ++it) {
                 int g, m0, n0;
                 ptile(G, t, g, m0, n0);
-                const GemmArgs& a = G.a[g];
-                const int buf = it & 1;
-                if (it >= 2 && !(CG == 2 ? mbar_wait_cluster(&tempty[buf], ((it >> 1) - 1) & 1)
-                                         : mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1))) {
-                    abort_cta();
-                    break;
-                }
+                const int k_tiles = G.a[g].k_tiles, buf = it & 1;
+                if (it >= 2)
+                    ok = __all_sync(0xffffffffu, CG == 2 ? mbar_wait_cluster(&tempty[buf], ((it >> 1) - 1) & 1)
+                                                         : mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1));
+                if (!ok) break;
                 tc::fence_after();
                 const uint32_t d_tmem = tmem + (uint32_t)(buf * 256);
-                const uint32_t idesc = tc::idesc_f16(kBM * CG, BN);
-                bool ok = true;
-                for (int kt = 0; kt < a.k_tiles; kt += T, ++k) {
-                    const int s = (int)(k % (uint32_t)S);
-                    if (!mbar_wait(&full[s], (k / S) & 1)) {
-                        ok = false;
-                        break;
-                    }
+                for (int kt = 0; kt < k_tiles; kt += T) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&full[slot], phase) && !*(volatile int*)&s_err);
+                    if (!ok) break;
                     tc::fence_after();
-                    const uint32_t s0 = smem_u32(smem + (size_t)s * stage_bytes);
-                    for (int j = 0; j < T && kt + j < a.k_tiles; ++j) {
-                        const uint32_t sa = s0 + (uint32_t)j * kABytes, sb = s0 + a_bytes + (uint32_t)j * b_tile;
+                    const uint32_t s0 = smem_u32(smem) + slot * stage_bytes;
+                    const uint32_t da = tc::desc_sw128_lo(s0), db = tc::desc_sw128_lo(s0 + a_bytes);
+                    const int nt = min(T, k_tiles - kt);
+                    if (elect_one()) {
+                        for (int j = 0; j < nt; ++j) {
 #pragma unroll
-                        for (int kk = 0; kk < kBK / 16; ++kk) {
-                            if constexpr (CG == 2)
-                                tc::mma_f16_pair(d_tmem, tc::desc_sw128(sa + kk * 32), tc::desc_sw128(sb + kk * 32), idesc,
-                                                 (kt + j | kk) != 0);
-                            else
-                                tc::mma_f16(d_tmem, tc::desc_sw128(sa + kk * 32), tc::desc_sw128(sb + kk * 32), idesc,
-                                            (kt + j | kk) != 0);
+                            for (int kk = 0; kk < kBK / 16; ++kk) {
+                                const uint64_t ad = tc::desc_of(tc::kDescSw128Hi, da + (uint32_t)j * (kABytes >> 4) + kk * 2);
+                                const uint64_t bd = tc::desc_of(tc::kDescSw128Hi, db + (uint32_t)j * (b_tile >> 4) + kk * 2);
+                                if constexpr (CG == 2) tc::mma_f16_pair(d_tmem, ad, bd, idesc, (kt + j | kk) != 0);
+                                else tc::mma_f16(d_tmem, ad, bd, idesc, (kt + j | kk) != 0);
+                            }
                         }
+                        if constexpr (CG == 2) tc::mma_commit_pair_both(&empty[slot]);
+                        else tc::mma_commit(&empty[slot]);
                     }
-                    if constexpr (CG == 2) tc::mma_commit_pair_both(&empty[s]);
-                    else tc::mma_commit(&empty[s]);
+                    __syncwarp();
+                    if (++slot == (uint32_t)S) {
+                        slot = 0;
+                        phase ^= 1u;
+                    }
                 }
-                if (!ok) {
-                    abort_cta();
-                    break;
+                if (!ok) break;
+                if (elect_one()) {
+                    if constexpr (CG == 2) tc::mma_commit_pair_both(&tfull[buf]);
+                    else tc::mma_commit(&tfull[buf]);
                 }
-                if constexpr (CG == 2) tc::mma_commit_pair_both(&tfull[buf]);
-                else tc::mma_commit(&tfull[buf]);
+                __syncwarp();
             }
-            if constexpr (CG == 2) tc::mma_commit_pair(done);
-            else tc::mma_commit(done);
-            if (!mbar_wait(done, 0)) set_status(status, VT_DEV_WAIT_TIMEOUT);
+            if (!ok && lane == 0) abort_cta();
+            if (elect_one()) {
+                if constexpr (CG == 2) tc::mma_commit_pair(done);
+                else tc::mma_commit(done);
+            }
+            __syncwarp();
+            if (!mbar_wait_warp(done, 0) && lane == 0) set_status(status, VT_DEV_WAIT_TIMEOUT);
         }
     } else {
         // ------------------------------------------------------------ epilogue (warps 2-5)
@@ -1233,9 +1247,12 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
 
     pdl_wait();  // q and the cache rows were written by the preceding kernel
     // Q does not depend on the KV length: its load goes out first
-    if (warp == 0 && lane == 0 && r0 < a.n) {
-        mbar_arrive_expect_tx(q_full, kQBytes);
-        for (int c = 0; c < DH / 64; ++c) tc::tma_load_2d(Qs + c * kAtom, &G.tq[gi], h * DH + 64 * c, r0, q_full);
+    if (warp == 0 && r0 < a.n) {
+        if (elect_one()) {
+            mbar_arrive_expect_tx(q_full, kQBytes);
+            for (int c = 0; c < DH / 64; ++c) tc::tma_load_2d(Qs + c * kAtom, &G.tq[gi], h * DH + 64 * c, r0, q_full);
+        }
+        __syncwarp();
     }
     const int P0 = *a.len + a.row_offset;
     const int rlast = min(r0 + kFaRows - 1, a.n - 1);
@@ -1244,90 +1261,110 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
     const int nb = kend > kbeg ? (kend - kbeg + kFaKeys - 1) / kFaKeys : 0;
 
     if (warp == 0) {
-        if (lane == 0 && nb == 0) mbar_wait(q_full, 0);  // no copy may be in flight when the CTA ends
-        if (lane == 0 && nb > 0) {
-            // one thread serves both rings, each load as soon as its slot is free (a blocked wait on
+        if (nb == 0) mbar_wait_warp(q_full, 0);  // no copy may be in flight when the CTA ends
+        if (nb > 0) {
+            // the warp serves both rings, each load as soon as its slot is free (a blocked wait on
             // one ring would hold up the other); V_j goes out after K_{j+1}, so that the copies the
             // first MMAs need (Q, K_0, K_1) are ahead of V in the copy engine
             const int krow0 = kvh * a.cap + kbeg;
             auto load = [&](bool is_v, int j) {
                 const int s = j & 1;
                 uint64_t* full = is_v ? &v_full[s] : &k_full[s];
-                mbar_arrive_expect_tx(full, kKVBytes);
-                for (int c = 0; c < DH / 64; ++c)
-                    tc::tma_load_2d((is_v ? Vs : Ks) + s * kKVBytes + c * kAtom, is_v ? &G.tv[gi] : &G.tk[gi], 64 * c,
-                                    krow0 + j * kFaKeys, full);
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, kKVBytes);
+                    for (int c = 0; c < DH / 64; ++c)
+                        tc::tma_load_2d((is_v ? Vs : Ks) + s * kKVBytes + c * kAtom, is_v ? &G.tv[gi] : &G.tk[gi], 64 * c,
+                                        krow0 + j * kFaKeys, full);
+                }
+                __syncwarp();
+            };
+            auto free_slot = [&](uint64_t* empty, int j) {
+                return j < 2 || __all_sync(0xffffffffu, fa_test(&empty[j & 1], ((j - 2) >> 1) & 1));
             };
             int jk = 0, jv = 0;
             uint32_t idle = 0;
             bool ok = true;
             while (jk < nb || jv < nb) {
                 bool moved = false;
-                if (jk < nb && (jk < 2 || fa_test(&k_empty[jk & 1], ((jk - 2) >> 1) & 1))) {
+                if (jk < nb && free_slot(k_empty, jk)) {
                     load(false, jk++);
                     moved = true;
                 }
-                if (jv < nb && (jk > jv + 1 || jk == nb) && (jv < 2 || fa_test(&v_empty[jv & 1], ((jv - 2) >> 1) & 1))) {
+                if (jv < nb && (jk > jv + 1 || jk == nb) && free_slot(v_empty, jv)) {
                     load(true, jv++);
                     moved = true;
                 }
                 if (moved) {
                     idle = 0;
-                } else if (++idle > (kSpinLimit << 2) || *s_err) {
+                } else if (++idle > (kSpinLimit << 2) || __any_sync(0xffffffffu, *s_err)) {
                     ok = false;
                     break;
                 }
             }
             if (!ok) {
-                *s_err = 1;
-                set_status(a.status, VT_DEV_WAIT_TIMEOUT);
+                if (lane == 0) {
+                    *s_err = 1;
+                    set_status(a.status, VT_DEV_WAIT_TIMEOUT);
+                }
                 // no copy may still be in flight when the CTA ends
-                mbar_wait(q_full, 0);
-                for (int j = jk > 2 ? jk - 2 : 0; j < jk; ++j) mbar_wait(&k_full[j & 1], (j >> 1) & 1);
-                for (int j = jv > 2 ? jv - 2 : 0; j < jv; ++j) mbar_wait(&v_full[j & 1], (j >> 1) & 1);
+                mbar_wait_warp(q_full, 0);
+                for (int j = jk > 2 ? jk - 2 : 0; j < jk; ++j) mbar_wait_warp(&k_full[j & 1], (j >> 1) & 1);
+                for (int j = jv > 2 ? jv - 2 : 0; j < jv; ++j) mbar_wait_warp(&v_full[j & 1], (j >> 1) & 1);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && nb > 0) {
+        if (nb > 0) {
             constexpr uint32_t idesc_s = tc::idesc_f16(kFaRows, kFaKeys);
             constexpr uint32_t idesc_o = tc::idesc_f16_bmn(kFaRows, DH);
-            const uint32_t qa = smem_u32(Qs), ka = smem_u32(Ks), va = smem_u32(Vs), pa = smem_u32(Ps);
+            // descriptors (lower words) of the first tiles; slots and K steps add to them
+            const uint32_t qd = tc::desc_sw128_lo(smem_u32(Qs)), kd = tc::desc_sw128_lo(smem_u32(Ks)),
+                           pd = tc::desc_sw128_lo(smem_u32(Ps));
+            const uint64_t vd = tc::desc_sw128_mn(smem_u32(Vs), kAtom);
+            const uint32_t vd_hi = (uint32_t)(vd >> 32), vd_lo = (uint32_t)vd;
+            auto all = [](bool x) { return __all_sync(0xffffffffu, x) != 0; };
             auto qk = [&](int j) -> bool {
                 const int s = j & 1;
-                if (!mbar_wait(&k_full[s], (j >> 1) & 1)) return false;
-                if (j >= 2 && !mbar_wait(&s_free[s], ((j - 2) >> 1) & 1)) return false;
-                if (*s_err) return false;
+                if (!mbar_wait_warp(&k_full[s], (j >> 1) & 1)) return false;
+                if (j >= 2 && !mbar_wait_warp(&s_free[s], ((j - 2) >> 1) & 1)) return false;
+                if (!all(*s_err == 0)) return false;
                 tc::fence_after();
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < DH / 16; ++kk) {
-                    const uint32_t off = (uint32_t)(kk >> 2) * kAtom + (uint32_t)(kk & 3) * 32;
-                    tc::mma_f16(tmem + (uint32_t)(s * kFaKeys), tc::desc_sw128(qa + off),
-                                tc::desc_sw128(ka + s * kKVBytes + off), idesc_s, kk > 0);
+                    for (int kk = 0; kk < DH / 16; ++kk) {
+                        const uint32_t off = (uint32_t)(kk >> 2) * (kAtom >> 4) + (uint32_t)(kk & 3) * 2;
+                        tc::mma_f16(tmem + (uint32_t)(s * kFaKeys), tc::desc_of(tc::kDescSw128Hi, qd + off),
+                                    tc::desc_of(tc::kDescSw128Hi, kd + (uint32_t)s * (kKVBytes >> 4) + off), idesc_s, kk > 0);
+                    }
+                    tc::mma_commit(&k_empty[s]);
+                    tc::mma_commit(&s_full[s]);
                 }
-                tc::mma_commit(&k_empty[s]);
-                tc::mma_commit(&s_full[s]);
+                __syncwarp();
                 return true;
             };
             auto qk_ready = [&](int j) -> bool {
-                return fa_test(&k_full[j & 1], (j >> 1) & 1) && (j < 2 || fa_test(&s_free[j & 1], ((j - 2) >> 1) & 1));
+                return all(fa_test(&k_full[j & 1], (j >> 1) & 1) && (j < 2 || fa_test(&s_free[j & 1], ((j - 2) >> 1) & 1)));
             };
             auto pv = [&](int j) -> bool {
                 const int s = j & 1;
-                if (!mbar_wait(&v_full[s], (j >> 1) & 1)) return false;
-                if (!mbar_wait(&p_full[s], (j >> 1) & 1)) return false;
-                if (*s_err) return false;
+                if (!mbar_wait_warp(&v_full[s], (j >> 1) & 1)) return false;
+                if (!mbar_wait_warp(&p_full[s], (j >> 1) & 1)) return false;
+                if (!all(*s_err == 0)) return false;
                 tc::fence_after();
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kFaKeys / 16; ++kk)
-                    tc::mma_f16(tmem + kOCol,
-                                tc::desc_sw128(pa + s * kPBytes + (uint32_t)(kk >> 2) * kAtom + (uint32_t)(kk & 3) * 32),
-                                tc::desc_sw128_mn(va + s * kKVBytes + (uint32_t)kk * 2048, kAtom), idesc_o,
-                                (j > 0 || kk > 0) ? 1u : 0u);
-                tc::mma_commit(&v_empty[s]);
-                tc::mma_commit(&o_full[s]);
+                    for (int kk = 0; kk < kFaKeys / 16; ++kk)
+                        tc::mma_f16(tmem + kOCol,
+                                    tc::desc_of(tc::kDescSw128Hi, pd + (uint32_t)s * (kPBytes >> 4) +
+                                                                      (uint32_t)(kk >> 2) * (kAtom >> 4) + (uint32_t)(kk & 3) * 2),
+                                    tc::desc_of(vd_hi, vd_lo + (uint32_t)s * (kKVBytes >> 4) + (uint32_t)kk * (2048 >> 4)), idesc_o,
+                                    (j > 0 || kk > 0) ? 1u : 0u);
+                    tc::mma_commit(&v_empty[s]);
+                    tc::mma_commit(&o_full[s]);
+                }
+                __syncwarp();
                 return true;
             };
-            bool ok = mbar_wait(q_full, 0);
+            bool ok = mbar_wait_warp(q_full, 0);
             ok = ok && qk(0);
             if (ok && nb > 1) ok = qk(1);
             for (int j = 0; ok && j < nb; ++j) {
@@ -1339,13 +1376,14 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
                 ok = ok && pv(j);
                 if (ok && j + 2 < nb && !issued) ok = qk(j + 2);
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 *s_err = 1;
                 set_status(a.status, VT_DEV_WAIT_TIMEOUT);
             }
             // tensor memory is freed only after every MMA issued has completed
-            tc::mma_commit(done);
-            if (!mbar_wait(done, 0)) set_status(a.status, VT_DEV_WAIT_TIMEOUT);
+            if (elect_one()) tc::mma_commit(done);
+            __syncwarp();
+            if (!mbar_wait_warp(done, 0) && lane == 0) set_status(a.status, VT_DEV_WAIT_TIMEOUT);
         }
     } else {
         const int g = (warp - 2) >> 2, quad = warp & 3, row = quad * 32 + lane;
