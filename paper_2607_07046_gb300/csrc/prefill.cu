@@ -13,10 +13,8 @@
 //   k_combine_norm   residual + shard partials in shard order, then the next block's RMSNorm
 //   k_gemm_p         C = A . B^T, A [M][K] and B [N][K] fp16 (K contiguous), persistent over the
 //                    output tiles of every shard's GEMM of a block: CTA pairs (tcgen05 cta_group::2,
-//                    256 x BN tiles) or single CTAs (128 x 256); epilogues: fp32 store, RoPE + q
+//                    256 x BN tiles) or single CTAs (128 x BN); epilogues: fp32 store, RoPE + q
 //                    store + KV append, SwiGLU
-//   k_gemm           the same MMA and copies, one 128 x 256 tile per CTA with an optional
-//                    cluster split-K, for groups too small to fill the GPU
 //   k_prefill_attn_tc causal flash attention on tcgen05 (S and O in tensor memory, K / V by TMA),
 //                    128 query rows of one head per CTA, one launch over every shard's heads
 #include <cuda.h>
@@ -26,14 +24,38 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <climits>
 #include <cstdlib>
 #include <string>
+#include <utility>
 
 #include "device.cuh"
 #include "internal.h"
 
 namespace vt {
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pk(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st,
+                             Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    int na = 0;
+    if (cluster > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = (unsigned)cluster;
+        attr[na].val.clusterDim.y = 1;
+        attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = (unsigned)na;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
 
 // ================================================================== tcgen05 / TMA primitives
 
@@ -49,21 +71,31 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
-// 3-D tiled TMA load: box (0, y, z) of a map whose third dimension steps one 64-column k-tile, so
-// one box brings several consecutive k-tiles of the same rows (one swizzled tile after the other).
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
+// 3-D tiled TMA load of box (x, y, z): a map whose third dimension steps one 64-column k-tile (x = 0)
+// or from the hi to the lo half of a split input, so that one box brings two tiles of the same rows
+// (one swizzled tile after the other).
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
             smem_u32(dst)),
-        "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar)
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, int y, int z, uint32_t bar) {
+__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
         "%4}], [%5];" ::"r"(smem_u32(dst)),
-        "l"(map), "r"(0), "r"(y), "r"(z), "r"(bar)
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
+}
+
+// Requests the box into L2.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z)
+                 : "memory");
 }
 
 // The same load issued by either CTA of a pair that shares one MMA (cta_group::2): the box lands in
@@ -82,12 +114,6 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, const void* src) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(map), "r"(x),
                  "r"(y), "r"(smem_u32(src))
-                 : "memory");
-}
-
-// 16-byte store into the shared memory of a CTA of the cluster (address from mapa).
-__device__ __forceinline__ void dsmem_st4(uint32_t addr, float a, float b, float c, float d) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
                  : "memory");
 }
 
@@ -390,25 +416,20 @@ cudaError_t launch_combine_norm(const CombineArgs& a, int rows, int d, const __h
     if (rows <= 0) return cudaSuccess;
     if (d % 8 != 0 || d > 16384) return cudaErrorInvalidValue;
     const int mc = row_mc(rows, d), t = row_threads(mc, d);
-    if (mc == 1) k_combine_norm<1><<<rows, t, 0, st>>>(a, d, gain, eps, xhat, split);
-    else k_combine_norm<2><<<rows, t, 0, st>>>(a, d, gain, eps, xhat, split);
-    return cudaGetLastError();
+    return mc == 1 ? launch_pk(k_combine_norm<1>, dim3(rows), t, 0, 1, st, a, d, gain, eps, xhat, split)
+                   : launch_pk(k_combine_norm<2>, dim3(rows), t, 0, 1, st, a, d, gain, eps, xhat, split);
 }
 
 // ================================================================== tensor-core GEMM
 
-constexpr int kBM = 128, kBK = 64, kBN = 256, kStages = 4;
-constexpr int kGemmThreads = 192;  // warp 0: TMA, warp 1: MMA + tensor memory, warps 2-5: epilogue
-constexpr int kABytes = kBM * kBK * 2, kBBytes = kBN * kBK * 2, kStageBytes = kABytes + kBBytes;
-constexpr size_t kGemmSmem = (size_t)kStages * kStageBytes + 1024 /* alignment */ + 256 /* barriers */;
+constexpr int kBM = 128, kBK = 64;  // rows of A per CTA, columns of a k-tile
 
 enum GemmEpi : int { kGemmF32 = 0, kGemmQkv = 1, kGemmSwiglu = 2 };
 
+constexpr int kGemmGroups = 8;  // GEMMs (shards of a block) in one launch
+
 struct GemmArgs {
-    int m, n, k_tiles;
-    int kb_wrap;  // > 0: A's k-tile kt multiplies B's k-tile kt mod kb_wrap (B read twice: hi / lo A halves)
-    const __half* b;  // B [n][ldb] (prefetched into L2 by the epilogue warps while they wait)
-    int64_t ldb;
+    int m, n, k_tiles;  // k_tiles: k-tiles of B (a split input has twice as many of A)
     // kGemmF32: c[row][col], row stride ldc
     float* c;
     int ldc;
@@ -426,315 +447,52 @@ struct GemmArgs {
     uint32_t* status;
 };
 
-// Up to kGemmGroups independent GEMMs of the same row count in one launch (the shards of one
-// block, which share M and often A): group g owns the CTAs with blockIdx.x in
-// [tile_end[g - 1], tile_end[g]), one per 256-column tile of its N.
-constexpr int kGemmGroups = 8;
-struct GemmGroup {
-    int n_groups;
-    int tile_end[kGemmGroups];
-    CUtensorMap ta[kGemmGroups], tb[kGemmGroups];
-    GemmArgs a[kGemmGroups];
-};
-static_assert(sizeof(GemmGroup) <= 4096, "the GEMM launch's parameters must fit in 4 KB");
-
-// 16-byte slot of the split-K receive buffer that holds floats [4e, 4e + 4) of 32-column chunk
-// `chunk` of local row `lr`.  128-bit shared accesses are served 8 threads at a time; the slot
-// permutation keeps those 8 threads on distinct banks both for the writer (8 consecutive rows, one
-// chunk) and for the reader (one row, 8 consecutive chunks).
-__device__ __forceinline__ int recv_slot(int chunk, int e, int lr) { return chunk * 8 + (e ^ ((chunk + lr) & 7)); }
-
-// B's k-tile for A's k-tile kt.
-__device__ __forceinline__ int bk_tile(const GemmArgs& a, int kt) {
-    return a.kb_wrap > 0 && kt >= a.kb_wrap ? kt - a.kb_wrap : kt;
-}
-
-// Epilogue of 4 consecutive columns [col, col + 4) of one output row (col a multiple of 4).
-template <int EPI>
-__device__ __forceinline__ void gemm_epilogue_quad(const GemmArgs& a, int row, int col, float4 v, int pos) {
-    if constexpr (EPI == kGemmF32) {
-        float* dst = a.c + (size_t)row * a.ldc + col;
-        if (col + 4 <= a.n) {
-            *reinterpret_cast<float4*>(dst) = v;
-        } else {
-            const float f[4] = {v.x, v.y, v.z, v.w};
-            for (int j = 0; j < 4 && col + j < a.n; ++j) dst[j] = f[j];
-        }
-    } else if constexpr (EPI == kGemmQkv) {
-        // columns (col, col + 1) and (col + 2, col + 3): RoPE pairs (i, i + dh/2) and (i + 1, ...)
-        const int dh = a.dh, half = dh / 2;
-        const int b = col / dh, i = (col % dh) / 2;
-        float l0 = v.x, h0 = v.y, l1 = v.z, h1 = v.w;
-        if (b < a.hq + a.hk) {
-            const float4 cs = *reinterpret_cast<const float4*>(a.rope + (size_t)pos * half + i);
-            l0 = v.x * cs.x - v.y * cs.y;
-            h0 = v.x * cs.y + v.y * cs.x;
-            l1 = v.z * cs.z - v.w * cs.w;
-            h1 = v.z * cs.w + v.w * cs.z;
-        }
-        __half* dst;
-        if (b < a.hq) dst = a.q + ((size_t)row * a.hq + b) * dh;
-        else if (b < a.hq + a.hk) dst = a.kcache + ((size_t)(b - a.hq) * a.cap + pos) * dh;
-        else dst = a.vcache + ((size_t)(b - a.hq - a.hk) * a.cap + pos) * dh;
-        *reinterpret_cast<__half2*>(dst + i) = __floats2half2_rn(l0, l1);
-        *reinterpret_cast<__half2*>(dst + i + half) = __floats2half2_rn(h0, h1);
-    } else {
-        // columns (gate, up) of intermediate columns col / 2 and col / 2 + 1
-        __half* dst = a.u + (size_t)row * a.ldu + a.ushift + col / 2;
-        if (col == 0)
-            for (int j = 0; j < a.ushift; ++j) dst[j - a.ushift] = __float2half_rn(0.f);
-        dst[0] = __float2half_rn(silu(v.x) * v.y);
-        if (col + 2 < a.n) dst[1] = __float2half_rn(silu(v.z) * v.w);
-    }
-}
-
-// One 128 x 256 tile of C = A . B^T per CTA, or per cluster of S CTAs that split K.
-// A k-tile is 64 columns of K: TMA brings the A and B boxes (128-byte swizzle) into one of kStages
-// stages; the MMA thread issues four 128 x 256 x 16 MMAs per stage into one tensor-memory
-// accumulator (256 columns) and releases the stage through tcgen05.commit.  The CTA's B boxes are
-// first requested into L2 with TMA prefetches (the weights do not depend on the preceding kernel,
-// so this starts before griddepcontrol.wait), which hides the HBM latency the 4-stage ring cannot.
-//
-// Split K (gridDim.z = S > 1, one thread-block cluster per output tile): every CTA accumulates
-// k-tiles [k_tiles z / S, k_tiles (z + 1) / S).  After the last MMA of every CTA (cluster barrier),
-// the accumulators are reduce-scattered through distributed shared memory: tile row r belongs to
-// CTA r / ceil(128 / S), which receives every CTA's fp32 values of its rows into its (now free)
-// stage memory, adds the S contributions in rank order (so results do not depend on timing) and
-// runs the epilogue.  Rows >= m and columns >= n come from TMA's zero fill and are not stored.
-// Every wait is bounded; on a timeout the kernel sets VT_DEV_WAIT_TIMEOUT, stops issuing, waits
-// for the copies it issued, still reaches both cluster barriers, frees tensor memory and ends.
-template <int EPI>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant__ GemmGroup G) {
-    int g = 0;
-    while (g + 1 < G.n_groups && (int)blockIdx.x >= G.tile_end[g]) ++g;
-    const CUtensorMap& ta = G.ta[g];
-    const CUtensorMap& tb = G.tb[g];
-    const GemmArgs& a = G.a[g];
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
-    uint64_t* empty = full + kStages;
-    uint64_t* done = empty + kStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
-    __shared__ int s_err;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n0 = ((int)blockIdx.x - (g > 0 ? G.tile_end[g - 1] : 0)) * kBN, m0 = blockIdx.y * kBM;
-    const int S = gridDim.z, z = blockIdx.z;
-    const int kt0 = (int)((int64_t)a.k_tiles * z / S), kt1 = (int)((int64_t)a.k_tiles * (z + 1) / S);
-    const int nk = kt1 - kt0;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        mbar_init(done, 1);
-        s_err = 0;
-        fence_mbar_init();
-    }
-    if (warp == 1) {
-        tc::tmem_alloc(tmem_slot, kBN);
-        tc::tmem_relinquish();
-    }
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    const uint32_t tmem = *tmem_slot;
-    // B (the weights) does not depend on the preceding kernel: the B halves of the first stages
-    // and the L2 prefetch of the CTA's remaining B tiles are issued before griddepcontrol.wait, so
-    // they stream while the preceding kernel finishes; A, which it wrote, is loaded after the wait.
-    const int pre = nk < kStages ? nk : kStages;
-    if (warp == 0) {
-        for (int i = 0; i < pre; ++i) {
-            if (elect_one()) {
-                mbar_arrive_expect_tx(&full[i], kStageBytes);
-                tc::tma_load_2d(smem + i * kStageBytes + kABytes, &tb, bk_tile(a, kt0 + i) * kBK, n0, &full[i]);
-            }
-            __syncwarp();
-        }
-    } else if (warp >= 2) {
-        const int t = threadIdx.x - 64;
-        for (int i = kt0 + pre; i < kt1; ++i) {
-            if (a.kb_wrap > 0 && i >= a.kb_wrap && kt0 < a.kb_wrap) break;  // the second pass reads the same B again
-            for (int r = t; r < kBN; r += kGemmThreads - 64)
-                if (n0 + r < a.n)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.b + (size_t)(n0 + r) * a.ldb + (size_t)bk_tile(a, i) * kBK));
-        }
-    }
-    pdl_wait();  // A was written by the preceding kernel
-
-    bool ok = true;
-    if (warp == 0) {
-        int issued = 0;
-        for (int i = 0; i < nk; ++i) {
-            const int s = i % kStages;
-            ok = __all_sync(0xffffffffu, (i < kStages || mbar_wait(&empty[s], ((i / kStages) - 1) & 1)) && !*(volatile int*)&s_err);
-            if (!ok) break;
-            uint8_t* st = smem + s * kStageBytes;
-            if (elect_one()) {
-                if (i >= pre) {  // (before that, B of the stage is already on its way)
-                    mbar_arrive_expect_tx(&full[s], kStageBytes);
-                    tc::tma_load_2d(st + kABytes, &tb, bk_tile(a, kt0 + i) * kBK, n0, &full[s]);
-                }
-                tc::tma_load_2d(st, &ta, (kt0 + i) * kBK, m0, &full[s]);
-            }
-            __syncwarp();
-            issued = i + 1;
-        }
-        if (!ok && lane == 0) {
-            s_err = 1;
-            set_status(a.status, VT_DEV_WAIT_TIMEOUT);
-        }
-        // no copy may still be in flight when the stage memory is reused or the CTA ends (after an
-        // early stop this includes the B halves issued before griddepcontrol.wait: their stages
-        // never complete, and the bounded wait outlasts the copies)
-        if (issued < pre) issued = pre;
-        for (int i = issued > kStages ? issued - kStages : 0; i < issued; ++i)
-            if (!mbar_wait_warp(&full[i % kStages], (i / kStages) & 1) && lane == 0) set_status(a.status, VT_DEV_WAIT_TIMEOUT);
-    } else if (warp == 1) {
-        constexpr uint32_t idesc = tc::idesc_f16(kBM, kBN);
-        for (int i = 0; i < nk; ++i) {
-            const int s = i % kStages;
-            ok = mbar_wait_warp(&full[s], (i / kStages) & 1);
-            if (!ok) break;
-            tc::fence_after();
-            const uint32_t sa = smem_u32(smem) + s * kStageBytes;
-            const uint32_t da = tc::desc_sw128_lo(sa), db = tc::desc_sw128_lo(sa + kABytes);
-            if (elect_one()) {
-#pragma unroll
-                for (int k = 0; k < kBK / 16; ++k)
-                    tc::mma_f16(tmem, tc::desc_of(tc::kDescSw128Hi, da + k * 2), tc::desc_of(tc::kDescSw128Hi, db + k * 2), idesc,
-                                (i | k) != 0);
-                tc::mma_commit(&empty[s]);
-            }
-            __syncwarp();
-        }
-        if (!ok && lane == 0) {
-            s_err = 1;
-            set_status(a.status, VT_DEV_WAIT_TIMEOUT);
-        }
-        if (elect_one()) tc::mma_commit(done);
-        __syncwarp();
-    } else {
-        // one lane per warp polls the barrier (128 pollers would compete with the TMA and MMA
-        // threads for issue slots and shared-memory bandwidth during the whole main loop)
-        if (lane == 0) {
-            ok = mbar_wait(done, 0);
-            if (!ok) set_status(a.status, VT_DEV_WAIT_TIMEOUT);
-            ok = ok && !*(volatile int*)&s_err;
-        }
-        __syncwarp();
-        // tcgen05.ld is warp-collective: the whole warp reads the accumulator or none of it
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        tc::fence_after();
-    }
-
-    // Epilogue.  recv[slot][local row][256] (fp32, 16-byte groups permuted by recv_slot) lives in
-    // the stage memory, free once the accumulator is complete (and, with split K, once every CTA
-    // of the cluster has passed the first cluster barrier).  Tile row r belongs to CTA
-    // r / rows_per of the cluster; every CTA sends each row of its accumulator to the owner's
-    // slot `z` (its own rank), the owner adds the S slots in rank order, and each warp then writes
-    // whole rows (lane = 4 consecutive columns) so every store instruction covers 512 bytes.
-    float* recv = reinterpret_cast<float*>(smem);
-    const int rows_per = (kBM + S - 1) / S;
-    if (S > 1) cluster_sync();  // every CTA's MMAs have completed; stage memory is free everywhere
-    if (warp >= 2 && ok) {
-        const int sub = warp & 3, tr = sub * 32 + lane;  // tile row held by this thread
-        const int owner = tr / rows_per, lr = tr - owner * rows_per;
-        float* row_dst = recv + (size_t)(z * rows_per + lr) * kBN;
-        const uint32_t dst = S > 1 ? dsmem_addr(row_dst, (uint32_t)owner) : smem_u32(row_dst);
-        for (int c = 0; c < kBN; c += 32) {
-            uint32_t r[32];
-            tc::tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)c, r);
-            tc::tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint32_t at = dst + (uint32_t)recv_slot(c / 32, e, lr) * 16;
-                if (S > 1)
-                    tc::dsmem_st4(at, __uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]),
-                                  __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3]));
-                else
-                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(__uint_as_float(r[4 * e])),
-                                 "f"(__uint_as_float(r[4 * e + 1])), "f"(__uint_as_float(r[4 * e + 2])),
-                                 "f"(__uint_as_float(r[4 * e + 3]))
-                                 : "memory");
-            }
-        }
-    }
-    if (S > 1) cluster_sync();  // every contribution has landed (all threads of every CTA)
-    else if (warp >= 2) asm volatile("bar.sync 1, %0;" ::"n"(kGemmThreads - 64) : "memory");  // the 4 epilogue warps
-    if (warp >= 2) {
-        const int r0 = z * rows_per, nr = min(kBM, r0 + rows_per) - r0;
-        int len0 = 0;
-        if constexpr (EPI == kGemmQkv) len0 = *a.len + a.row_offset;
-        for (int lr = warp - 2; lr < nr; lr += (kGemmThreads - 64) / 32) {
-            const int row = m0 + r0 + lr;
-            if (row >= a.m) break;
-            const int pos = len0 + row;
-            if constexpr (EPI == kGemmQkv) {
-                if (pos < 0 || pos >= a.cap) {
-                    if (lane == 0) set_status(a.status, VT_DEV_KV_OVERFLOW);
-                    continue;
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int f = h * 32 + lane;  // float4 index in the row
-                const int col = n0 + 4 * f;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int sl = 0; sl < S; ++sl) {
-                    const uint4 x = lds128(recv + (size_t)(sl * rows_per + lr) * kBN + recv_slot(f / 8, f % 8, lr) * 4);
-                    v.x += __uint_as_float(x.x);
-                    v.y += __uint_as_float(x.y);
-                    v.z += __uint_as_float(x.z);
-                    v.w += __uint_as_float(x.w);
-                }
-                if (col < a.n) gemm_epilogue_quad<EPI>(a, row, col, v, pos);
-            }
-        }
-    }
-    tc::fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc::fence_after();
-        tc::tmem_dealloc(tmem, kBN);
-    }
-}
-
-// ================================================================== persistent tensor-core GEMM
-//
 // The grouped projections of a block (every shard's GEMM of one kind) as one persistent launch.
 // Each worker walks output tiles t = w, w + workers, ... of the group in an order where the row
 // tile is the fastest index, so the tiles that share a weight tile run at the same time and the
 // weights leave DRAM once.  A worker is a pair of CTAs on two SMs (CG = 2: 256 x BN tiles, one
 // tcgen05.mma cta_group::2 over both CTAs' shared memory, each CTA holding 128 rows of A, half of
-// B and its 128 rows of the accumulator) or a single CTA (CG = 1: 128 x 256 tiles).
-//   warp 0   TMA producer: per stage, one box of A rows and one of B rows, each bringing two
-//            consecutive k-tiles (3-D tensor maps) or one, into a ring of stages as deep as shared
-//            memory allows, continuing across tiles.  The copy engine's cost is per box, so two
-//            k-tiles per box nearly halve it;
+// B and its 128 rows of the accumulator) or a single CTA (CG = 1: 128 x BN tiles).
+//   warp 0   TMA producer: per stage, one box of A rows and one of B rows into a ring of stages as
+//            deep as shared memory allows, continuing across tiles.  A stage holds one or two k-tiles,
+//            or, for a split input (hi and lo halves that meet the same weights), both halves' k-tile
+//            and one k-tile of B.  B's boxes are requested into L2 kPPrefetch k-tiles ahead, since a
+//            ring of 190 KB covers an L2 round trip but not the stream from DRAM;
 //   warp 1   tensor memory (512 columns: two accumulators of up to 256) and, in the CTA of rank 0,
-//            the MMA thread: the tile's k-tiles into accumulator (tile index & 1), a commit per
+//            the MMA warp: the tile's k-tiles into accumulator (tile index & 1), a commit per
 //            stage that frees it in both CTAs, and a commit that releases the accumulator to both
 //            CTAs' epilogues;
-//   warps 2-5 epilogue: each warp reads its 32 accumulator lanes (rows) in chunks of 32 columns
-//            and writes the tile's outputs (fp32 partials through a shared-memory turn so each
-//            store writes whole rows); after the last chunk it hands the accumulator back, so the
-//            epilogue of one tile overlaps the MMAs of the next.
+//   warps 2-9 epilogue: two warps for each 32 accumulator lanes (rows), on alternate chunks of 32
+//            columns, the next chunk's load in flight while one is written; the accumulator is
+//            handed back once its last load has completed, so the epilogue of one tile overlaps the
+//            MMAs of the next.
+// What bounds it (cycles per 64-column k-tile and pair, at 256 x 192 to 256 x 256): the MMAs 2 BN,
+// shared-memory fill (A 16 KB + B 12-16 KB a CTA at 66-75 bytes a cycle) 400-470, and about 15 us
+// a launch outside the main loop (fill, last epilogue, launch).  Four shards of the 7B shapes at
+// 512 rows, us per launch with (and before) the split input's shared B tile, eight epilogue warps
+// and the L2 requests ahead: QKV 71 (90), gate/up 70 (76), O 22.7 (25), down 42 (45.6); shapes of
+// the 13B layer at 1024 rows run at 1.65 to 1.7 PFLOP/s (QKV, gate/up).
 // Every wait is bounded; on a timeout the CTA sets VT_DEV_WAIT_TIMEOUT and an abort flag, every
 // role stops at its next wait, copies and MMAs in flight are waited for (bounded), and tensor
 // memory is freed.
 
 constexpr int kPStages = 8;     // most ring stages
+constexpr int kPPrefetch = 6;    // k-tiles by which B is requested into L2 ahead of its copy
 constexpr int kPTmemCols = 512;  // two accumulators
 constexpr size_t kPGemmSmem = 227 * 1024;
 constexpr size_t kPBarBytes = 256;                    // barriers and the tensor-memory slot
-constexpr size_t kPEpiBytes = 4 * 32 * 33 * 4;        // fp32 epilogue staging, one 32 x 33 block per warp
+constexpr int kPEpiWarps = 8;
+constexpr int kPThreads = 64 + kPEpiWarps * 32;       // warp 0: TMA, warp 1: MMA + tensor memory, then the epilogue
+constexpr size_t kPEpiBytes = kPEpiWarps * 32 * 20 * 4;  // fp32 epilogue staging, one 32 x 20 block per warp
 
 struct PGemmGroup {
     int n_groups, tiles_m, tm, bn, total_tiles, stages;
-    int kts;  // k-tiles per stage: 2 (one 3-D box per operand brings two) or 1
+    int am;  // rows of an A box: 128, or the launch's rows rounded up to 8 when there are fewer (the
+             // accumulator's other rows then hold products of stale shared memory, never stored)
+
+    // k-tiles per stage: 1, or 2 (one 3-D box per operand brings two).  ab = 1 (split inputs): a stage
+    // is one k-tile of B with the hi and the lo half of A's k-tile, so that B is copied once for both.
+    int kts, ab;
     int tile_end[kGemmGroups];  // cumulative tiles (tiles_m x column tiles of each group)
     CUtensorMap ta[kGemmGroups], tb[kGemmGroups];
     GemmArgs a[kGemmGroups];
@@ -751,35 +509,27 @@ __device__ __forceinline__ void ptile(const PGemmGroup& G, int t, int& g, int& m
     n0 = (u / G.tiles_m) * G.bn;
 }
 
-// Epilogue of 32 consecutive columns [col0, col0 + 32) of row `row` (col0 a multiple of 32).
+// QKV or SwiGLU epilogue of 32 consecutive columns [col0, col0 + 32) of row `row` (col0 a multiple of 32).
 template <int EPI>
 __device__ __forceinline__ void pepi_chunk(const GemmArgs& a, int row, int col0, const uint32_t (&r)[32], int pos) {
-    if constexpr (EPI == kGemmF32) {
-        float* dst = a.c + (size_t)row * a.ldc + col0;
-        if (col0 + 32 <= a.n) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                reinterpret_cast<float4*>(dst)[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                                                __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (col0 + j < a.n) dst[j] = __uint_as_float(r[j]);
-        }
-    } else if constexpr (EPI == kGemmQkv) {
+    if constexpr (EPI == kGemmQkv) {
         // 16 RoPE pairs (columns 2p, 2p + 1 = dims i0 + p and i0 + p + dh / 2 of one head block)
         if (col0 >= a.n) return;
         const int dh = a.dh, half = dh / 2;
         const int b = col0 / dh, i0 = (col0 % dh) / 2;
         float lo[16], hi[16];
         if (b < a.hq + a.hk) {
-            const float2* cs = a.rope + (size_t)pos * half + i0;
+            // 16 (cos, sin) pairs, two per 16-byte load (i0 is a multiple of 16)
+            const float4* cs = reinterpret_cast<const float4*>(a.rope + (size_t)pos * half + i0);
+            float4 c[8];
+#pragma unroll
+            for (int p = 0; p < 8; ++p) c[p] = cs[p];
 #pragma unroll
             for (int p = 0; p < 16; ++p) {
-                const float2 c = cs[p];
+                const float co = p & 1 ? c[p >> 1].z : c[p >> 1].x, si = p & 1 ? c[p >> 1].w : c[p >> 1].y;
                 const float x0 = __uint_as_float(r[2 * p]), x1 = __uint_as_float(r[2 * p + 1]);
-                lo[p] = x0 * c.x - x1 * c.y;
-                hi[p] = x0 * c.y + x1 * c.x;
+                lo[p] = x0 * co - x1 * si;
+                hi[p] = x0 * si + x1 * co;
             }
         } else {
 #pragma unroll
@@ -830,38 +580,47 @@ __device__ __forceinline__ void pepi_chunk(const GemmArgs& a, int row, int col0,
 }
 
 // fp32 epilogue of a warp's 32 rows [row0, row0 + 32) x 32 columns [col0, col0 + 32): lane l holds
-// row row0 + l.  The chunk is turned around in shared memory (`stg`, 32 x 33 floats, padded so
-// both the row-wise writes and the column-wise reads hit 32 distinct banks), then each store
-// instruction writes one row's 32 consecutive floats (one 128-byte line) instead of 32 scattered
-// 16-byte pieces.
+// row row0 + l.  Half a chunk at a time is turned around in shared memory (`stg`, 32 rows of 16
+// floats, 20 apart: conflict-free 16-byte stores), so that each store instruction writes 64
+// consecutive bytes of 8 rows instead of 16 bytes of 32.
 __device__ __forceinline__ void pepi_f32_rows(const GemmArgs& a, float* stg, int row0, int col0, const uint32_t (&r)[32]) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, rows = a.m - row0, q = 4 * (lane & 3);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) stg[lane * 33 + j] = __uint_as_float(r[j]);
-    __syncwarp();
-    const int col = col0 + lane;
-    const int rows = min(32, a.m - row0);
-    if (col < a.n)
-        for (int i = 0; i < rows; ++i) a.c[(size_t)(row0 + i) * a.ldc + col] = stg[i * 33 + lane];
-    __syncwarp();
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<uint4*>(stg + lane * 20 + 4 * j) =
+                make_uint4(r[16 * h + 4 * j], r[16 * h + 4 * j + 1], r[16 * h + 4 * j + 2], r[16 * h + 4 * j + 3]);
+        __syncwarp();
+        const int col = col0 + 16 * h + q;  // (n and ldc are multiples of 4)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int rr = 8 * i + (lane >> 2);
+            if (rr < rows && col < a.n)
+                *reinterpret_cast<uint4*>(a.c + (size_t)(row0 + rr) * a.ldc + col) =
+                    *reinterpret_cast<const uint4*>(stg + rr * 20 + q);
+        }
+        __syncwarp();
+    }
 }
 
 template <int EPI, int CG>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constant__ PGemmGroup G) {
+__global__ void __launch_bounds__(kPThreads, 1) k_gemm_p(const __grid_constant__ PGemmGroup G) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int S = G.stages, BN = G.bn, BNc = BN / CG;  // BNc: rows of each B tile this CTA holds
-    const int T = G.kts;
-    // stage: T A tiles (128 x 64) then T B tiles (BNc x 64), each a 128-byte-swizzled K-major tile
-    const uint32_t a_bytes = (uint32_t)(T * kABytes), b_tile = (uint32_t)BNc * kBK * 2;
-    const uint32_t stage_bytes = a_bytes + (uint32_t)T * b_tile;
+    const int T = G.kts, TB = G.ab ? 1 : T;
+    // stage: T A tiles (am x 64) then TB B tiles (BNc x 64), each a 128-byte-swizzled K-major tile (the
+    // MMA reads 128 rows from an A tile: with fewer, the rest comes from what follows it)
+    const uint32_t a_tile = (uint32_t)G.am * kBK * 2, a_bytes = (uint32_t)T * a_tile, b_tile = (uint32_t)BNc * kBK * 2;
+    const uint32_t stage_bytes = a_bytes + (uint32_t)TB * b_tile;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * stage_bytes);
     uint64_t* empty = full + kPStages;
     uint64_t* tfull = empty + kPStages;  // [2] accumulator b holds a finished tile
     uint64_t* tempty = tfull + 2;        // [2] accumulator b was read by the epilogue
     uint64_t* done = tempty + 2;         // every MMA issued by this CTA has completed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
-    float* epi_stage = reinterpret_cast<float*>(smem + (size_t)S * stage_bytes + kPBarBytes);  // [4][32][33]
+    float* epi_stage = reinterpret_cast<float*>(smem + (size_t)S * stage_bytes + kPBarBytes);  // [warps][32][20]
     __shared__ int s_err;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -877,7 +636,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], 4 * CG);
+            mbar_init(&tempty[b], kPEpiWarps * CG);
         }
         mbar_init(done, 1);
         s_err = 0;
@@ -910,40 +669,42 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
         // ------------------------------------------------------------ TMA producer (the whole warp)
         pdl_wait();  // A was written by the preceding kernel
         uint32_t slot = 0, phase = 0, filled = 0;  // ring position; stages filled so far
+        // boxes of fewer rows do not fill the ring's copy rate anyway (48-row boxes: 31.2 us without
+        // the requests, 33.1 with them; 64 rows: 32.4 and 29.3)
+        const bool ahead = BNc >= 64;
         bool ok = true;
         for (int t = cid; t < G.total_tiles && ok; t += nctas) {
             int g, m0, n0;
             ptile(G, t, g, m0, n0);
-            const int ya = m0 + rank * kBM, yb = n0 + rank * BNc, k_tiles = G.a[g].k_tiles, wrap = G.a[g].kb_wrap;
+            const int ya = m0 + rank * kBM, yb = n0 + rank * BNc, k_tiles = G.a[g].k_tiles;
             const CUtensorMap *ta = &G.ta[g], *tb = &G.tb[g];
-            for (int kt = 0; kt < k_tiles; kt += T) {
+            for (int kt = 0; kt < k_tiles; kt += TB) {
                 // (the first round of the ring passes at once: the phase before a barrier's first is complete)
                 ok = __all_sync(0xffffffffu, mbar_wait(&empty[slot], phase ^ 1u) && !*(volatile int*)&s_err);
                 if (!ok) break;
                 uint8_t* st = smem + (size_t)slot * stage_bytes;
                 // a 3-D box past the last k-tile is filled with zeros and still counts its bytes
                 const uint32_t fb = full0 + slot * 8;
-                const int kb = wrap > 0 && kt >= wrap ? kt - wrap : kt;  // B's k-tile
                 if (elect_one()) {
+                    // A: two k-tiles (third coordinate kt), or the hi and lo halves of one
+                    const int xa = G.ab ? kt * kBK : 0, za = G.ab ? 0 : kt;
+                    if (ahead && m0 == 0 && kt + kPPrefetch < k_tiles) {
+                        if (TB == 2) tc::tma_prefetch_3d(tb, 0, yb, kt + kPPrefetch);
+                        else tc::tma_prefetch_2d(tb, (kt + kPPrefetch) * kBK, yb);
+                    }
                     if constexpr (CG == 2) {
                         // rank 0 expects both CTAs' bytes; each CTA loads its own A rows and B half
                         if (rank == 0) mbar_arrive_expect_tx(&full[slot], 2 * stage_bytes);
-                        if (T == 2) {
-                            tc::tma_load_3d_pair(st, ta, ya, kt, fb);
-                            tc::tma_load_3d_pair(st + a_bytes, tb, yb, kb, fb);
-                        } else {
-                            tc::tma_load_2d_pair(st, ta, kt * kBK, ya, fb);
-                            tc::tma_load_2d_pair(st + a_bytes, tb, kb * kBK, yb, fb);
-                        }
+                        if (T == 2) tc::tma_load_3d_pair(st, ta, xa, ya, za, fb);
+                        else tc::tma_load_2d_pair(st, ta, kt * kBK, ya, fb);
+                        if (TB == 2) tc::tma_load_3d_pair(st + a_bytes, tb, 0, yb, kt, fb);
+                        else tc::tma_load_2d_pair(st + a_bytes, tb, kt * kBK, yb, fb);
                     } else {
                         mbar_arrive_expect_tx(&full[slot], stage_bytes);
-                        if (T == 2) {
-                            tc::tma_load_3d(st, ta, ya, kt, fb);
-                            tc::tma_load_3d(st + a_bytes, tb, yb, kb, fb);
-                        } else {
-                            tc::tma_load_2d(st, ta, kt * kBK, ya, &full[slot]);
-                            tc::tma_load_2d(st + a_bytes, tb, kb * kBK, yb, &full[slot]);
-                        }
+                        if (T == 2) tc::tma_load_3d(st, ta, xa, ya, za, fb);
+                        else tc::tma_load_2d(st, ta, kt * kBK, ya, &full[slot]);
+                        if (TB == 2) tc::tma_load_3d(st + a_bytes, tb, 0, yb, kt, fb);
+                        else tc::tma_load_2d(st + a_bytes, tb, kt * kBK, yb, &full[slot]);
                     }
                 }
                 __syncwarp();
@@ -960,6 +721,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
         if (rank == 0)
             for (uint32_t i = filled > (uint32_t)S ? filled - S : 0; i < filled; ++i)
                 if (!mbar_wait_warp(&full[i % S], (i / S) & 1) && lane == 0) set_status(status, VT_DEV_WAIT_TIMEOUT);
+        // nor may the CTA end while the commits that release its last stages are on their way: rank 0's
+        // arrive on both CTAs' barriers, and a late one would reach the next kernel's CTA on this SM
+        if (ok)
+            for (uint32_t i = filled > (uint32_t)S ? filled - S : 0; i < filled; ++i)
+                if (!mbar_wait_warp(&empty[i % S], (i / S) & 1) && lane == 0) set_status(status, VT_DEV_WAIT_TIMEOUT);
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (rank 0, the whole warp)
         if (rank == 0) {
@@ -967,6 +733,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
             int it = 0;
             bool ok = true;
             const uint32_t idesc = tc::idesc_f16(kBM * CG, BN);
+            const uint32_t b_step = G.ab ? 0u : b_tile >> 4;  // split inputs: both halves meet the same B tile
             for (int t = cid; t < G.total_tiles && ok; t += nctas, ++it) {
                 int g, m0, n0;
                 ptile(G, t, g, m0, n0);
@@ -977,23 +744,25 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
                 if (!ok) break;
                 tc::fence_after();
                 const uint32_t d_tmem = tmem + (uint32_t)(buf * 256);
-                for (int kt = 0; kt < k_tiles; kt += T) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&full[slot], phase) && !*(volatile int*)&s_err);
+                for (int kt = 0; kt < k_tiles; kt += TB) {
+                    ok = mbar_wait_warp(&full[slot], phase);
                     if (!ok) break;
                     tc::fence_after();
                     const uint32_t s0 = smem_u32(smem) + slot * stage_bytes;
                     const uint32_t da = tc::desc_sw128_lo(s0), db = tc::desc_sw128_lo(s0 + a_bytes);
-                    const int nt = min(T, k_tiles - kt);
-                    if (elect_one()) {
-                        for (int j = 0; j < nt; ++j) {
+                    const bool two = G.ab || (T == 2 && kt + 1 < k_tiles);  // A k-tiles in the stage
+                    // one k-tile: four MMAs of 16 columns; only a tile's first MMA may clear the accumulator
+                    auto ktile = [&](uint32_t ta_lo, uint32_t tb_lo, uint32_t first) {
 #pragma unroll
-                            for (int kk = 0; kk < kBK / 16; ++kk) {
-                                const uint64_t ad = tc::desc_of(tc::kDescSw128Hi, da + (uint32_t)j * (kABytes >> 4) + kk * 2);
-                                const uint64_t bd = tc::desc_of(tc::kDescSw128Hi, db + (uint32_t)j * (b_tile >> 4) + kk * 2);
-                                if constexpr (CG == 2) tc::mma_f16_pair(d_tmem, ad, bd, idesc, (kt + j | kk) != 0);
-                                else tc::mma_f16(d_tmem, ad, bd, idesc, (kt + j | kk) != 0);
-                            }
+                        for (int kk = 0; kk < kBK / 16; ++kk) {
+                            const uint64_t ad = tc::desc_of(tc::kDescSw128Hi, ta_lo + kk * 2), bd = tc::desc_of(tc::kDescSw128Hi, tb_lo + kk * 2);
+                            if constexpr (CG == 2) tc::mma_f16_pair(d_tmem, ad, bd, idesc, kk == 0 ? first : 1u);
+                            else tc::mma_f16(d_tmem, ad, bd, idesc, kk == 0 ? first : 1u);
                         }
+                    };
+                    if (elect_one()) {
+                        ktile(da, db, kt != 0);
+                        if (two) ktile(da + (a_tile >> 4), db + b_step, 1u);
                         if constexpr (CG == 2) tc::mma_commit_pair_both(&empty[slot]);
                         else tc::mma_commit(&empty[slot]);
                     }
@@ -1019,8 +788,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
             if (!mbar_wait_warp(done, 0) && lane == 0) set_status(status, VT_DEV_WAIT_TIMEOUT);
         }
     } else {
-        // ------------------------------------------------------------ epilogue (warps 2-5)
-        const int sub = warp & 3;  // accumulator lanes [32 sub, 32 sub + 32)
+        // ------------------------------------------------------------ epilogue (warps 2-9)
+        // accumulator lanes [32 sub, 32 sub + 32) (a warp reads the lanes of its number mod 4), 32-column
+        // chunks `half`, half + 2, ...: the next chunk's load is in flight while one is written
+        const int sub = warp & 3, half = (warp - 2) >> 2;
         int it = 0;
         for (int t = cid; t < G.total_tiles; t += nctas, ++it) {
             int g, m0, n0;
@@ -1046,21 +817,43 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
                 }
             }
             const uint32_t base = tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(buf * 256);
-            for (int c = 0; c < BN; c += 32) {
-                uint32_t r[32];
-                tc::tmem_ld32(base + (uint32_t)c, r);  // warp-collective: every lane takes part
-                tc::tmem_ld_wait();
-                if constexpr (EPI == kGemmF32) {
-                    if (n0 + c < a.n) pepi_f32_rows(a, epi_stage + sub * (32 * 33), row - lane, n0 + c, r);
-                } else {
-                    if (row_ok && n0 + c < a.n) pepi_chunk<EPI>(a, row, n0 + c, r, pos);
+            const int cend = min(BN, a.n - n0);  // columns of the tile that exist
+            auto release = [&]() {               // every load of this warp has completed
+                tc::fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if constexpr (CG == 2) mbar_arrive_cluster(tempty0 + (uint32_t)buf * 8);
+                    else mbar_arrive(&tempty[buf]);
                 }
+            };
+            auto write = [&](int c, const uint32_t (&r)[32]) {
+                if constexpr (EPI == kGemmF32) {
+                    pepi_f32_rows(a, epi_stage + (warp - 2) * (32 * 20), row - lane, n0 + c, r);
+                } else {
+                    if (row_ok) pepi_chunk<EPI>(a, row, n0 + c, r, pos);
+                    __syncwarp();
+                }
+            };
+            uint32_t r0[32], r1[32];
+            int c = 32 * half;
+            if (c >= cend) {
+                release();
+                continue;
             }
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                if constexpr (CG == 2) mbar_arrive_cluster(tempty0 + (uint32_t)buf * 8);
-                else mbar_arrive(&tempty[buf]);
+            tc::tmem_ld32(base + (uint32_t)c, r0);  // warp-collective: every lane takes part
+            while (true) {
+                tc::tmem_ld_wait_on(r0);
+                if (c + 64 < cend) tc::tmem_ld32(base + (uint32_t)c + 64, r1);
+                else release();
+                write(c, r0);
+                c += 64;
+                if (c >= cend) break;
+                tc::tmem_ld_wait_on(r1);
+                if (c + 64 < cend) tc::tmem_ld32(base + (uint32_t)c + 64, r0);
+                else release();
+                write(c, r1);
+                c += 64;
+                if (c >= cend) break;
             }
         }
     }
@@ -1075,22 +868,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_p(const __grid_constan
     }
 }
 
-// Tile width of the single-CTA persistent GEMM: 128 x 256.  Its ring moves 384 lines of 128 bytes
-// (A 128 + B 256) per k-tile through shared memory, which the copy engine delivers at about half a
-// line per cycle (measured: a stage of that size fills in 600-700 cycles), against 512 cycles of
-// MMA; narrower tiles do less MMA work per line, so the widest is the fastest (measured against
-// 128, 160 and 192 on the 7B prefill).
-constexpr int kPBn = 256;
-
-// bn_cta: rows of the B tile one CTA holds (the tile width, or half of it for a CTA pair);
-// kts: k-tiles per stage
-static size_t pgemm_stage_bytes(int bn_cta, int kts) { return (size_t)kts * ((size_t)kABytes + (size_t)bn_cta * kBK * 2); }
-static int pgemm_stages(int bn_cta, int kts) {
+// am: rows of an A box; bn_cta: rows of the B tile one CTA holds (the tile width, or half of it for
+// a CTA pair); kts: k-tiles of A per stage; ab: one k-tile of B for both halves of a split input
+static size_t pgemm_stage_bytes(int am, int bn_cta, int kts, int ab) {
+    return ((size_t)kts * am + (size_t)(ab ? 1 : kts) * bn_cta) * kBK * 2;
+}
+static int pgemm_stages(int am, int bn_cta, int kts, int ab) {
     // the launch may use kPGemmSmem - 1024 bytes, 1024 of them lost to aligning the ring
     const size_t room = kPGemmSmem - 2048 - kPBarBytes - kPEpiBytes;
-    int s = (int)(room / pgemm_stage_bytes(bn_cta, kts));
+    int s = (int)(room / pgemm_stage_bytes(am, bn_cta, kts, ab));
     return s > kPStages ? kPStages : s;
 }
+// An MMA reads 128 rows from each A tile: past a shorter last tile it reaches at most this far into
+// the barriers and the epilogue's staging.
+static_assert((kBM - 8) * kBK * 2 <= kPBarBytes + kPEpiBytes, "short A tiles must not lead past the CTA's shared memory");
 
 __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
     const __half2 h = __floats2half2_rn(lo, hi);
@@ -1563,10 +1354,7 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
 // ================================================================== host side
 
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-static bool g_gemm_persistent = true;  // VT_GEMM_PERSISTENT=0 keeps every GEMM on k_gemm
-static int g_pgemm_pairs = 0;          // co-resident CTA pairs of the persistent GEMM (0: single CTAs)
-constexpr int kMaxSplit = 4;
-static int g_split_clusters[kMaxSplit + 1];  // co-resident clusters of S GEMM CTAs (index S)
+static int g_pgemm_pairs = 0;  // co-resident CTA pairs of the persistent GEMM (0: single CTAs)
 
 cudaError_t init_prefill_kernels() {
     void* fn = nullptr;
@@ -1575,46 +1363,18 @@ cudaError_t init_prefill_kernels() {
     if (e != cudaSuccess) return e;
     if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
     g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    if ((e = cudaFuncSetAttribute(k_gemm<kGemmF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_gemm<kGemmQkv>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_gemm<kGemmSwiglu>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem)) != cudaSuccess)
-        return e;
-    // how many clusters of S GEMM CTAs fit at once (the split factor's wave size)
-    for (int sp = 2; sp <= kMaxSplit; ++sp) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1, 1, sp * 64);
-        cfg.blockDim = dim3(kGemmThreads);
-        cfg.dynamicSmemBytes = kGemmSmem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = sp;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, k_gemm<kGemmF32>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            nc = 0;
-        }
-        g_split_clusters[sp] = nc;
-    }
     for (auto f : {k_gemm_p<kGemmF32, 1>, k_gemm_p<kGemmQkv, 1>, k_gemm_p<kGemmSwiglu, 1>, k_gemm_p<kGemmF32, 2>,
                    k_gemm_p<kGemmQkv, 2>, k_gemm_p<kGemmSwiglu, 2>})
         if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPGemmSmem - 1024))) != cudaSuccess)
             return e;
     {
-        const char* v = getenv("VT_GEMM_PERSISTENT");
-        g_gemm_persistent = !(v && v[0] == '0');
         // VT_GEMM_PAIR=0 keeps the persistent GEMM on single CTAs
         const char* pv = getenv("VT_GEMM_PAIR");
         g_pgemm_pairs = 0;
         if (!(pv && pv[0] == '0')) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(2 * 64);
-            cfg.blockDim = dim3(kGemmThreads);
+            cfg.blockDim = dim3(kPThreads);
             cfg.dynamicSmemBytes = kPGemmSmem - 1024;
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1665,21 +1425,22 @@ static bool make_map(CUtensorMap* map, const void* base, int64_t inner, int64_t 
     return true;
 }
 
-// The same operand as a 3-D map {64, rows, inner / 64} whose third dimension steps one k-tile
-// (128 bytes), read in boxes of 64 x box_rows x 2: two consecutive k-tiles per copy.  inner must
-// be a multiple of 64 (the box does not stop at the row's end).
+// The same operand as a 3-D map whose box brings two tiles of the same rows: {64, rows, inner / 64},
+// the third dimension stepping one k-tile (128 bytes; inner a multiple of 64: the box does not stop
+// at the row's end), or, for a split input of `half` columns per half, {half, rows, 2}, the third
+// dimension stepping from the hi to the lo half.
 static bool make_map_k2(CUtensorMap* map, const void* base, int64_t inner, int64_t rows, int64_t ld, int box_rows,
-                        std::string* err) {
+                        int64_t half, std::string* err) {
     if (!g_encode) {
         *err = "the tensor-map encoder is not available";
         return false;
     }
-    if (((uintptr_t)base & 15) != 0 || (ld * 2) % 16 != 0 || inner % kBK != 0) {
+    if (((uintptr_t)base & 15) != 0 || (ld * 2) % 16 != 0 || (half > 0 ? half : inner) % kBK != 0) {
         *err = "a GEMM operand is not 16-byte aligned or its K is not a multiple of 64";
         return false;
     }
-    const cuuint64_t dims[3] = {(cuuint64_t)kBK, (cuuint64_t)rows, (cuuint64_t)(inner / kBK)};
-    const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)kBK * 2};
+    const cuuint64_t dims[3] = {(cuuint64_t)(half > 0 ? half : kBK), (cuuint64_t)rows, (cuuint64_t)(half > 0 ? 2 : inner / kBK)};
+    const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)(half > 0 ? half : kBK) * 2};
     const cuuint32_t box[3] = {(cuuint32_t)kBK, (cuuint32_t)box_rows, 2};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box,
@@ -1690,29 +1451,6 @@ static bool make_map_k2(CUtensorMap* map, const void* base, int64_t inner, int64
         return false;
     }
     return true;
-}
-
-// Split factor for `tiles` output tiles of `k_tiles` k-tiles, from a time model of one launch:
-// per wave, a fixed cost (first loads, epilogue) plus the k-tiles of one split; with S > 1, the
-// cluster reduction of the accumulators.  The constants are measured on GB300 (microseconds).
-// k_tiles: the longest GEMM of the launch (its time); min_k_tiles: the shortest, which must still
-// give every CTA of a split at least 4 k-tiles (a CTA without k-tiles has no accumulator).
-static int choose_split(int tiles, int k_tiles, int min_k_tiles) {
-    constexpr double kTile = 0.33, kFixed = 4.0, kReduce = 3.5;
-    int best = 1;
-    double best_t = 1e30;
-    for (int s = 1; s <= kMaxSplit; ++s) {
-        if (s > 1 && min_k_tiles / s < 4) break;
-        const int per_wave = s == 1 ? g_num_sms : g_split_clusters[s];
-        if (per_wave < 1) continue;
-        const int waves = (tiles + per_wave - 1) / per_wave;
-        const double t = waves * (kFixed + kTile * k_tiles / s) + (s > 1 ? kReduce : 0.0);
-        if (t < best_t - 1e-9) {
-            best = s;
-            best_t = t;
-        }
-    }
-    return best;
 }
 
 // One GEMM of a grouped launch: C_g = A_g . B_g^T with m rows (shared by the group), n_g columns
@@ -1728,22 +1466,51 @@ struct GemmSpec {
 };
 
 
-// Width of a CTA-pair tile (256 rows).  The copy engine's cost is per box rather than per byte
-// (measured on GB300: a ring stage of one A box and one B box turns over in about 1000 cycles
-// whether the boxes carry one k-tile or two), so a k-tile costs about 500 cycles of copying with
-// two k-tiles per box, 900 with one, against 2w cycles of MMA; the width is the one whose rounds
-// of tiles over the co-resident pairs cost least (ties to the wider).
-static int choose_pair_bn(const GemmSpec* specs, int ng, int tiles_m, int pairs, int kts) {
-    int best = 256;
-    long best_cost = -1;
-    for (int w = 256; w >= 128; w -= 32) {
-        int tiles = 0;
-        for (int g = 0; g < ng; ++g) tiles += tiles_m * ((specs[g].n + w - 1) / w);
-        const long rounds = (tiles + pairs - 1) / pairs;
-        const long cost = rounds * (long)std::max(2 * w, kts == 2 ? 500 : 900);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best = w;
+// How a grouped launch is cut: CTA pairs (256-row tiles) or single CTAs (128), the rows of an A box,
+// the tile width, the k-tiles per stage, and the time the model gives it (cycles).
+struct PGemmPlan {
+    int cg = 2, am = kBM, bn = 256, kts = 2, ab = 0;
+    double cost = 1e30;
+};
+// Model of one launch: rounds of tiles over the CTAs or pairs that run at once; in each, per k-tile
+// of A, the largest of the MMAs, one CTA's copies (L2 to shared memory) and the weights' stream from
+// DRAM, plus a fixed cost to fill the ring, and the last tile's epilogue.  The rates are measured
+// (at 1.92 GHz); the plan it picks was the fastest or within 4% of it of all pairs and widths on 19
+// shapes of 77 to 4096 rows.  Short prompts thus run as one round of narrow single-CTA tiles over
+// the whole GPU (77 rows of the 8B shapes, four shards: gate/up 61 -> 44 us, O 16.7 -> 10.4, down
+// 37 -> 27 against 128 x 256 tiles with split K), long ones as pairs of 192 to 256 columns.
+constexpr double kPCopyRate = 66;    // bytes per cycle and SM, L2 to shared memory
+constexpr double kPDramRate = 3400;  // bytes per cycle from DRAM, the whole GPU
+constexpr double kPDramSm = 20;      // bytes per cycle and SM of weights that no other row tile shares
+constexpr double kPFixed = 3000;     // cycles per round
+static PGemmPlan plan_pgemm(const GemmSpec* specs, int ng, int m) {
+    PGemmPlan best;
+    // two k-tiles per box need every K in whole k-tiles: a 3-D box past K would read the next row
+    // instead of zeros; a split input always has two halves of whole k-tiles
+    const int ab = specs[0].kb > 0;
+    bool whole = true;
+    double steps = 0;
+    for (int g = 0; g < ng; ++g) {
+        whole &= specs[g].k % kBK == 0;
+        steps = std::max(steps, (double)((specs[g].k + kBK - 1) / kBK));
+    }
+    const int am = std::min(kBM, (m + 7) / 8 * 8);
+    for (int cg = g_pgemm_pairs > 0 && m > kBM ? 2 : 1; cg >= 1; --cg) {
+        const int slots = cg == 2 ? g_pgemm_pairs : (g_num_sms > 0 ? g_num_sms : 148);
+        const int tiles_m = (m + kBM * cg - 1) / (kBM * cg);
+        for (int bn = 256; bn >= 32; bn -= 32) {
+            long tiles = 0;
+            for (int g = 0; g < ng; ++g) tiles += (long)tiles_m * ((specs[g].n + bn - 1) / bn);
+            const long rounds = (tiles + slots - 1) / slots;
+            // two k-tiles per stage halve the boxes (bn 224, 512 rows: 72.9 against 77.0 us)
+            const int kts = ab || (whole && pgemm_stages(am, bn / cg, 2, 0) >= 3) ? 2 : 1;
+            const double b_rows = (double)bn / cg / (ab ? 2 : 1);
+            const double mma = std::max(2.0 * bn, 440.0) + 30;
+            const double copy = (am + b_rows) * 128 / kPCopyRate + (kts == 2 ? 60 : 120);
+            const double dram = std::max((double)std::min<long>(tiles, slots) / tiles_m * bn / (ab ? 2 : 1) * 128 / kPDramRate,
+                                         tiles_m == 1 ? b_rows * 128 / kPDramSm : 0.0);
+            const double cost = rounds * (steps * std::max({mma, copy, dram}) + kPFixed) + 20.0 * bn;
+            if (cost < best.cost - 1e-9) best = PGemmPlan{cg, am, bn, kts, ab, cost};
         }
     }
     return best;
@@ -1752,57 +1519,42 @@ static int choose_pair_bn(const GemmSpec* specs, int ng, int tiles_m, int pairs,
 // The grouped GEMMs of `specs` (all with m rows) as one persistent launch: one CTA (CG = 1) or
 // one CTA pair (CG = 2, 256-row tiles) per SM or SM pair, or one per tile when there are fewer.
 template <int EPI, int CG>
-static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, cudaStream_t st, std::string* err) {
+static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, const PGemmPlan& plan, cudaStream_t st,
+                                     std::string* err) {
     PGemmGroup G{};
     G.n_groups = ng;
     G.tm = kBM * CG;
     G.tiles_m = (m + G.tm - 1) / G.tm;
+    G.bn = plan.bn;
+    G.kts = plan.kts;
+    G.ab = plan.ab;
+    G.am = plan.am;
+    G.stages = pgemm_stages(G.am, G.bn / CG, G.kts, G.ab);
     const int slots = CG == 2 ? g_pgemm_pairs : (g_num_sms > 0 ? g_num_sms : 148);
-    // two k-tiles per box needs every K (and the wrap of a split GEMM) in whole pairs of k-tiles'
-    // worth of columns: a 3-D box past K would read the next row instead of zeros
-    G.kts = 2;
-    for (int g = 0; g < ng; ++g)
-        if (specs[g].k % kBK != 0 || (specs[g].kb > 0 && specs[g].kb % (2 * kBK) != 0)) G.kts = 1;
-    G.bn = CG == 2 ? choose_pair_bn(specs, ng, G.tiles_m, slots, G.kts) : kPBn;
-    G.stages = pgemm_stages(G.bn / CG, G.kts);
     int acc = 0;
     for (int g = 0; g < ng; ++g) {
         const GemmSpec& sp = specs[g];
-        if (sp.kb > 0 && (sp.kb % kBK != 0 || sp.k != 2 * sp.kb)) {
+        if ((sp.kb > 0) != (G.ab != 0) || (sp.kb > 0 && (sp.kb % kBK != 0 || sp.k != 2 * sp.kb))) {
             *err = "a split GEMM needs k = 2 kb with kb a multiple of 64";
             return VT_ERR_INVALID_ARG;
         }
-        const bool ok = G.kts == 2
-                            ? make_map_k2(&G.ta[g], sp.A, sp.k, m, sp.lda, kBM, err) &&
-                                  make_map_k2(&G.tb[g], sp.B, sp.kb > 0 ? sp.kb : sp.k, sp.n, sp.ldb, G.bn / CG, err)
-                            : make_map(&G.ta[g], sp.A, sp.k, m, sp.lda, kBM, err) &&
-                                  make_map(&G.tb[g], sp.B, sp.kb > 0 ? sp.kb : sp.k, sp.n, sp.ldb, G.bn / CG, err);
+        const int kb = G.ab ? sp.kb : sp.k;  // B's columns
+        const bool ok = (G.kts == 2 ? make_map_k2(&G.ta[g], sp.A, sp.k, m, sp.lda, G.am, G.ab ? sp.kb : 0, err)
+                                    : make_map(&G.ta[g], sp.A, sp.k, m, sp.lda, G.am, err)) &&
+                        (G.kts == 2 && !G.ab ? make_map_k2(&G.tb[g], sp.B, kb, sp.n, sp.ldb, G.bn / CG, 0, err)
+                                             : make_map(&G.tb[g], sp.B, kb, sp.n, sp.ldb, G.bn / CG, err));
         if (!ok) return VT_ERR_INVALID_ARG;
         GemmArgs& a = G.a[g];
         a = sp.base;
         a.m = m;
         a.n = sp.n;
-        a.b = static_cast<const __half*>(sp.B);
-        a.ldb = sp.ldb;
-        a.k_tiles = (sp.k + kBK - 1) / kBK;
-        a.kb_wrap = sp.kb > 0 ? sp.kb / kBK : 0;
+        a.k_tiles = (kb + kBK - 1) / kBK;
         acc += G.tiles_m * ((sp.n + G.bn - 1) / G.bn);
         G.tile_end[g] = acc;
     }
     G.total_tiles = acc;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(CG * std::min(acc, slots)));
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = 1024 + (size_t)G.stages * pgemm_stage_bytes(G.bn / CG, G.kts) + kPBarBytes + kPEpiBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CG;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = CG == 2 ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_p<EPI, CG>, G);
+    const size_t smem = 1024 + (size_t)G.stages * pgemm_stage_bytes(G.am, G.bn / CG, G.kts, G.ab) + kPBarBytes + kPEpiBytes;
+    const cudaError_t e = launch_pk(k_gemm_p<EPI, CG>, dim3((unsigned)(CG * std::min(acc, slots))), kPThreads, smem, CG, st, G);
     if (e != cudaSuccess) {
         *err = std::string("persistent GEMM launch failed: ") + cudaGetErrorString(e);
         return VT_ERR_CUDA;
@@ -1810,77 +1562,17 @@ static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, cudaS
     return VT_OK;
 }
 
-// Launches the GEMMs of `specs` (all with m rows) kGemmGroups at a time.  A group with at least
-// as many 128 x 256 tiles as half the SMs runs as one persistent launch (k_gemm_p); a smaller one
-// (short prompts, a single shard) as one CTA, or split-K cluster, per output tile (k_gemm), so
-// that its few tiles still spread over the GPU.
+// Launches the GEMMs of `specs` (all with m rows) kGemmGroups at a time.
 template <int EPI>
 static vt_status run_gemm_group(const GemmSpec* specs, int n_specs, int m, cudaStream_t st, std::string* err) {
     for (int g0 = 0; g0 < n_specs; g0 += kGemmGroups) {
         const int ng = std::min(kGemmGroups, n_specs - g0);
-        {
-            int tiles = 0;
-            for (int g = 0; g < ng; ++g) tiles += ((m + kBM - 1) / kBM) * ((specs[g0 + g].n + kBN - 1) / kBN);
-            if (g_gemm_persistent && 2 * tiles >= (g_num_sms > 0 ? g_num_sms : 148)) {
-                const vt_status r = g_pgemm_pairs > 0 ? run_gemm_persistent<EPI, 2>(specs + g0, ng, m, st, err)
-                                                      : run_gemm_persistent<EPI, 1>(specs + g0, ng, m, st, err);
-                if (r != VT_OK) return r;
-                continue;
-            }
-        }
-        GemmGroup G{};
-        G.n_groups = ng;
-        int tiles_n = 0, max_k_tiles = 1, min_k_tiles = 1 << 30;
-        for (int g = 0; g < ng; ++g) {
-            const GemmSpec& sp = specs[g0 + g];
-            if (sp.kb > 0 && (sp.kb % kBK != 0 || sp.k != 2 * sp.kb)) {
-                *err = "a split GEMM needs k = 2 kb with kb a multiple of 64";
-                return VT_ERR_INVALID_ARG;
-            }
-            if (!make_map(&G.ta[g], sp.A, sp.k, m, sp.lda, kBM, err) ||
-                !make_map(&G.tb[g], sp.B, sp.kb > 0 ? sp.kb : sp.k, sp.n, sp.ldb, kBN, err))
-                return VT_ERR_INVALID_ARG;
-            GemmArgs& a = G.a[g];
-            a = sp.base;
-            a.m = m;
-            a.n = sp.n;
-            a.b = static_cast<const __half*>(sp.B);
-            a.ldb = sp.ldb;
-            a.k_tiles = (sp.k + kBK - 1) / kBK;
-            a.kb_wrap = sp.kb > 0 ? sp.kb / kBK : 0;
-            max_k_tiles = std::max(max_k_tiles, a.k_tiles);
-            min_k_tiles = std::min(min_k_tiles, a.k_tiles);
-            tiles_n += (sp.n + kBN - 1) / kBN;
-            G.tile_end[g] = tiles_n;
-        }
-        const int tiles_m = (m + kBM - 1) / kBM;
-        const int split = choose_split(tiles_n * tiles_m, max_k_tiles, min_k_tiles);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(tiles_n, tiles_m, split);
-        cfg.blockDim = dim3(kGemmThreads);
-        cfg.dynamicSmemBytes = kGemmSmem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = split;
-        cfg.attrs = attr;
-        cfg.numAttrs = split > 1 ? 1 : 0;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm<EPI>, G);
-        if (e != cudaSuccess) {
-            *err = std::string("GEMM launch failed: ") + cudaGetErrorString(e);
-            return VT_ERR_CUDA;
-        }
+        const PGemmPlan plan = plan_pgemm(specs + g0, ng, m);
+        const vt_status r = plan.cg == 2 ? run_gemm_persistent<EPI, 2>(specs + g0, ng, m, plan, st, err)
+                                         : run_gemm_persistent<EPI, 1>(specs + g0, ng, m, plan, st, err);
+        if (r != VT_OK) return r;
     }
     return VT_OK;
-}
-
-template <int EPI>
-static vt_status run_gemm(const void* A, int64_t lda, const void* B, int64_t ldb, int m, int n, int k,
-                          const GemmArgs& base, cudaStream_t st, std::string* err) {
-    const GemmSpec sp{A, lda, B, ldb, n, k, base};
-    return run_gemm_group<EPI>(&sp, 1, m, st, err);
 }
 
 cudaError_t launch_rmsnorm_rows(const __half* x, const __half* gain, float eps, int rows, int d, __half* y,
@@ -1888,9 +1580,8 @@ cudaError_t launch_rmsnorm_rows(const __half* x, const __half* gain, float eps, 
     if (rows <= 0) return cudaSuccess;
     if (d % 8 != 0 || d > 16384) return cudaErrorInvalidValue;
     const int mc = row_mc(rows, d), t = row_threads(mc, d);
-    if (mc == 1) k_rmsnorm_rows<1><<<rows, t, 0, st>>>(x, gain, eps, d, y, split);
-    else k_rmsnorm_rows<2><<<rows, t, 0, st>>>(x, gain, eps, d, y, split);
-    return cudaGetLastError();
+    return mc == 1 ? launch_pk(k_rmsnorm_rows<1>, dim3(rows), t, 0, 1, st, x, gain, eps, d, y, split)
+                   : launch_pk(k_rmsnorm_rows<2>, dim3(rows), t, 0, 1, st, x, gain, eps, d, y, split);
 }
 
 static vt_status run_rmsnorm(const __half* x, const __half* gain, float eps, int n, int d, __half* y, int split,
@@ -1959,9 +1650,8 @@ static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, cudaStre
         G.n_groups = ng;
         if (heads < 1 || as[0].n < 1) continue;
         const dim3 grid(heads, (as[0].n + kFaRows - 1) / kFaRows);
-        if (as[0].dh == 128) k_prefill_attn_tc<128><<<grid, kFaThreads, fa_smem<128>(), st>>>(G);
-        else k_prefill_attn_tc<64><<<grid, kFaThreads, fa_smem<64>(), st>>>(G);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = as[0].dh == 128 ? launch_pk(k_prefill_attn_tc<128>, grid, kFaThreads, fa_smem<128>(), 1, st, G)
+                                              : launch_pk(k_prefill_attn_tc<64>, grid, kFaThreads, fa_smem<64>(), 1, st, G);
         if (e != cudaSuccess) {
             *err = std::string("prefill attention launch failed: ") + cudaGetErrorString(e);
             return VT_ERR_CUDA;

@@ -61,3 +61,25 @@ def test_prefill_rows_of_every_width(vtlib, d_model, n_dev):
         vt.vt_prefill_tokens(st.part, st.kv, torch.from_numpy(X).cuda(), 5, out)
         assert_close(out.cpu().numpy(), ref, f"prefill at d_model {d_model}")
         assert vt.vt_kv_status(st.kv) == 0
+
+
+@pytest.mark.parametrize("rows", [1, 8, 9, 120, 128, 129, 256, 257, 400])
+def test_prefill_gemm_tile_edges(vtlib, rows):
+    """Row counts around the GEMMs' A boxes (rows rounded up to 8, up to 128) and their 128- and
+    256-row tiles, an odd number of k-tiles, and down projections whose K is no multiple of 64 and
+    starts at columns that are no multiple of 8 (one k-tile per copy, shifted U)."""
+    vt = vtlib
+    from paper_2607_07046_gb300.stack import Stack
+    wl = synthetic.small("edges", n_layers=2, d_model=192, n_heads=6, n_kv_heads=3, d_head=64, d_ffn=424,
+                         head_ranges=((0, 2), (2, 6)), ffn_ranges=((0, 101), (101, 424)),
+                         kv_len=0, decode_steps=0, prompt_len=rows, model_id=145)
+    X = wl.hidden(rows, stream=13)
+    ref = X
+    for l in range(2):
+        kc, vc = oracle.new_cache(wl, rows)
+        _, ref, _, _ = oracle.tp_layer(wl, wl.layer_weights(l), ref, 0, kc, vc)
+    with Stack(shapes_of(vt, wl, max_seq=512), wl.layer_weights, wl.head_ranges, wl.ffn_ranges, rows) as st:
+        out = torch.empty((rows, 192), dtype=torch.float16, device="cuda")
+        vt.vt_prefill_tokens(st.part, st.kv, torch.from_numpy(X).cuda(), rows, out)
+        assert_close(out.cpu().numpy(), ref, f"prefill of {rows} rows")
+        assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
