@@ -35,6 +35,8 @@
 
 namespace vt {
 
+// Launch in the library's chain of programmatic dependent launches: a kernel's CTAs start, and set up
+// their barriers and tensor memory, while the preceding kernel's last CTAs finish.
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_pk(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st,
                              Args&&... args) {
@@ -43,13 +45,18 @@ static cudaError_t launch_pk(void (*kern)(KArgs...), dim3 grid, int threads, siz
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     int na = 0;
     if (cluster > 1) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
         attr[na].val.clusterDim.x = (unsigned)cluster;
         attr[na].val.clusterDim.y = 1;
         attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    if (g_use_pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
         ++na;
     }
     cfg.attrs = attr;
@@ -306,6 +313,7 @@ __global__ void __launch_bounds__(1024) k_rmsnorm_rows(const __half* __restrict_
                                                        float eps, int d, __half* __restrict__ y, int split) {
     __shared__ float red[32];
     pdl_wait();
+    pdl_launch_dependents();
     const __half* xr = x + (size_t)blockIdx.x * d;
     __half* yr = y + (size_t)blockIdx.x * d * (split ? 2 : 1);
     float v[MC][8];
@@ -350,6 +358,7 @@ __global__ void __launch_bounds__(1024) k_combine_norm(const __grid_constant__ C
                                                        __half* __restrict__ xhat, int split) {
     __shared__ float red[32];
     pdl_wait();
+    pdl_launch_dependents();
     const size_t row = blockIdx.x;
     float v[MC][8];
     float ss = 0.f;
@@ -668,6 +677,7 @@ __global__ void __launch_bounds__(kPThreads, 1) k_gemm_p(const __grid_constant__
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (the whole warp)
         pdl_wait();  // A was written by the preceding kernel
+        pdl_launch_dependents();
         uint32_t slot = 0, phase = 0, filled = 0;  // ring position; stages filled so far
         // boxes of fewer rows do not fill the ring's copy rate anyway (48-row boxes: 31.2 us without
         // the requests, 33.1 with them; 64 rows: 32.4 and 29.3)
@@ -1037,6 +1047,7 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
     const uint32_t tmem = *tmem_slot;
 
     pdl_wait();  // q and the cache rows were written by the preceding kernel
+    pdl_launch_dependents();
     // Q does not depend on the KV length: its load goes out first
     if (warp == 0 && r0 < a.n) {
         if (elect_one()) {
