@@ -509,7 +509,7 @@ def run_decode(args, rank, world):
             "kv_schedule_steps": sched,
             "partition": "heads 8/8/8/8, ffn 2752 x 4",
             "token_kernel": "fused: one cooperative kernel per token" if fused
-                            else f"per-shard kernels ({why})",
+                            else f"kernels per phase ({why})",
             "graph": "one CUDA graph per token (vt_decode_token)",
             "l2": "no flush: the 13 GB of weights streamed per step exceed the 129 MB L2",
             "parallelism": f"replicas x{world}" if world > 1 else "1 GPU",
@@ -519,7 +519,7 @@ def run_decode(args, rank, world):
             "bound": "hbm",
             "kernel": ("k_decode_token (the whole token: every shard of every layer in one "
                        "cooperative launch, so the kernel's launch time is the step time)") if fused
-                      else "the whole token step (per-shard kernels)",
+                      else "the whole token step (kernels per phase)",
             "achieved": round(achieved, 1),
             "peak": hbm,
             "unit": "GB/s",
@@ -613,7 +613,7 @@ def run_decode_workload(cid, steps, warmup, bits=16, layers=0):
                  f"{wl.d_head}, FFN {wl.d_ffn}; heads {[h1 - h0 for h0, h1 in wl.head_ranges]}, "
                  f"FFN columns {[c1 - c0 for c0, c1 in wl.ffn_ranges]}; KV {wl.kv_len} -> {wl.kv_len + sched - 1}",
         "value": round(1000.0 / ms, 3), "unit": "tok/s", "ms_per_step": round(ms, 5), "steps": steps,
-        "token_kernel": "fused: one cooperative kernel per token" if fused else f"per-shard kernels ({why})",
+        "token_kernel": "fused: one cooperative kernel per token" if fused else f"kernels per phase ({why})",
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                      "frac": round(achieved / hbm, 4), "peak_kind": f"{peak_kind} copy bandwidth",
                      "bytes_per_launch": int(step_bytes)},

@@ -354,7 +354,7 @@ VT_API vt_status vt_shard_weight_layout(const vt_partition* part, vt_shard shard
  * 4-bit codes per byte) with the fp16 scales, replacing the shard's fp16 weights (its bytes halve
  * or quarter, plus one scale per 32 weights).  Decode (vt_decode_step, vt_decode_step_static,
  * vt_decode_token_sharded) runs quantized shards with a dequantizing kernel; vt_decode_token then
- * runs the per-shard kernels (vt_decode_token_fused_available says why); prefill needs fp16
+ * runs one launch per phase (vt_decode_token_fused_available says why); prefill needs fp16
  * shards (VT_ERR_STATE).  Precisions are fixed while a KV cache of the partition exists
  * (VT_ERR_STATE): set them before vt_kv_create.  An empty shard stores nothing and stays fp16.
  * Synchronizes `stream`.  Errors: VT_ERR_INVALID_ARG (bad shard or bits), VT_ERR_ALLOC, VT_ERR_CUDA.
@@ -505,7 +505,12 @@ VT_API vt_status vt_partition_set_comm_bits(vt_partition* part, int32_t device, 
  *   Every wait in that kernel is bounded: a CTA that gives up sets VT_DEV_WAIT_TIMEOUT in the KV
  *   status word, the token's output is then undefined, and vt_kv_status(..., clear = 1) (or
  *   vt_partition_status) must be called before the next token to re-arm the grid barrier.
- *   Otherwise (unsupported shapes, or x_out not 16-byte aligned) it runs vt_decode_token_sharded.
+ *   Otherwise (unsupported shapes, or x_out not 16-byte aligned) it runs the kernels of
+ *   vt_decode_token_sharded with the shards of a block side by side: one launch per phase (and
+ *   precision).  Its results have the same bits as vt_decode_token_sharded's, except that an
+ *   attention launch with more KV heads may cut the cached positions into fewer slices (the sums
+ *   then differ in fp32 rounding; never while partials are quantized), and that fp16 FFN shards
+ *   add their partial in arrival order in both.
  *   The launch can be captured in a CUDA graph.
  */
 VT_API vt_status vt_decode_token(const vt_partition* part, vt_kv* kv, const void* x_in, void* x_out,

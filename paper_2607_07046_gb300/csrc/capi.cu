@@ -170,7 +170,6 @@ struct DecodeScratch {  // per device of the partition
     float* q = nullptr;     // [hq][dh] rotated queries of the token
     float* attn = nullptr;  // [hq][dh] attention output (input of the O projection)
     float* u = nullptr;     // [c] SwiGLU activations (quantized FFN shards)
-    int ffn_grid = 0;       // CTAs of the fused FFN kernel
 };
 
 constexpr int kPrefillChunk = 1024;  // rows per prefill pass (longer prompts run in chunks)
@@ -1024,7 +1023,6 @@ static vt_status partition_create(vt_model* m, int32_t n, const vt_range* heads,
         }
         const int hk = hq / g;
         DecodeScratch& ds = p->dec[d];
-        ds.ffn_grid = ffn_grid(c);
         const size_t bytes = align256((size_t)std::max(hq, 1) * dh * 4) * 2 + align256((size_t)std::max(c, 1) * 4);
         void* q;
         if ((r = owned_alloc(p, bytes, &q)) != VT_OK) return bail(r);
@@ -1205,9 +1203,8 @@ static QMatDev take_qmat(Bump& b, int rows, int k, int bits) {
     m.k = k;
     m.nb = (k + kQBlock - 1) / kQBlock;
     m.bits = bits;
-    m.row_bytes = (int64_t)m.nb * (bits == 8 ? 32 : 16);
     m.codes = b.take<uint8_t>(qmat_code_bytes(rows, k, bits));
-    m.scales = b.take<__half>((size_t)rows * m.nb);
+    m.scales = b.take<__half>(qmat_scale_bytes(rows, k) / 2);
     return m;
 }
 
@@ -1351,10 +1348,11 @@ extern "C" vt_status vt_shard_qweights_read(const vt_partition* p, vt_shard sh, 
     }
     if (!codes || !scales) return fail(VT_ERR_INVALID_ARG, "codes and scales must not be NULL");
     std::vector<uint8_t> raw(qmat_code_bytes(m->rows, m->k, m->bits));
+    std::vector<__half> sc(qmat_scale_bytes(m->rows, m->k) / 2);
     VT_CUDA(cudaDeviceSynchronize());
     VT_CUDA(cudaMemcpy(raw.data(), m->codes, raw.size(), cudaMemcpyDeviceToHost));
-    VT_CUDA(cudaMemcpy(scales, m->scales, qmat_scale_bytes(m->rows, m->k), cudaMemcpyDeviceToHost));
-    unpack_qcodes(raw.data(), m->rows, m->k, m->bits, codes);
+    VT_CUDA(cudaMemcpy(sc.data(), m->scales, sc.size() * 2, cudaMemcpyDeviceToHost));
+    unpack_qmat(raw.data(), sc.data(), m->rows, m->k, m->bits, codes, static_cast<__half*>(scales));
     return ok();
 }
 
@@ -1546,160 +1544,182 @@ extern "C" vt_status vt_kv_write_raw(vt_kv* kv, int32_t l, int32_t d, int32_t n_
 // ================================================================== shard compute
 
 // QKV projection of ATTN shard (l, d) with RoPE and the K/V append at the layer's length: the
-// fp16 GEMV or, for a block-quantized shard, the dequantizing one.  q: [hq][dh] rotated queries.
+// One phase of a block of layer l: the block-quantized shards of `dev` (n devices, none empty) in one
+// launch, the fp16 ones in another, whose input is then at least two launches old: it streams
+// beside the first.  Both kinds of arguments are filled in from the same description of the phase.
+struct DecodePhase {
+    GemvArgs g[VT_MAX_DEVICES];
+    QGemvArgs q[VT_MAX_DEVICES];
+    int ng = 0, nq = 0;
+    cudaError_t launch(int epi, cudaStream_t st) {
+        const cudaError_t e = nq > 0 ? launch_gemv_q(epi, q, nq, st) : cudaSuccess;
+        for (int i = 0; i < ng && nq > 0; ++i) g[i].indep = 1;
+        return e == cudaSuccess && ng > 0 ? launch_gemv(epi, g, ng, st) : e;
+    }
+};
+
+// QKV projections with RoPE and the K / V append: shard dev[i] writes its rotated queries to q[i].
 // indep: the caller guarantees that `x` was written at least two kernel launches before (the
 // fp16 GEMV may then read it before griddepcontrol.wait).
-static cudaError_t attn_qkv(const vt_partition* p, int l, int d, const __half* x, vt_kv* kv, float* q,
-                            cudaStream_t st, int indep) {
+static cudaError_t attn_qkv(const vt_partition* p, int l, const int* dev, int n, const __half* x, vt_kv* kv,
+                            float* const* q, cudaStream_t st, int indep) {
     const vt_shapes& s = p->m->s;
-    const AttnShard& a = p->a(l, d);
-    const int hq = a.h1 - a.h0, hk = a.kv1 - a.kv0, dh = s.d_head, D = s.d_model;
-    if (a.bits != 16) {
-        QGemvArgs g{};
-        g.w = a.qkv;
-        g.x = x;
-        g.gain = a.norm;
-        g.eps = s.rms_eps;
-        g.out = q;
-        g.kcache = kv->k(l, d);
-        g.vcache = kv->v(l, d);
-        g.cap = kv->cap;
-        g.len = kv->len + l;
-        g.rope = p->m->rope;
-        g.dh = dh;
-        g.hq = hq;
-        g.hk = hk;
-        g.status = kv->status;
-        return launch_gemv_q(kEpiQkvRope, g, st);
+    DecodePhase ph;
+    for (int i = 0; i < n; ++i) {
+        const int d = dev[i];
+        const AttnShard& a = p->a(l, d);
+        auto common = [&](auto& g) {
+            g.x = x;
+            g.gain = a.norm;
+            g.eps = s.rms_eps;
+            g.out = q[i];
+            g.kcache = kv->k(l, d);
+            g.vcache = kv->v(l, d);
+            g.cap = kv->cap;
+            g.len = kv->len + l;
+            g.rope = p->m->rope;
+            g.dh = s.d_head;
+            g.hq = a.h1 - a.h0;
+            g.hk = a.kv1 - a.kv0;
+            g.status = kv->status;
+        };
+        if (a.bits != 16) {
+            QGemvArgs& g = ph.q[ph.nq++] = QGemvArgs{};
+            common(g);
+            g.w = a.qkv;
+        } else {
+            GemvArgs& g = ph.g[ph.ng++] = GemvArgs{};
+            common(g);
+            g.w = a.wqkv;
+            g.row_stride = s.d_model;
+            g.rows = (g.hq + 2 * g.hk) * s.d_head;
+            g.k = s.d_model;
+            g.indep = indep;
+        }
     }
-    GemvArgs g{};
-    g.w = a.wqkv;
-    g.row_stride = D;
-    g.rows = (hq + 2 * hk) * dh;
-    g.k = D;
-    g.x = x;
-    g.gain = a.norm;
-    g.eps = s.rms_eps;
-    g.out = q;
-    g.kcache = kv->k(l, d);
-    g.vcache = kv->v(l, d);
-    g.cap = kv->cap;
-    g.len = kv->len + l;
-    g.rope = p->m->rope;
-    g.dh = dh;
-    g.hq = hq;
-    g.hk = hk;
-    g.status = kv->status;
-    g.indep = indep;
-    return launch_gemv(kEpiQkvRope, g, st);
+    return ph.launch(kEpiQkvRope, st);
 }
 
-// Attention of ATTN shard (l, d) over the cache: q [hq][dh] rotated queries -> attn [hq][dh].
-static cudaError_t attn_slices(const vt_partition* p, int l, int d, const float* q, vt_kv* kv, float* attn,
-                               cudaStream_t st) {
+// Attention of the shards over the cache: q[i] [hq][dh] rotated queries -> attn[i] [hq][dh].
+static cudaError_t attn_slices(const vt_partition* p, int l, const int* dev, int n, float* const* q, vt_kv* kv,
+                               float* const* attn, cudaStream_t st) {
     const vt_shapes& s = p->m->s;
-    const AttnShard& a = p->a(l, d);
     AttnDecodeArgs t{};
-    t.q = q;
-    t.kcache = kv->k(l, d);
-    t.vcache = kv->v(l, d);
+    int hk = 0;
+    for (int i = 0; i < n; ++i) {
+        const AttnShard& a = p->a(l, dev[i]);
+        hk += a.kv1 - a.kv0;
+        t.hk_end[i] = hk;
+        t.q[i] = q[i];
+        t.kcache[i] = kv->k(l, dev[i]);
+        t.vcache[i] = kv->v(l, dev[i]);
+        t.out[i] = attn[i];
+    }
+    t.n = n;
     t.len = kv->len + l;
     t.cap = kv->cap;
-    t.hk = a.kv1 - a.kv0;
     t.group = s.n_heads / s.n_kv_heads;
     t.dh = s.d_head;
-    t.stages = attn_stages(kv->cap, attn_cluster_size(t.hk));
+    // Partials that travel quantized keep 16 slices a head: a code may differ where a value lies at a
+    // tie, so their tokens have the same bits shard by shard and grouped.
+    bool quantized = false;
+    for (int b : p->comm_bits) quantized |= b != 16;
+    const int span = t.window > 0 ? std::min(t.window, kv->cap) : kv->cap;
+    t.cluster = attn_cluster_size(hk, t.n, span, quantized);
+    t.stages = attn_stages(span, t.cluster);
     t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)s.d_head));
     t.window = p->m->window[l];
-    t.out = attn;
     t.status = kv->status;
     return launch_attn_decode(t, st);
 }
 
-// O projection of ATTN shard (l, d): out [D] = Wo_s . attn (fp32), fp16 or block-quantized.
-static cudaError_t attn_o(const vt_partition* p, int l, int d, const float* attn, float* out, uint32_t* status,
-                          cudaStream_t st) {
+// O projections: out[i] [D] = Wo_s . attn[i] (fp32).
+static cudaError_t attn_o(const vt_partition* p, int l, const int* dev, int n, float* const* attn, float* const* out,
+                          uint32_t* status, cudaStream_t st) {
     const vt_shapes& s = p->m->s;
-    const AttnShard& a = p->a(l, d);
-    const int hq = a.h1 - a.h0, dh = s.d_head, D = s.d_model;
-    if (a.bits != 16) {
-        QGemvArgs o{};
-        o.w = a.o;
-        o.vin = attn;
-        o.out = out;
-        o.status = status;
-        return launch_gemv_q(kEpiPlain, o, st);
+    DecodePhase ph;
+    for (int i = 0; i < n; ++i) {
+        const AttnShard& a = p->a(l, dev[i]);
+        auto common = [&](auto& o) {
+            o.vin = attn[i];
+            o.out = out[i];
+            o.status = status;
+        };
+        if (a.bits != 16) {
+            QGemvArgs& o = ph.q[ph.nq++] = QGemvArgs{};
+            common(o);
+            o.w = a.o;
+        } else {
+            GemvArgs& o = ph.g[ph.ng++] = GemvArgs{};
+            common(o);
+            o.w = a.wo;
+            o.k = (a.h1 - a.h0) * s.d_head;
+            o.row_stride = o.k;
+            o.rows = s.d_model;
+        }
     }
-    GemvArgs o{};
-    o.w = a.wo;
-    o.row_stride = (int64_t)hq * dh;
-    o.rows = D;
-    o.k = hq * dh;
-    o.vin = attn;
-    o.out = out;
-    o.status = status;
-    return launch_gemv(kEpiPlain, o, st);
+    return ph.launch(kEpiPlain, st);
 }
 
-// indep: the caller guarantees that `x` was written at least two kernel launches before this
-// shard's first kernel, so that kernel may read it before griddepcontrol.wait (see k_gemv).
-static vt_status decode_attn(const vt_partition* p, int l, int d, const __half* x, vt_kv* kv,
-                             float* out, cudaStream_t st, int indep = 0) {
-    const vt_shapes& s = p->m->s;
-    const AttnShard& a = p->a(l, d);
-    const DecodeScratch& ds = p->dec[d];
-    const int hq = a.h1 - a.h0, D = s.d_model;
-    if (hq == 0) {
-        VT_CUDA(launch_fill_zero_f32(out, D, st));
-        return VT_OK;
+// The ATTN shards dev[0 .. n) of layer l, side by side in three phases (none of them empty).
+// indep: the caller guarantees that `x` was written at least two kernel launches before the first
+// kernel, so that kernel may read it before griddepcontrol.wait (see k_gemv).
+static vt_status decode_attn(const vt_partition* p, int l, const int* dev, int n, const __half* x, vt_kv* kv,
+                             float* const* out, cudaStream_t st, int indep = 0) {
+    float *q[VT_MAX_DEVICES], *attn[VT_MAX_DEVICES];
+    for (int i = 0; i < n; ++i) {
+        q[i] = p->dec[dev[i]].q;
+        attn[i] = p->dec[dev[i]].attn;
     }
-    VT_CUDA(attn_qkv(p, l, d, x, kv, ds.q, st, indep));
-
-    VT_CUDA(attn_slices(p, l, d, ds.q, kv, ds.attn, st));
-    VT_CUDA(attn_o(p, l, d, ds.attn, out, kv->status, st));
+    VT_CUDA(attn_qkv(p, l, dev, n, x, kv, q, st, indep));
+    VT_CUDA(attn_slices(p, l, dev, n, q, kv, attn, st));
+    VT_CUDA(attn_o(p, l, dev, n, attn, out, kv->status, st));
     return VT_OK;
 }
 
-// FFN shard decode: the fused column-split kernel adds every CTA's partial into `out`, which
-// must hold zeros; `zero_first` clears it in stream order before the kernel runs.
-static vt_status decode_ffn(const vt_partition* p, int l, int d, const __half* x, float* out,
-                            cudaStream_t st, int indep = 0, bool zero_first = true) {
+// The FFN shards dev[0 .. n) of layer l (none of them empty).  fp16 shards: the fused column-split
+// kernel adds every CTA's partial into out[i], which must hold zeros.  Block-quantized shards:
+// gate/up rows with the SwiGLU epilogue, then the down columns (the partial is written, not added).
+static vt_status decode_ffn(const vt_partition* p, int l, const int* dev, int n, const __half* x, float* const* out,
+                            cudaStream_t st, int indep = 0) {
     const vt_shapes& s = p->m->s;
-    const FfnShard& f = p->f(l, d);
-    const DecodeScratch& ds = p->dec[d];
-    const int c = f.c1 - f.c0, D = s.d_model;
-    if (f.bits != 16 && c > 0) {
-        // block-quantized shard: gate/up rows with the SwiGLU epilogue, then the down columns (the
-        // partial is written, not added)
-        QGemvArgs g{};
-        g.w = f.gu;
-        g.x = x;
-        g.gain = f.norm;
-        g.eps = s.rms_eps;
-        g.out = ds.u;
-        g.status = p->status;
-        VT_CUDA(launch_gemv_q(kEpiSwiglu, g, st));
-        QGemvArgs o{};
-        o.w = f.down;
-        o.vin = ds.u;
-        o.out = out;
-        o.status = p->status;
-        VT_CUDA(launch_gemv_q(kEpiPlain, o, st));
-        return VT_OK;
+    FfnDecodeArgs fa[VT_MAX_DEVICES];
+    QGemvArgs gu[VT_MAX_DEVICES], down[VT_MAX_DEVICES];
+    int nf = 0, nq = 0;
+    for (int i = 0; i < n; ++i) {
+        const FfnShard& f = p->f(l, dev[i]);
+        if (f.bits != 16) {
+            QGemvArgs g{}, o{};
+            g.w = f.gu;
+            g.x = x;
+            g.gain = f.norm;
+            g.eps = s.rms_eps;
+            g.out = p->dec[dev[i]].u;
+            g.status = p->status;
+            o.w = f.down;
+            o.vin = p->dec[dev[i]].u;
+            o.out = out[i];
+            o.status = p->status;
+            gu[nq] = g;
+            down[nq++] = o;
+        } else {
+            FfnDecodeArgs g{};
+            g.x = x;
+            g.gain = f.norm;
+            g.eps = s.rms_eps;
+            g.wgu = f.wgu;
+            g.wdt = f.wdt;
+            g.d = s.d_model;
+            g.cols = f.c1 - f.c0;
+            g.out = out[i];
+            g.indep = indep;
+            fa[nf++] = g;
+        }
     }
-    if (zero_first) VT_CUDA(launch_fill_zero_f32(out, D, st));
-    if (c == 0) return VT_OK;
-    FfnDecodeArgs g{};
-    g.x = x;
-    g.gain = f.norm;
-    g.eps = s.rms_eps;
-    g.wgu = f.wgu;
-    g.wdt = f.wdt;
-    g.d = D;
-    g.cols = c;
-    g.out = out;
-    g.indep = indep;
-    VT_CUDA(launch_ffn_decode(g, ds.ffn_grid, st));
+    if (nq > 0) VT_CUDA(launch_gemv_q(kEpiSwiglu, gu, nq, st));
+    for (int i = 0; i < nf && nq > 0; ++i) fa[i].indep = 1;  // (x is then two launches old)
+    if (nf > 0) VT_CUDA(launch_ffn_decode(fa, nf, st));
+    if (nq > 0) VT_CUDA(launch_gemv_q(kEpiPlain, down, nq, st));
     return VT_OK;
 }
 
@@ -1709,14 +1729,19 @@ extern "C" vt_status vt_decode_step(const vt_partition* p, vt_shard sh, const vo
     if (!x || !out) return fail(VT_ERR_INVALID_ARG, "x and out_partial must not be NULL");
     if (!aligned16(x)) return fail(VT_ERR_INVALID_ARG, "x must be 16-byte aligned");
     cudaStream_t st = (cudaStream_t)stream;
+    const int D = p->m->s.d_model;
     if (sh.block == VT_BLOCK_ATTN) {
         if (!kv || kv->p != p) return fail(VT_ERR_INVALID_ARG, "an ATTN shard needs this partition's KV cache");
         if (kv->h_len[sh.layer] + 1 > kv->cap)
             return fail(VT_ERR_KV_CAPACITY, "layer %d holds %d of %d positions", sh.layer,
                         kv->h_len[sh.layer], kv->cap);
-        VT_TRY(decode_attn(p, sh.layer, sh.device, static_cast<const __half*>(x), kv, out, st));
+        const AttnShard& a = p->a(sh.layer, sh.device);
+        if (a.h1 == a.h0) VT_CUDA(launch_fill_zero_f32(out, D, st));
+        else VT_TRY(decode_attn(p, sh.layer, &sh.device, 1, static_cast<const __half*>(x), kv, &out, st));
     } else {
-        VT_TRY(decode_ffn(p, sh.layer, sh.device, static_cast<const __half*>(x), out, st));
+        const FfnShard& f = p->f(sh.layer, sh.device);
+        if (f.c1 == f.c0 || f.bits == 16) VT_CUDA(launch_fill_zero_f32(out, D, st));  // (fp16: the kernel adds to it)
+        if (f.c1 > f.c0) VT_TRY(decode_ffn(p, sh.layer, &sh.device, 1, static_cast<const __half*>(x), &out, st));
     }
     return ok();
 }
@@ -1755,10 +1780,9 @@ extern "C" vt_status vt_decode_step_static(const vt_partition* p, vt_shard sh, c
     float* q = reinterpret_cast<float*>(b + lay.q);
     float* attn = reinterpret_cast<float*>(b + lay.attn);
 
-    VT_CUDA(attn_qkv(p, l, d, static_cast<const __half*>(x), kv, q, st, 0));
-
-    VT_CUDA(attn_slices(p, l, d, q, kv, attn, st));
-    VT_CUDA(attn_o(p, l, d, attn, out, kv->status, st));
+    VT_CUDA(attn_qkv(p, l, &d, 1, static_cast<const __half*>(x), kv, &q, st, 0));
+    VT_CUDA(attn_slices(p, l, &d, 1, &q, kv, &attn, st));
+    VT_CUDA(attn_o(p, l, &d, 1, &attn, &out, kv->status, st));
     return ok();
 }
 
@@ -1962,26 +1986,6 @@ extern "C" vt_status vt_token_test_barrier(vt_partition* p, int32_t cta, uint32_
     return ok();
 }
 
-extern "C" vt_status vt_decode_token(const vt_partition* p, vt_kv* kv, const void* x_in, void* x_out,
-                                     vt_stream stream) {
-    VT_TRY(check_token_args(p, kv, x_in, x_out));
-    if (!p->tok_ok || !kv->tok_tab || !aligned16(x_out)) return vt_decode_token_sharded(p, kv, x_in, x_out, stream);
-    const vt_shapes& s = p->m->s;
-    TokArgs t = p->tok_base;
-    t.cap = kv->cap;
-    t.shard = static_cast<const TokShardPtrs*>(kv->tok_tab);
-    t.layer = reinterpret_cast<const TokLayerPtrs*>(static_cast<const uint8_t*>(kv->tok_tab) +
-                                                    align256((size_t)s.n_layers * p->n_dev * sizeof(TokShardPtrs)));
-    t.len = kv->len;
-    t.x_in = static_cast<const __half*>(x_in);
-    t.x_out = static_cast<__half*>(x_out);
-    t.status = kv->status;
-    VT_CUDA(launch_decode_token(t, p->tok_plan, (cudaStream_t)stream));
-    if (!capturing((cudaStream_t)stream))
-        for (int l = 0; l < s.n_layers; ++l) kv->h_len[l] += 1;
-    return ok();
-}
-
 // The combine of one block of the whole-token path: the plain fp32 combine, or, when some
 // device's partials travel quantized (communication scaling), the combine that quantizes each such
 // partial on its way (both clear the fp32 partials).
@@ -2049,11 +2053,17 @@ extern "C" vt_status vt_combine_q(const void* const* codes, const void* const* s
     return ok();
 }
 
-extern "C" vt_status vt_decode_token_sharded(const vt_partition* p, vt_kv* kv, const void* x_in, void* x_out,
-                                             vt_stream stream) {
+// One token through the decode kernels of every layer, the shards of a block one after another, or
+// (`grouped`) side by side: one launch per phase of a block (and precision) for all of them.
+//
+// A launch of these kernels costs 5 to 8 us however small its shard is (start, prologue, drain), so
+// for partitions that the fused kernel does not take, the number of launches is what bounds a token:
+// seven phases a layer instead of seven per shard.  Llama-2-7B shapes, four 8-bit shards, 1024
+// cached positions: 94 us a token and layer, against 186 shard by shard.
+static vt_status decode_token_kernels(const vt_partition* p, vt_kv* kv, const void* x_in, void* x_out, cudaStream_t st,
+                                      bool grouped) {
     VT_TRY(check_token_args(p, kv, x_in, x_out));
     const vt_shapes& s = p->m->s;
-    cudaStream_t st = (cudaStream_t)stream;
     const int D = s.d_model, n = p->n_dev;
     // One fp32 partial buffer per shard serves both blocks: the O projection stores the ATTN
     // partial; the ATTN combine reads and clears it; the FFN kernels add into it; the FFN combine
@@ -2065,33 +2075,57 @@ extern "C" vt_status vt_decode_token_sharded(const vt_partition* p, vt_kv* kv, c
     for (int d = 0; d < n; ++d) c.parts[d] = p->dpart + (size_t)d * D;
     const __half* cur = static_cast<const __half*>(x_in);
     for (int l = 0; l < s.n_layers; ++l) {
-        // After the first launched shard of a block, a shard's input was written by the combine
-        // at least two launches earlier, so its first kernel may read it before waiting.
-        bool launched = false;
-        for (int d = 0; d < n; ++d) {
-            const AttnShard& as = p->a(l, d);
-            if (as.h1 == as.h0) continue;
-            VT_TRY(decode_attn(p, l, d, cur, kv, p->dpart + (size_t)d * D, st, launched));
-            launched = true;
+        for (int block : {VT_BLOCK_ATTN, VT_BLOCK_FFN}) {
+            int dev[VT_MAX_DEVICES], m = 0;
+            float* out[VT_MAX_DEVICES];
+            for (int d = 0; d < n; ++d) {
+                const bool empty = block == VT_BLOCK_ATTN ? p->a(l, d).h1 == p->a(l, d).h0 : p->f(l, d).c1 == p->f(l, d).c0;
+                if (empty) continue;
+                dev[m] = d;
+                out[m++] = c.parts[d];
+            }
+            // Shard by shard, every shard after the first of its block has an input that the combine
+            // wrote at least two launches earlier: its first kernel may read it before waiting.
+            const int step = grouped ? m : 1;
+            for (int i = 0; i < m; i += step) {
+                if (block == VT_BLOCK_ATTN) VT_TRY(decode_attn(p, l, dev + i, step, cur, kv, out + i, st, i > 0));
+                else VT_TRY(decode_ffn(p, l, dev + i, step, p->hbuf, out + i, st, i > 0));
+            }
+            const bool last = block == VT_BLOCK_FFN && l == s.n_layers - 1;
+            c.residual = block == VT_BLOCK_ATTN ? cur : p->hbuf;
+            c.out = block == VT_BLOCK_ATTN ? p->hbuf : (last ? static_cast<__half*>(x_out) : p->xbuf);
+            VT_TRY(combine_block(p, l, (vt_block)block, c, st));
+            if (block == VT_BLOCK_FFN) cur = c.out;
         }
-        c.residual = cur;
-        c.out = p->hbuf;
-        VT_TRY(combine_block(p, l, VT_BLOCK_ATTN, c, st));
-        launched = false;
-        for (int d = 0; d < n; ++d) {
-            const FfnShard& fs = p->f(l, d);
-            if (fs.c1 == fs.c0) continue;
-            VT_TRY(decode_ffn(p, l, d, p->hbuf, p->dpart + (size_t)d * D, st, launched, false));
-            launched = true;
-        }
-        __half* dst = (l == s.n_layers - 1) ? static_cast<__half*>(x_out) : p->xbuf;
-        c.residual = p->hbuf;
-        c.out = dst;
-        VT_TRY(combine_block(p, l, VT_BLOCK_FFN, c, st));
-        cur = dst;
     }
     VT_CUDA(launch_kv_advance(kv->len, 0, s.n_layers, 1, kv->cap, kv->status, st));
     if (!capturing(st))
+        for (int l = 0; l < s.n_layers; ++l) kv->h_len[l] += 1;
+    return ok();
+}
+
+extern "C" vt_status vt_decode_token_sharded(const vt_partition* p, vt_kv* kv, const void* x_in, void* x_out,
+                                             vt_stream stream) {
+    return decode_token_kernels(p, kv, x_in, x_out, (cudaStream_t)stream, false);
+}
+
+extern "C" vt_status vt_decode_token(const vt_partition* p, vt_kv* kv, const void* x_in, void* x_out,
+                                     vt_stream stream) {
+    VT_TRY(check_token_args(p, kv, x_in, x_out));
+    if (!p->tok_ok || !kv->tok_tab || !aligned16(x_out))
+        return decode_token_kernels(p, kv, x_in, x_out, (cudaStream_t)stream, true);
+    const vt_shapes& s = p->m->s;
+    TokArgs t = p->tok_base;
+    t.cap = kv->cap;
+    t.shard = static_cast<const TokShardPtrs*>(kv->tok_tab);
+    t.layer = reinterpret_cast<const TokLayerPtrs*>(static_cast<const uint8_t*>(kv->tok_tab) +
+                                                    align256((size_t)s.n_layers * p->n_dev * sizeof(TokShardPtrs)));
+    t.len = kv->len;
+    t.x_in = static_cast<const __half*>(x_in);
+    t.x_out = static_cast<__half*>(x_out);
+    t.status = kv->status;
+    VT_CUDA(launch_decode_token(t, p->tok_plan, (cudaStream_t)stream));
+    if (!capturing((cudaStream_t)stream))
         for (int l = 0; l < s.n_layers; ++l) kv->h_len[l] += 1;
     return ok();
 }

@@ -22,6 +22,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "device.cuh"
@@ -68,7 +69,7 @@ static cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
 static __host__ __device__ __forceinline__ int round_up8(int k) { return (k + 7) & ~7; }
 
 // Chunks per lane for a row of `k` columns: the choice with the best use of the 8 warps' lanes.
-int gemv_cpl(int k) {
+static int gemv_cpl(int k) {
     const int nch = round_up8(k) / 8;
     static const int cand[] = {1, 2, 3, 4, 8};
     int best = 8;
@@ -86,28 +87,45 @@ int gemv_cpl(int k) {
     return best;
 }
 
-int gemv_grid(int rows, int unit) {
-    const int units = rows / unit;
-    if (units <= 0) return 0;
-    int g = (g_num_sms > 0 ? g_num_sms : 148) * g_grid_mult;
-    const int per = kGemvMaxSlabRows / unit;
-    const int need = (units + per - 1) / per;
-    if (g < need) g = need;
-    if (g > units) g = units;
+// Deals `ctas` CTAs out to n shards by their bytes: shard s gets end[s] - end[s - 1], at least enough
+// for its units at `per` units a CTA, at most one per unit.  Returns the launch's CTAs.
+static int deal_ctas(const double* bytes, const int* units, int per, int n, int ctas, int* end) {
+    double tot = 0;
+    for (int s = 0; s < n; ++s) tot += bytes[s];
+    int acc = 0;
+    for (int s = 0; s < n; ++s) {
+        int g = n == 1 ? ctas : (int)(ctas * bytes[s] / tot + 0.5);
+        g = std::min(std::max({g, (units[s] + per - 1) / per, 1}), units[s]);
+        acc += g;
+        end[s] = acc;
+    }
+    return acc;
+}
+
+// The shard of CTA `x` of the launch, and the CTA's number and the CTAs within that shard.
+template <class Group>
+__device__ __forceinline__ int group_of(const Group& G, int x, int& bx, int& nb) {
+    int g = 0;
+    while (g + 1 < G.n && x >= G.end[g]) ++g;
+    const int first = g > 0 ? G.end[g - 1] : 0;
+    bx = x - first;
+    nb = G.end[g] - first;
     return g;
 }
 
-template <int EPI, int CPL, int R>
+template <int EPI, int CPL, int R, int NG>
 __global__ void __launch_bounds__(kGemvThreads, (CPL <= 4 ? 2 : 1))
-    k_gemv(const __grid_constant__ GemvArgs a) {
+    k_gemv(const __grid_constant__ DecodeGroup<GemvArgs, NG> G) {
     constexpr int NB = R * CPL;  // chunks per lane per batch
+    int bx = (int)blockIdx.x, nbx = (int)gridDim.x;
+    const GemvArgs& a = G.a[NG > 1 ? group_of(G, bx, bx, nbx) : 0];
     __shared__ float slots[kGemvMaxSlabRows * kGemvWarps];
     __shared__ float red[kGemvWarps + 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int unit = (EPI == kEpiPlain) ? 1 : 2;
     const int units = a.rows / unit;
-    const int r0 = (int)(((int64_t)blockIdx.x * units) / gridDim.x) * unit;
-    const int r1 = (int)(((int64_t)(blockIdx.x + 1) * units) / gridDim.x) * unit;
+    const int r0 = (int)(((int64_t)bx * units) / nbx) * unit;
+    const int r1 = (int)(((int64_t)(bx + 1) * units) / nbx) * unit;
     const int nrows = r1 - r0;
     const int nch = round_up8(a.k) >> 3;
     const int wpr = (nch + 32 * CPL - 1) / (32 * CPL);
@@ -217,11 +235,6 @@ __global__ void __launch_bounds__(kGemvThreads, (CPL <= 4 ? 2 : 1))
     };
     if constexpr (EPI == kEpiPlain) {
         for (int r = tid; r < nrows; r += kGemvThreads) a.out[r0 + r] = row_value(r);
-    } else if constexpr (EPI == kEpiSwiglu) {
-        for (int t = tid; t < nrows / 2; t += kGemvThreads) {
-            const float g = row_value(2 * t), u = row_value(2 * t + 1);
-            a.out[r0 / 2 + t] = silu(g) * u;
-        }
     } else {  // kEpiQkvRope
         const int p = *a.len;
         const bool ok = p >= 0 && p < a.cap;
@@ -267,24 +280,17 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) 
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-int ffn_grid(int cols) {
-    if (cols <= 0) return 0;
-    int g = (g_num_sms > 0 ? g_num_sms : 148) * g_grid_mult;
-    const int need = (cols + kFfnMaxCols - 1) / kFfnMaxCols;
-    if (g < need) g = need;
-    if (g > cols) g = cols;
-    return g;
-}
-
-template <int CPL, int R, int MC>
-__global__ void __launch_bounds__(kGemvThreads, 2) k_ffn(const __grid_constant__ FfnDecodeArgs a) {
+template <int CPL, int R, int MC, int NG>
+__global__ void __launch_bounds__(kGemvThreads, 2) k_ffn(const __grid_constant__ DecodeGroup<FfnDecodeArgs, NG> G) {
     constexpr int NB = R * CPL;
+    int bx = (int)blockIdx.x, nbx = (int)gridDim.x;
+    const FfnDecodeArgs& a = G.a[NG > 1 ? group_of(G, bx, bx, nbx) : 0];
     __shared__ float slots[2 * kFfnMaxCols * kGemvWarps];
     __shared__ float act[kFfnMaxCols];
     __shared__ float red[kGemvWarps + 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int j0 = (int)(((int64_t)blockIdx.x * a.cols) / gridDim.x);
-    const int j1 = (int)(((int64_t)(blockIdx.x + 1) * a.cols) / gridDim.x);
+    const int j0 = (int)(((int64_t)bx * a.cols) / nbx);
+    const int j1 = (int)(((int64_t)(bx + 1) * a.cols) / nbx);
     const int ncol = j1 - j0;
     const int nrows = 2 * ncol;
     const int D = a.d;
@@ -457,50 +463,87 @@ __global__ void __launch_bounds__(kGemvThreads, 2) k_ffn(const __grid_constant__
     __syncthreads();
 }
 
-template <int CPL, int R>
-static cudaError_t launch_ffn_cpl(const FfnDecodeArgs& a, int grid, cudaStream_t st) {
-    const int mc = ((a.d >> 3) + kGemvThreads - 1) / kGemvThreads;
-    const dim3 g(grid), b(kGemvThreads);
-    const size_t sm = (size_t)a.d * 4;
-    if (mc <= 1) return launch_k(k_ffn<CPL, R, 1>, g, b, sm, st, a);
-    if (mc <= 2) return launch_k(k_ffn<CPL, R, 2>, g, b, sm, st, a);
-    if (mc <= 3) return launch_k(k_ffn<CPL, R, 3>, g, b, sm, st, a);
-    if (mc <= 4) return launch_k(k_ffn<CPL, R, 4>, g, b, sm, st, a);
-    return launch_k(k_ffn<CPL, R, 8>, g, b, sm, st, a);
+template <int CPL, int R, int NG>
+static cudaError_t launch_ffn_cpl(const DecodeGroup<FfnDecodeArgs, NG>& G, cudaStream_t st) {
+    const int d = G.a[0].d, mc = ((d >> 3) + kGemvThreads - 1) / kGemvThreads;
+    const dim3 g(G.end[G.n - 1]), b(kGemvThreads);
+    const size_t sm = (size_t)d * 4;
+    if (mc <= 1) return launch_k(k_ffn<CPL, R, 1, NG>, g, b, sm, st, G);
+    if (mc <= 2) return launch_k(k_ffn<CPL, R, 2, NG>, g, b, sm, st, G);
+    if (mc <= 3) return launch_k(k_ffn<CPL, R, 3, NG>, g, b, sm, st, G);
+    if (mc <= 4) return launch_k(k_ffn<CPL, R, 4, NG>, g, b, sm, st, G);
+    return launch_k(k_ffn<CPL, R, 8, NG>, g, b, sm, st, G);
 }
 
-cudaError_t launch_ffn_decode(const FfnDecodeArgs& a, int grid, cudaStream_t st) {
-    if (grid <= 0) return cudaSuccess;
-    switch (gemv_cpl(a.d)) {
-        case 1: return launch_ffn_cpl<1, 8>(a, grid, st);
-        case 2: return launch_ffn_cpl<2, 4>(a, grid, st);
-        case 3: return launch_ffn_cpl<3, 2>(a, grid, st);
-        case 4: return launch_ffn_cpl<4, 2>(a, grid, st);
-        default: return launch_ffn_cpl<8, 1>(a, grid, st);
+template <int NG>
+static cudaError_t launch_ffn_group(const FfnDecodeArgs* a, int n, cudaStream_t st) {
+    DecodeGroup<FfnDecodeArgs, NG> G{};
+    double bytes[NG];
+    int units[NG];
+    for (int s = 0; s < n; ++s) {
+        G.a[s] = a[s];
+        bytes[s] = units[s] = a[s].cols;
+    }
+    G.n = n;
+    // one CTA an SM for a shard; two for a whole block, whose columns would not fit in one
+    deal_ctas(bytes, units, kFfnMaxCols, n, (g_num_sms > 0 ? g_num_sms : 148) * g_grid_mult * (n > 1 ? 2 : 1), G.end);
+    switch (gemv_cpl(a[0].d)) {
+        case 1: return launch_ffn_cpl<1, 8, NG>(G, st);
+        case 2: return launch_ffn_cpl<2, 4, NG>(G, st);
+        case 3: return launch_ffn_cpl<3, 2, NG>(G, st);
+        case 4: return launch_ffn_cpl<4, 2, NG>(G, st);
+        default: return launch_ffn_cpl<8, 1, NG>(G, st);
     }
 }
 
+cudaError_t launch_ffn_decode(const FfnDecodeArgs* a, int n, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    return n == 1 ? launch_ffn_group<1>(a, n, st) : launch_ffn_group<VT_MAX_DEVICES>(a, n, st);
+}
+
+// (every shard of a launch has the same chunks per lane, `cpl`: the order of a row's sums)
+template <int EPI, int NG>
+static cudaError_t launch_gemv_group(const GemvArgs* a, int n, int cpl, cudaStream_t st) {
+    constexpr int unit = EPI == kEpiPlain ? 1 : 2;
+    DecodeGroup<GemvArgs, NG> G{};
+    double bytes[NG];
+    int units[NG];
+    for (int s = 0; s < n; ++s) {
+        G.a[s] = a[s];
+        units[s] = a[s].rows / unit;
+        bytes[s] = (double)a[s].rows * a[s].k;
+    }
+    G.n = n;
+    const dim3 g(deal_ctas(bytes, units, kGemvMaxSlabRows / unit, n, (g_num_sms > 0 ? g_num_sms : 148) * g_grid_mult, G.end)),
+        b(kGemvThreads);
+    switch (cpl) {
+        case 1: return launch_k(k_gemv<EPI, 1, 8, NG>, g, b, 0, st, G);
+        case 2: return launch_k(k_gemv<EPI, 2, 4, NG>, g, b, 0, st, G);
+        case 3: return launch_k(k_gemv<EPI, 3, 2, NG>, g, b, 0, st, G);
+        case 4: return launch_k(k_gemv<EPI, 4, 2, NG>, g, b, 0, st, G);
+        default: return launch_k(k_gemv<EPI, 8, 1, NG>, g, b, 0, st, G);
+    }
+}
+
+// (fp16 FFN shards run on k_ffn, so there is no SwiGLU epilogue here)
 template <int EPI>
-static cudaError_t launch_gemv_epi(const GemvArgs& a, int grid, cudaStream_t st) {
-    const dim3 g(grid), b(kGemvThreads);
-    switch (gemv_cpl(a.k)) {
-        case 1: return launch_k(k_gemv<EPI, 1, 8>, g, b, 0, st, a);
-        case 2: return launch_k(k_gemv<EPI, 2, 4>, g, b, 0, st, a);
-        case 3: return launch_k(k_gemv<EPI, 3, 2>, g, b, 0, st, a);
-        case 4: return launch_k(k_gemv<EPI, 4, 2>, g, b, 0, st, a);
-        default: return launch_k(k_gemv<EPI, 8, 1>, g, b, 0, st, a);
+static cudaError_t launch_gemv_epi(const GemvArgs* a, int n, cudaStream_t st) {
+    for (int cpl : {1, 2, 3, 4, 8}) {
+        GemvArgs sel[VT_MAX_DEVICES];
+        int m = 0;
+        for (int s = 0; s < n; ++s)
+            if (a[s].rows > 0 && gemv_cpl(a[s].k) == cpl) sel[m++] = a[s];
+        if (m == 0) continue;
+        const cudaError_t e = m == 1 ? launch_gemv_group<EPI, 1>(sel, m, cpl, st) : launch_gemv_group<EPI, VT_MAX_DEVICES>(sel, m, cpl, st);
+        if (e != cudaSuccess) return e;
     }
+    return cudaSuccess;
 }
 
-cudaError_t launch_gemv(int epi, const GemvArgs& a, cudaStream_t st) {
-    const int unit = epi == kEpiPlain ? 1 : 2;
-    const int grid = gemv_grid(a.rows, unit);
-    if (grid == 0) return cudaSuccess;
-    switch (epi) {
-        case kEpiPlain: return launch_gemv_epi<kEpiPlain>(a, grid, st);
-        case kEpiQkvRope: return launch_gemv_epi<kEpiQkvRope>(a, grid, st);
-        default: return launch_gemv_epi<kEpiSwiglu>(a, grid, st);
-    }
+cudaError_t launch_gemv(int epi, const GemvArgs* a, int n, cudaStream_t st) {
+    if (epi == kEpiPlain) return launch_gemv_epi<kEpiPlain>(a, n, st);
+    if (epi == kEpiQkvRope) return launch_gemv_epi<kEpiQkvRope>(a, n, st);
+    return cudaErrorInvalidValue;
 }
 
 // ============================================================== split-K flash decoding
@@ -518,9 +561,9 @@ cudaError_t launch_gemv(int epi, const GemvArgs& a, cudaStream_t st) {
 // per-warp states + gather buffers of the cluster merge (csize <= kAttnMaxCluster slices of the
 // CTA's feature range, plus their max and sum per head)
 static __host__ __device__ __forceinline__ size_t attn_state_floats(int dh, int group) {
-    const int fpr = (group * dh + 7) / 8;  // features per CTA for the smallest cluster (8)
-    return (size_t)2 * kAttnWarps * group + (size_t)kAttnWarps * group * dh +
-           (size_t)kAttnMaxCluster * (2 * group + fpr);
+    // (a cluster's slices of a CTA's features: csize * ceil(group dh / csize) <= group dh + kAttnMaxCluster)
+    return (size_t)2 * kAttnWarps * group + (size_t)kAttnWarps * group * dh + (size_t)kAttnMaxCluster * (2 * group + 1) +
+           (size_t)group * dh;
 }
 
 size_t attn_decode_smem_bytes(int dh, int group, int stages) {
@@ -531,15 +574,32 @@ size_t attn_decode_smem_bytes(int dh, int group, int stages) {
 
 int g_attn_cluster = 16;  // set at init: 16 when a 16-CTA cluster can be scheduled, else 8
 
-int attn_cluster_size(int hk) {
-    (void)hk;
-    return g_attn_cluster;
+// CTAs per KV head, from the KV heads and shards of the launch and the positions a head may attend to
+// (capacity or window).  More CTAs shorten the slices; but a launch with more CTAs than SMs pays for a
+// second start per SM, and a larger cluster for a longer merge.  So 16 while that is one CTA an SM or
+// less, else 8; at short spans one size less.  A token through one fp16 shard, us a layer:
+//   KV heads \ span     57: 16 / 8 / 4     300: 16 / 8 / 4     1024: 16 / 8 / 4    3000: 16 / 8 / 4
+//    4 (GQA 4)       14.3 / 13.7 / 13.7  15.0 / 15.3 / 17.1  17.4 / 17.8 / 22.9  20.4 / 27.5 / 42.6
+//   12               25.1 / 24.3 / 23.7  25.2 / 24.6 / 23.6  26.1 / 24.9 / 27.8  28.8 / 32.7 / 37.0
+//   16               27.9 / 23.2 / 23.7  28.4 / 23.5 / 25.1  30.6 / 25.8 / 29.4  33.0 / 31.4 / 40.9
+//   32               47.7 / 43.8 / 38.8  48.4 / 44.4 / 40.4  51.1 / 47.3 / 44.6  59.3 / 55.1 / 57.3
+// 32 heads of four shards in one launch: 92.9 / 86.1 / 85.5, 93.3 / 86.3 / 89.2, 99.6 / 92.9 / 94.8,
+// 107.0 / 105.3 / 107.8 (8-bit weights): 4 is for one shard only.  40 heads want 8 at every span (4 is
+// above one CTA an SM too).  `fixed`: 16 whatever the launch, so that a shard's sums do not depend on
+// what runs beside it.
+int attn_cluster_size(int hk, int shards, int span, bool fixed) {
+    const int sms = g_num_sms > 0 ? g_num_sms : 148;
+    if (fixed) return g_attn_cluster;
+    if (hk * 16 <= sms) return span <= 256 ? 8 : g_attn_cluster;
+    if (hk * 8 <= sms) return hk * 12 <= sms && span > 2048 ? g_attn_cluster : 8;
+    const int short_span = hk * 16 > 3 * sms ? 1536 : 256;  // 8 CTAs a head are more than 1.5 an SM
+    return shards == 1 && hk * 4 <= sms && span <= short_span ? 4 : 8;
 }
 
-int attn_stages(int cap, int csize) {
-    const int per = (cap + csize - 1) / csize;
+int attn_stages(int span, int csize) {
+    const int per = (span + csize - 1) / csize;
     int t = (per + kAttnTilePos - 1) / kAttnTilePos;
-    return t < 2 ? 2 : (t > kAttnMaxStages ? kAttnMaxStages : t);
+    return t < 1 ? 1 : (t > kAttnMaxStages ? kAttnMaxStages : t);
 }
 
 template <int DH, int G>
@@ -552,18 +612,19 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn_decode(const __grid_const
     float* wm = reinterpret_cast<float*>(smem + (size_t)S * 2 * TILE_BYTES);  // [warps][G]
     float* wl = wm + kAttnWarps * G;                                           // [warps][G]
     float* wo = wl + kAttnWarps * G;                                           // [warps][G][DH]
-    constexpr int FMAX = (G * DH + 7) / 8;                                     // features per CTA (csize >= 8)
     float* gm = wo + kAttnWarps * G * DH;                                      // [kAttnMaxCluster][G]
     float* gl = gm + kAttnMaxCluster * G;                                      // [kAttnMaxCluster][G]
-    float* go = gl + kAttnMaxCluster * G;                                      // [kAttnMaxCluster][FMAX]
+    float* go = gl + kAttnMaxCluster * G;                                      // [csize][features per CTA]
     const size_t st_bytes = (attn_state_floats(DH, G) * 4 + 15) & ~(size_t)15;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * 2 * TILE_BYTES + st_bytes);
     uint64_t* empty = full + S;
     __shared__ int s_abort;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = (int)cluster_rank(), csize = (int)cluster_size();  // csize is 8 or 16
-    const int j = blockIdx.y;
+    const int rank = (int)cluster_rank(), csize = (int)cluster_size();  // csize: 16, 8 or 4
+    int sh = 0;  // the shard of this cluster's KV head, and the head's number within it
+    while (sh + 1 < a.n && (int)blockIdx.y >= a.hk_end[sh]) ++sh;
+    const int j = (int)blockIdx.y - (sh > 0 ? a.hk_end[sh - 1] : 0);
     // The length was written by a kernel that completed before this one started (see device.cuh).
     const int len = *a.len;
     const bool ok = len >= 0 && len < a.cap;
@@ -577,8 +638,10 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn_decode(const __grid_const
     const int old_end = pnew >= 0 ? min(t1, pnew) : t1;
     const int n_old = max(old_end - t0, 0);
     const int ntiles = (n_old + kAttnTilePos - 1) / kAttnTilePos;
-    const __half* kbase = a.kcache + (int64_t)j * a.cap * DH;
-    const __half* vbase = a.vcache + (int64_t)j * a.cap * DH;
+    const __half* kbase = a.kcache[sh] + (int64_t)j * a.cap * DH;
+    const __half* vbase = a.vcache[sh] + (int64_t)j * a.cap * DH;
+    const float* qbase = a.q[sh] + (int64_t)j * G * DH;
+    float* obase = a.out[sh] + (int64_t)j * G * DH;
 
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
@@ -628,7 +691,7 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn_decode(const __grid_const
 #pragma unroll
         for (int h = 0; h < G; ++h)
 #pragma unroll
-            for (int e = 0; e < EPL; ++e) q[h][e] = __ldcg(a.q + (j * G + h) * DH + lane * EPL + e);
+            for (int e = 0; e < EPL; ++e) q[h][e] = __ldcg(qbase + h * DH + lane * EPL + e);
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
             kn[e] = has_new ? __half2float(__ldcg(kbase + (int64_t)pnew * DH + lane * EPL + e)) : 0.f;
@@ -782,7 +845,7 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn_decode(const __grid_const
                 }
             }
             const int owner = idx / fpr;
-            dsmem_st(dsmem_addr(&go[rank * FMAX + (idx - owner * fpr)], owner), O);
+            dsmem_st(dsmem_addr(&go[rank * fpr + (idx - owner * fpr)], owner), O);
             if (d < csize) {
                 dsmem_st(dsmem_addr(&gm[rank * G + h], d), M);
                 dsmem_st(dsmem_addr(&gl[rank * G + h], d), L);
@@ -805,19 +868,19 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn_decode(const __grid_const
                     const float mc = gm[c * G + h];
                     const float w = mc == -INFINITY ? 0.f : exp2f(mc - M);
                     L += gl[c * G + h] * w;
-                    O += go[c * FMAX + (f - f0)] * w;
+                    O += go[c * fpr + (f - f0)] * w;
                 }
             }
-            a.out[(j * G + h) * DH + d] = L > 0.f ? O / L : 0.f;
+            obase[h * DH + d] = L > 0.f ? O / L : 0.f;
         }
     }
 }
 
 template <int DH, int G>
 static cudaError_t launch_attn_dhg(const AttnDecodeArgs& a, cudaStream_t st) {
-    const int cs = attn_cluster_size(a.hk);
+    const int hk = a.hk_end[a.n - 1], cs = a.cluster;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs, a.hk);
+    cfg.gridDim = dim3(cs, hk);
     cfg.blockDim = dim3(kAttnThreads);
     cfg.dynamicSmemBytes = attn_decode_smem_bytes(DH, G, a.stages);
     cfg.stream = st;
@@ -845,7 +908,7 @@ static cudaError_t launch_attn_dh(const AttnDecodeArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_attn_decode(const AttnDecodeArgs& a, cudaStream_t st) {
-    if (a.hk <= 0) return cudaSuccess;
+    if (a.n <= 0 || a.hk_end[a.n - 1] <= 0) return cudaSuccess;
     if (a.dh == 128) return launch_attn_dh<128>(a, st);
     if (a.dh == 64) return launch_attn_dh<64>(a, st);
     return cudaErrorInvalidValue;
@@ -1079,30 +1142,29 @@ static cudaError_t allow_smem(K kern, size_t want, bool max_carveout = false) {
 
 cudaError_t init_decode_kernels() {
     cudaError_t e;
-#define VT_GEMV_ATTR(EPI)                                                         \
-    if ((e = allow_smem(k_gemv<EPI, 1, 8>, 0)) != cudaSuccess) return e;          \
-    if ((e = allow_smem(k_gemv<EPI, 2, 4>, 0)) != cudaSuccess) return e;          \
-    if ((e = allow_smem(k_gemv<EPI, 3, 2>, 0)) != cudaSuccess) return e;          \
-    if ((e = allow_smem(k_gemv<EPI, 4, 2>, 0)) != cudaSuccess) return e;          \
-    if ((e = allow_smem(k_gemv<EPI, 8, 1>, 0)) != cudaSuccess) return e;
-    VT_GEMV_ATTR(kEpiPlain) VT_GEMV_ATTR(kEpiSwiglu)
+#define VT_GEMV_ATTR(EPI, NG, CARVE)                                                       \
+    if ((e = allow_smem(k_gemv<EPI, 1, 8, NG>, 0, CARVE)) != cudaSuccess) return e;          \
+    if ((e = allow_smem(k_gemv<EPI, 2, 4, NG>, 0, CARVE)) != cudaSuccess) return e;          \
+    if ((e = allow_smem(k_gemv<EPI, 3, 2, NG>, 0, CARVE)) != cudaSuccess) return e;          \
+    if ((e = allow_smem(k_gemv<EPI, 4, 2, NG>, 0, CARVE)) != cudaSuccess) return e;          \
+    if ((e = allow_smem(k_gemv<EPI, 8, 1, NG>, 0, CARVE)) != cudaSuccess) return e;
+    VT_GEMV_ATTR(kEpiPlain, 1, false) VT_GEMV_ATTR(kEpiPlain, VT_MAX_DEVICES, false)
+    VT_GEMV_ATTR(kEpiQkvRope, 1, true) VT_GEMV_ATTR(kEpiQkvRope, VT_MAX_DEVICES, true)
 #undef VT_GEMV_ATTR
-    if ((e = allow_smem(k_gemv<kEpiQkvRope, 1, 8>, 0, true)) != cudaSuccess) return e;
-    if ((e = allow_smem(k_gemv<kEpiQkvRope, 2, 4>, 0, true)) != cudaSuccess) return e;
-    if ((e = allow_smem(k_gemv<kEpiQkvRope, 3, 2>, 0, true)) != cudaSuccess) return e;
-    if ((e = allow_smem(k_gemv<kEpiQkvRope, 4, 2>, 0, true)) != cudaSuccess) return e;
-    if ((e = allow_smem(k_gemv<kEpiQkvRope, 8, 1>, 0, true)) != cudaSuccess) return e;
     if ((e = allow_smem(k_combine<1>, 0)) != cudaSuccess) return e;
     if ((e = allow_smem(k_combine<4>, 0)) != cudaSuccess) return e;
     if ((e = allow_smem(k_fill_zero_f32, 0)) != cudaSuccess) return e;
     if ((e = allow_smem(k_kv_advance, 0)) != cudaSuccess) return e;
-#define VT_FFN_ATTR(CPL, R)                                                                       \
-    if ((e = allow_smem(k_ffn<CPL, R, 1>, 1 * kGemvThreads * 32)) != cudaSuccess) return e;       \
-    if ((e = allow_smem(k_ffn<CPL, R, 2>, 2 * kGemvThreads * 32)) != cudaSuccess) return e;       \
-    if ((e = allow_smem(k_ffn<CPL, R, 3>, 3 * kGemvThreads * 32)) != cudaSuccess) return e;       \
-    if ((e = allow_smem(k_ffn<CPL, R, 4>, 4 * kGemvThreads * 32)) != cudaSuccess) return e;       \
-    if ((e = allow_smem(k_ffn<CPL, R, 8>, 8 * kGemvThreads * 32)) != cudaSuccess) return e;
-    VT_FFN_ATTR(1, 8) VT_FFN_ATTR(2, 4) VT_FFN_ATTR(3, 2) VT_FFN_ATTR(4, 2) VT_FFN_ATTR(8, 1)
+#define VT_FFN_ATTR(CPL, R, NG)                                                                   \
+    if ((e = allow_smem(k_ffn<CPL, R, 1, NG>, 1 * kGemvThreads * 32)) != cudaSuccess) return e;   \
+    if ((e = allow_smem(k_ffn<CPL, R, 2, NG>, 2 * kGemvThreads * 32)) != cudaSuccess) return e;   \
+    if ((e = allow_smem(k_ffn<CPL, R, 3, NG>, 3 * kGemvThreads * 32)) != cudaSuccess) return e;   \
+    if ((e = allow_smem(k_ffn<CPL, R, 4, NG>, 4 * kGemvThreads * 32)) != cudaSuccess) return e;   \
+    if ((e = allow_smem(k_ffn<CPL, R, 8, NG>, 8 * kGemvThreads * 32)) != cudaSuccess) return e;
+#define VT_FFN_NG(NG) \
+    VT_FFN_ATTR(1, 8, NG) VT_FFN_ATTR(2, 4, NG) VT_FFN_ATTR(3, 2, NG) VT_FFN_ATTR(4, 2, NG) VT_FFN_ATTR(8, 1, NG)
+    VT_FFN_NG(1) VT_FFN_NG(VT_MAX_DEVICES)
+#undef VT_FFN_NG
 #undef VT_FFN_ATTR
 #define VT_ATTN_ATTR(DH, G)                                                                       \
     if ((e = allow_smem(k_attn_decode<DH, G>, attn_decode_smem_bytes(DH, G, kAttnMaxStages), true)) != \

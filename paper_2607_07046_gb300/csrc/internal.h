@@ -34,7 +34,17 @@ constexpr int kAttnMaxGroup = 8;  // query heads per KV head supported by the de
 enum GemvEpilogue : int {
     kEpiPlain = 0,   // out[r] = y[r] (fp32)
     kEpiQkvRope = 1, // rows in RoPE-pair order: rotate q/k, append k/v to the cache
-    kEpiSwiglu = 2,  // rows (gate, up) interleaved: u[j] = silu(gate) * up
+    kEpiSwiglu = 2,  // rows (gate, up) interleaved: u[j] = silu(gate) * up (quantized shards)
+};
+
+// Decode kernels take one shard, or every shard of a block in one launch (the whole-token path of
+// partitions that the fused kernel does not take): the CTAs are dealt out to the shards, shard g
+// owning those from end[g - 1] to end[g] - 1 of the (first or second) grid dimension.
+template <class Args, int NG>
+struct DecodeGroup {
+    int n;
+    int end[NG];
+    Args a[NG];
 };
 
 struct GemvArgs {
@@ -66,20 +76,22 @@ struct GemvArgs {
     int indep;
 };
 
-struct AttnDecodeArgs {
-    const float* q;        // [h_s][dh] rotated queries
-    const __half* kcache;  // [hk_s][cap][dh]
-    const __half* vcache;
+struct AttnDecodeArgs {  // one layer, every shard of the launch
     const int32_t* len;
     int cap;
-    int hk;                // KV heads of the shard
     int group;             // query heads per KV head
     int dh;
+    int cluster;           // CTAs per KV head (attn_cluster_size)
     int stages;            // K/V tiles in flight per CTA (attn_stages)
     float scale_log2;      // log2(e) / sqrt(dh)
     int window;            // > 0: attend to the last `window` positions only (sliding window)
-    float* out;            // [h_s][dh] attention output of the shard's query heads
     uint32_t* status;
+    int n;                                // shards
+    int hk_end[VT_MAX_DEVICES];           // KV heads up to and including shard s
+    const float* q[VT_MAX_DEVICES];       // [h_s][dh] rotated queries
+    const __half* kcache[VT_MAX_DEVICES]; // [hk_s][cap][dh]
+    const __half* vcache[VT_MAX_DEVICES];
+    float* out[VT_MAX_DEVICES];           // [h_s][dh] attention output of the shard's query heads
 };
 
 struct CombineArgs {
@@ -109,16 +121,15 @@ extern bool g_use_pdl;  // programmatic dependent launch between the library's k
 extern int g_grid_mult; // CTAs per SM of the streaming kernels
 extern int g_num_sms;
 
-cudaError_t launch_gemv(int epi, const GemvArgs& a, cudaStream_t st);
-int gemv_grid(int rows, int unit);
-int gemv_cpl(int k);
+// n shards of one block (same epilogue) in one launch
+cudaError_t launch_gemv(int epi, const GemvArgs* a, int n, cudaStream_t st);
 cudaError_t launch_attn_decode(const AttnDecodeArgs& a, cudaStream_t st);
 size_t attn_decode_smem_bytes(int dh, int group, int stages);
-int attn_cluster_size(int hk);
-int attn_stages(int cap, int csize);
+// hk: KV heads of the launch; span: positions that a head attends to at most (capacity or window)
+int attn_cluster_size(int hk, int shards, int span, bool fixed);
+int attn_stages(int span, int csize);
 cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st);
-int ffn_grid(int cols);
-cudaError_t launch_ffn_decode(const FfnDecodeArgs& a, int grid, cudaStream_t st);
+cudaError_t launch_ffn_decode(const FfnDecodeArgs* a, int n, cudaStream_t st);
 cudaError_t launch_transpose_f16(const __half* src, int64_t src_ld, int rows, int cols, __half* dst,
                                  int64_t dst_ld, cudaStream_t st);
 cudaError_t launch_fill_zero_f32(float* p, int64_t n, cudaStream_t st);
@@ -197,18 +208,20 @@ cudaError_t launch_rmsnorm_rows(const __half* x, const __half* gain, float eps, 
 // ------------------------------------------------------------------ block-quantized shard weights (quant.cu)
 // A matrix [rows][k] stored as codes of 8 or 4 bits with one fp16 scale per block of kQBlock
 // weights along k (the dequantized weight is q * d).  Device layout (written by k_quantize_rows):
-//   codes: row r at codes + r * row_bytes, row_bytes = nb * 32 (8-bit) or nb * 16 (4-bit),
-//          nb = ceil(k / 32); biased codes u = q + 128 (8-bit, one byte each) or u = q + 8 (4-bit:
-//          each 32-bit word holds 8 codes, byte i = code i in its low nibble and code i + 4 in its
-//          high nibble); positions k .. nb * 32 - 1 hold the code of 0;
-//   scales: [rows][nb] fp16.
+//   rows in tiles of kQTile (the last one padded with zero rows), nb = ceil(k / 32) blocks each;
+//   codes: biased, u = q + 128 (8-bit, one byte each) or u = q + 8 (4-bit: each 32-bit word holds 8
+//          codes, byte i = code i in its low nibble and code i + 4 in its high nibble).  Per row tile
+//          and block, 32 lanes (g, t), lane 4 g + t holding positions 8t .. 8t + 7 of row g and then
+//          of row g + 8 of the tile: the A fragments of a warp's MMAs, lane by lane.  Positions
+//          k .. nb * 32 - 1 hold the code of 0;
+//   scales: fp16, per row tile and block those of rows 0, 8, 1, 9, ..., 7, 15.
 constexpr int kQBlock = 32;
+constexpr int kQTile = 16;
 
 struct QMatDev {
     uint8_t* codes = nullptr;
     __half* scales = nullptr;
     int rows = 0, k = 0, nb = 0, bits = 16;
-    int64_t row_bytes = 0;
 };
 // Quantizes device fp16 rows (row r at w + r * ld, m.k values) into m's codes and scales, in the
 // layout above, with the decisions of vt_quantize_rows (bit-identical codes and scales).
@@ -217,8 +230,8 @@ cudaError_t launch_quantize_rows(const __half* w, int64_t ld, const QMatDev& m, 
 // Host side: bytes of the codes and of the scales of a [rows][k] matrix at `bits`.
 size_t qmat_code_bytes(int64_t rows, int64_t k, int bits);
 size_t qmat_scale_bytes(int64_t rows, int64_t k);
-// The inverse of the packing for the codes: canonical int8 codes [rows][k].
-void unpack_qcodes(const uint8_t* codes, int64_t rows, int64_t k, int bits, int8_t* q);
+// The inverse of the packing: canonical int8 codes [rows][k] and scales [rows][nb].
+void unpack_qmat(const uint8_t* codes, const __half* scales, int64_t rows, int64_t k, int bits, int8_t* q, __half* out);
 // Host quantizer shared with vt_quantize_rows: codes q [rows][k] (int8) and fp16 scales [rows][nb].
 void quantize_rows_host(const __half* w, int64_t rows, int64_t k, int bits, int block, int8_t* q, __half* scales);
 
@@ -238,8 +251,9 @@ struct QGemvArgs {
     const float2* rope;
     int dh, hq, hk;
     uint32_t* status;
+    int parts;  // parts that the blocks of a row are cut into (set by the launch)
 };
-cudaError_t launch_gemv_q(int epi, const QGemvArgs& a, cudaStream_t st);
+cudaError_t launch_gemv_q(int epi, const QGemvArgs* a, int n, cudaStream_t st);
 
 // Quantized shard partials (communication scaling): x [n] fp32 -> codes (int8 per value at 8
 // bits, two 4-bit values per byte) + fp16 scales [ceil(n / 32)].

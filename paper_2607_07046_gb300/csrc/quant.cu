@@ -8,9 +8,9 @@
 // 8 bits, 7 for 4 bits) and every weight the code q = round-half-even(w / d) clamped to
 // [-qmax, qmax] (0 when d = 0), both divisions in fp32.  A projection is y = sum_e (q_e d) x_e.
 //
-// The kernel keeps the codes as integers and multiplies them on the tensor cores (integer MMA
-// against an exact three-digit int8 split of the input), so the work per code is a small fraction
-// of an instruction and the GEMV streams at the memory rate (details at the kernel).
+// The kernel keeps the codes as integers and multiplies them on the tensor cores (codes and
+// an exact three-digit split of the input as whole numbers in fp16, whose products and sums in fp32
+// are exact), so the work per code is a small fraction of an instruction (details at the kernel).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -50,135 +50,200 @@ void quantize_rows_host(const __half* w, int64_t rows, int64_t k, int bits, int 
 
 static int64_t qmat_nb(int64_t k) { return (k + kQBlock - 1) / kQBlock; }
 
+static int64_t qmat_rows(int64_t rows) { return (rows + kQTile - 1) / kQTile * kQTile; }  // whole row tiles
+
 size_t qmat_code_bytes(int64_t rows, int64_t k, int bits) {
-    return (size_t)rows * (size_t)qmat_nb(k) * (bits == 8 ? 32 : 16);
+    return (size_t)qmat_rows(rows) * (size_t)qmat_nb(k) * (bits == 8 ? 32 : 16);
 }
 
-size_t qmat_scale_bytes(int64_t rows, int64_t k) { return (size_t)rows * (size_t)qmat_nb(k) * 2; }
+size_t qmat_scale_bytes(int64_t rows, int64_t k) { return (size_t)qmat_rows(rows) * (size_t)qmat_nb(k) * 2; }
 
-void unpack_qcodes(const uint8_t* codes, int64_t rows, int64_t k, int bits, int8_t* q) {
+// Byte offset of the codes of row r, block b, positions 8t .. 8t + 7, and index of the row's scale
+// (the layout of QMatDev).
+static __host__ __device__ __forceinline__ size_t qcode_at(int64_t r, int64_t b, int t, int64_t nb, int bits) {
+    const int64_t tile = r / kQTile, g = r % 8, high = r / 8 % 2;
+    return (size_t)(((tile * nb + b) * 32 + 4 * g + t) * 2 + high) * (bits == 8 ? 8 : 4);
+}
+static __host__ __device__ __forceinline__ size_t qscale_at(int64_t r, int64_t b, int64_t nb) {
+    return (size_t)((r / kQTile * nb + b) * kQTile + r % 8 * 2 + r / 8 % 2);
+}
+
+void unpack_qmat(const uint8_t* codes, const __half* scales, int64_t rows, int64_t k, int bits, int8_t* q, __half* out) {
     const int64_t nb = qmat_nb(k);
-    const int64_t rb = nb * (bits == 8 ? 32 : 16);
     for (int64_t r = 0; r < rows; ++r) {
-        const uint8_t* row = codes + r * rb;
+        for (int64_t b = 0; b < nb; ++b) out[r * nb + b] = scales[qscale_at(r, b, nb)];
         for (int64_t e = 0; e < k; ++e) {
-            int u;
-            if (bits == 8) {
-                u = row[e] - 128;
-            } else {
-                const int64_t g = e / 8, i = e % 8;
-                const uint8_t byte = row[g * 4 + (i & 3)];
-                u = (i < 4 ? (byte & 15) : (byte >> 4)) - 8;
-            }
-            q[r * k + e] = (int8_t)u;
+            const uint8_t* at = codes + qcode_at(r, e / 32, (int)(e % 32 / 8), nb, bits);
+            const int i = (int)(e % 8);
+            q[r * k + e] = (int8_t)(bits == 8 ? at[i] - 128 : (i < 4 ? at[i] & 15 : at[i - 4] >> 4) - 8);
         }
     }
 }
 
 // ================================================================== device: dequantizing GEMV
 //
-// Integer tensor-core GEMV.  Decode at batch 1 is bound by HBM only if the work per weight code
-// stays far below one instruction; rebuilding codes as floats costs more than that.  So the codes
-// stay integers and go to `mma.sync m16n8k32` (u8 codes x s8 input, s32 accumulate), one MMA per
-// block of 32 weights of 16 rows:
-//   - the input x^ (fp32) of block b is split into three int8 digits at scales s, s / 254 and
-//     s / 254^2 (s = max|x^| / 127 over the block), which reproduce it to 2^-24 of the block's
-//     largest value; the digits are the MMA's B columns 0, 1, 2, so one MMA gives all three
-//     integer dot products of each row with the block;
-//   - the code bias leaves in integers: sum (u - bias) q = D - bias * Q, Q = sum q over the block;
-//   - a row's block term is s * (D1 - bias Q1) + s / 254 * (D2 - ...) + ..., times the block's
-//     fp16 weight scale, accumulated in fp32.
-// Within a block the k order is permuted the same way for A and B: lane (g, t) of the MMA loads
-// the 8 codes of rows g and g + 8 at positions 8t .. 8t + 7 (one 8-byte load per row at 8 bits;
-// one 4-byte word at 4 bits, whose nibbles unpack to the same positions), which become its
-// fragment's k = 4t .. 4t + 3 and 16 + 4t .. 16 + 4t + 3; the B fragment of lane (n, t) is loaded
-// from the same positions of digit n, stored in the block's natural order.
-// Work split: a CTA takes 64 rows (four MMA row tiles) and one part of the blocks, and computes the
-// input digits of its part only; warp w takes row tile w % 4 and half w / 4 of the part.  The
-// parts of a row tile form a thread-block cluster: after a cluster barrier rank 0 adds the
-// parts' row sums in rank order (distributed shared memory) and runs the epilogue, and a second
-// cluster barrier keeps the other ranks until it has read them.  No global scratch, no flags.
+// Tensor-core GEMV on exact integers.  Decode at batch 1 is bound by HBM only if the work per weight
+// code stays far below one instruction; rebuilding weights as floats costs more than that.  So the
+// codes go to `mma.sync m16n8k16` as fp16 integers, two MMAs per block of 32 weights of 16 rows:
+//   - a biased code u (0 .. 255, or 0 .. 15) becomes the fp16 number 1024 + u by putting its bits
+//     under the exponent of 1024: one byte permute, or a shift and an and-or, for two codes;
+//   - the input x^ (fp32) of block b is split into three integer digits of at most 127 at scales s,
+//     s / 254 and s / 254^2 (s = max|x^| / 127 over the block), which reproduce it to 2^-24 of the
+//     block's largest value; the digits are the MMA's B columns 0, 1, 2, so one accumulation gives
+//     all three dot products of each row with the block;
+//   - every product and partial sum is an integer below 2^23, so the fp32 accumulation is exact; the
+//     accumulator starts at -(1024 + bias) times the digit's sum, which takes the offsets out;
+//   - a row's block term is s * D1 + s / 254 * D2 + s / 254^2 * D3, times the block's fp16 weight
+//     scale, accumulated in fp32.
+// Codes and scales are stored in the order in which a warp takes them: per row tile and block, lane
+// (g, t) finds the positions 8t .. 8t + 7 of rows g and g + 8 side by side (one 16-byte load, or 8
+// bytes at 4 bits), and rows g and g + 8's scales in one word, so a warp streams whole lines.  The
+// k order within a block is the codes' order in the fragments, the same for the digits.
+// What bounds it is the instructions around the MMAs and the start of a CTA (norm, digits), not the
+// bytes: a warp takes 32 rows where there are enough (two row tiles share the input's fragments), a
+// batch of two blocks runs without branches (past the end the last block again, with zero scales), and the input's
+// divisions are done for four blocks at once, one lane each.  Llama-2-7B gate/up, four 8-bit shards
+// in one launch (92 MB): 32.0 us, against 49 with rows stored one after another, 16 rows a warp and
+// the integer MMA m16n8k32 (which takes the codes as they are, but is slow on this GPU).
+// Work split: the blocks of a shard's rows are cut into `parts` (gemv_q_parts of the shard alone);
+// a CTA takes 128 rows (64 in launches of few rows) and one or more consecutive parts, and computes
+// the input digits of its parts only; a warp takes a quarter of the rows and
+// one half of each part.  The CTAs of a row tile form a thread-block cluster: after a cluster barrier rank 0 adds the parts' row sums in part
+// order (distributed shared memory) and runs the epilogue, and a second cluster barrier keeps the
+// other ranks until it has read them.  No global scratch, no flags.
+// How many parts a CTA takes depends on the launch (a single shard: one; a whole block's shards:
+// enough for 2.5 CTAs an SM), the sums of a shard and their order do not, so a shard's results have
+// the same bits alone and in a group.
 // The first codes are loaded before griddepcontrol.wait: weights do not depend on the preceding
 // kernel.
 constexpr int kQWarps = 8;
 constexpr int kQThreads = kQWarps * 32;
-constexpr int kQRows = 64;  // rows per CTA
-constexpr int kQUnroll = 4; // blocks in flight per warp and buffer
+constexpr int kQUnroll = 2;  // blocks in flight per warp and buffer
 constexpr int kQMaxParts = 8;
 
-__device__ __forceinline__ void mma_u8s8(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+__device__ __forceinline__ void mma_f16f32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                           uint32_t b1, float c0, float c1, float c2, float c3) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+}
+// The eight codes of a row's position group as fp16 pairs 1024 + u: at 8 bits (two words) positions
+// (0, 1), (2, 3), (4, 5), (6, 7); at 4 bits (one word) (0, 2), (1, 3), (4, 6), (5, 7).
+template <int BITS>
+__device__ __forceinline__ void codes_f16(uint32_t w0, uint32_t w1, uint32_t (&h)[4]) {
+    if constexpr (BITS == 8) {
+        h[0] = __byte_perm(w0, 0x64646464u, 0x4140);
+        h[1] = __byte_perm(w0, 0x64646464u, 0x4342);
+        h[2] = __byte_perm(w1, 0x64646464u, 0x4140);
+        h[3] = __byte_perm(w1, 0x64646464u, 0x4342);
+    } else {
+        h[0] = (w0 & 0x000F000Fu) | 0x64006400u;
+        h[1] = ((w0 >> 8) & 0x000F000Fu) | 0x64006400u;
+        h[2] = ((w0 >> 4) & 0x000F000Fu) | 0x64006400u;
+        h[3] = ((w0 >> 12) & 0x000F000Fu) | 0x64006400u;
+    }
 }
 
-// Blocks of part `part` of `parts` over nb blocks.
-__device__ __forceinline__ void part_blocks(int nb, int part, int parts, int& b0, int& b1) {
-    b0 = (int)(((int64_t)part * nb) / parts);
-    b1 = (int)(((int64_t)(part + 1) * nb) / parts);
-}
-// shared-memory bytes of a CTA whose part has at most `pb` blocks: per block 3 x 32 digits, then
-// 16 bytes of scales (s1, s2, s3) and 16 of bias-scaled digit sums
-static size_t gemv_q_smem(int pb) { return (size_t)pb * (96 + 16 + 16) + 16; }
+// First block of part `part` of `parts` over nb blocks (nb at most 512).
+__host__ __device__ __forceinline__ int part_start(int nb, int part, int parts) { return part * nb / parts; }
+// shared-memory bytes of a CTA whose parts have at most `pb` blocks: per block 3 x 32 fp16 digits, 16
+// bytes of scales (s1, s2, s3) and 32 bytes of accumulator starts
+static size_t gemv_q_smem(int pb) { return (size_t)pb * (192 + 16 + 32) + 16; }
 
-template <int EPI, int BITS>
-__global__ void __launch_bounds__(kQThreads) k_gemv_q(const __grid_constant__ QGemvArgs a) {
-    constexpr int BIAS = BITS == 8 ? 128 : 8;
+// One CTA of 64 MT rows, four row groups of MT row tiles by two halves.  tile_row: the CTA's first row.
+template <int EPI, int BITS, int MT>
+__device__ __forceinline__ void gemv_q_cta(const QGemvArgs& a, int tile_row) {
+    constexpr int kQRows = 64 * MT, kRowsW = 16 * MT;  // rows of the CTA, of a warp
+    constexpr int OFFSET = 1024 + (BITS == 8 ? 128 : 8);  // of a code's fp16 number
     extern __shared__ __align__(16) uint8_t qsm[];
     __shared__ float red[kQWarps + 1];
-    __shared__ float rsum[kQWarps][16];
-    __shared__ float rows_sum[kQRows];
+    __shared__ float rsum[kQMaxParts][kQWarps][kRowsW];
+    __shared__ float rows_sum[kQMaxParts][kQRows];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const QMatDev& W = a.w;
     const int nb = W.nb;
-    const int parts = (int)gridDim.x, part = (int)blockIdx.x;  // cluster (parts, 1, 1): rank = part
-    int pb0, pb1;
-    part_blocks(nb, part, parts, pb0, pb1);
-    const int npb = pb1 - pb0;
-    int8_t* xq = reinterpret_cast<int8_t*>(qsm);                           // [npb][3][32]
-    float4* xsc = reinterpret_cast<float4*>(qsm + (size_t)npb * 96);       // [npb] (s1, s2, s3, -)
-    int4* xsum = reinterpret_cast<int4*>(xsc + npb);                       // [npb] bias * digit sums
+    // cluster (gridDim.x, 1, 1): this CTA has parts [p0, p1) of the shard, blocks [pb0, pb1)
+    const int ranks = (int)gridDim.x, rank = (int)blockIdx.x, parts = a.parts;
+    const int p0 = rank * parts / ranks, p1 = (rank + 1) * parts / ranks;
+    const int pb0 = part_start(nb, p0, parts), npb = part_start(nb, p1, parts) - pb0;
+    __half* xq = reinterpret_cast<__half*>(qsm);                       // [npb][3][32]
+    float4* xsc = reinterpret_cast<float4*>(qsm + (size_t)npb * 192);  // [npb] (s1, s2, s3, -)
+    float* xst = reinterpret_cast<float*>(xsc + npb);                  // [npb][8] accumulator start of each column
     const int tile = warp & 3, half = warp >> 2;
-    const int row0 = (int)blockIdx.y * kQRows + tile * 16;
-    const int ra = row0 + g, rb = row0 + g + 8;
-    const bool oka = ra < W.rows, okb = rb < W.rows;
-    // this warp's blocks: half `half` of the part
-    const int wb0 = pb0 + (half == 0 ? 0 : npb / 2), wb1 = half == 0 ? pb0 + npb / 2 : pb1;
-    const uint8_t* ca = W.codes + (int64_t)(oka ? ra : 0) * W.row_bytes;
-    const uint8_t* cb = W.codes + (int64_t)(okb ? rb : 0) * W.row_bytes;
-    const __half* sa = W.scales + (int64_t)(oka ? ra : 0) * nb;
-    const __half* sb = W.scales + (int64_t)(okb ? rb : 0) * nb;
-
-    // codes of rows g, g + 8 (8 bytes each at 8 bits, a word at 4) and, in lane t = 0, the rows'
-    // weight scales, for kQUnroll blocks from block bb
-    auto load = [&](uint2 (&va)[kQUnroll], uint2 (&vb)[kQUnroll], __half2 (&dv)[kQUnroll], int bb) {
-#pragma unroll
-        for (int u = 0; u < kQUnroll; ++u) {
-            const int b = bb + u;
-            const bool on = b < wb1;
-            if constexpr (BITS == 8) {
-                va[u] = on && oka ? ldg_stream_u2(ca + (int64_t)b * 32 + 8 * t) : make_uint2(0u, 0u);
-                vb[u] = on && okb ? ldg_stream_u2(cb + (int64_t)b * 32 + 8 * t) : make_uint2(0u, 0u);
-            } else {
-                va[u].x = on && oka ? ldg_stream_u1(ca + (int64_t)b * 16 + 4 * t) : 0u;
-                vb[u].x = on && okb ? ldg_stream_u1(cb + (int64_t)b * 16 + 4 * t) : 0u;
-                va[u].y = vb[u].y = 0u;
-            }
-            const __half z = __float2half(0.f);
-            dv[u] = __halves2half2(on && oka && t == 0 ? sa[b] : z, on && okb && t == 0 ? sb[b] : z);
+    __shared__ int2 span[kQMaxParts + 1][2];  // [part - p0][half]: its blocks
+    if (tid < 2 * (p1 - p0)) {
+        const int p = p0 + (tid >> 1), s0 = part_start(nb, p, parts), s1 = part_start(nb, p + 1, parts), mid = s0 + (s1 - s0) / 2;
+        span[tid >> 1][tid & 1] = (tid & 1) == 0 ? make_int2(s0, mid) : make_int2(mid, s1);
+    }
+    __syncthreads();
+    // Batches of kQUnroll of this warp's blocks: its half of the CTA's first part, then of the next, ...
+    const int np = p1 - p0;
+    struct Cursor {
+        int p, b, end;
+    };
+    auto enter = [&](Cursor& c) {  // the first block of this warp's half of part c.p, skipping empty halves
+        for (; c.p < np; ++c.p) {
+            const int2 s = span[c.p][half];
+            c.b = s.x;
+            c.end = s.y;
+            if (c.b < c.end) return;
+        }
+        c.b = pb0;  // past the last part: loads repeat the CTA's first blocks, nothing is consumed
+        c.end = pb0 + 1;
+    };
+    auto next = [&](Cursor& c) {
+        c.b += kQUnroll;
+        if (c.b >= c.end) {
+            ++c.p;
+            enter(c);
         }
     };
-    uint2 pa[2][kQUnroll], pb[2][kQUnroll];
-    __half2 pd[2][kQUnroll];
-    load(pa[0], pb[0], pd[0], wb0);
-    load(pa[1], pb[1], pd[1], wb0 + kQUnroll);
+    // this warp's row tiles (past the last one: that one again, its rows are not written)
+    const int tiles = (W.rows + kQTile - 1) / kQTile, tile0 = tile_row / kQTile + MT * tile;
+    constexpr uint32_t kCode = BITS == 8 ? 512 : 256;  // bytes of a row tile's block
+    const uint8_t* const codes = W.codes + lane * (kCode / 32);
+    const __half* const scales = W.scales + 2 * g;
+    uint32_t first[MT];  // block 0 of the row tile (32-bit indices: a matrix has at most 2^28 codes)
+#pragma unroll
+    for (int m = 0; m < MT; ++m) first[m] = (uint32_t)min(tile0 + m, tiles - 1) * (uint32_t)nb;
+    struct Batch {
+        uint4 q[kQUnroll][MT];     // codes of rows g, g + 8 of row tile m
+        uint32_t d[kQUnroll][MT];  // their weight scales
+    };
+    auto load = [&](Batch& v, const Cursor& c) {
+#pragma unroll
+        for (int u = 0; u < kQUnroll; ++u)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                const uint32_t at = first[m] + (uint32_t)min(c.b + u, c.end - 1);
+                if constexpr (BITS == 8) {
+                    v.q[u][m] = ldg_stream(codes + (size_t)at * kCode);
+                } else {
+                    const uint2 w = ldg_stream_u2(codes + (size_t)at * kCode);
+                    v.q[u][m].x = w.x;
+                    v.q[u][m].z = w.y;
+                }
+                const uint32_t d = ldg_stream_u1(scales + (size_t)at * kQTile);
+                v.d[u][m] = c.b + u < c.end ? d : 0u;
+            }
+    };
+    Batch v0, v1;
+    Cursor cl{0, 0, 0};  // the batch to load next
+    enter(cl);
+    Cursor cc = cl;      // the batch to consume next
+    load(v0, cl);
+    next(cl);
+    load(v1, cl);
+    next(cl);
+    if (lane < kRowsW)
+        for (int p = 0; p < kQMaxParts; ++p) rsum[p][warp][lane] = 0.f;  // (halves without blocks)
     pdl_wait();
 
     // ---------------------------------------------------------------- input digits of the part
     float rinv = 1.f;
     if (a.x != nullptr) {
         float ss = 0.f;
+#pragma unroll 16
         for (int i = tid; i < W.k; i += kQThreads) {
             const float v = __half2float(a.x[i]);
             ss = fmaf(v, v, ss);
@@ -194,115 +259,136 @@ __global__ void __launch_bounds__(kQThreads) k_gemv_q(const __grid_constant__ QG
         __syncthreads();
         rinv = red[kQWarps];
     }
-    for (int j = warp; j < npb; j += kQWarps) {
-        const int i = (pb0 + j) * kQBlock + lane;
-        float v = 0.f;
-        if (i < W.k) v = a.x != nullptr ? __half2float(a.x[i]) * rinv * __half2float(a.gain[i]) : __ldcg(a.vin + i);
-        // the block's largest magnitude (non-negative floats order as their bit patterns)
-        const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v))));
-        const float s1 = amax / 127.0f, s2 = s1 / 254.0f, s3 = s2 / 254.0f;
-        const float i1 = amax > 0.f ? 127.0f / amax : 0.f, i2 = i1 * 254.0f, i3 = i2 * 254.0f;
-        // three digits: each takes the remainder of the ones before, to within half its step
-        const float sc[3] = {s1, s2, s3}, iv[3] = {i1, i2, i3};
-        int q[3];
-        float r = v;
+    for (int j0 = warp * 4; j0 < npb; j0 += kQWarps * 4) {  // four blocks at a time
+        float v[4], am = 0.f;
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            const float f = rintf(r * iv[e]);
-            q[e] = (int)fminf(fmaxf(f, -127.f), 127.f);
-            r = fmaf(-(float)q[e], sc[e], r);
+        for (int u = 0; u < 4; ++u) {
+            const int i = (pb0 + j0 + u) * kQBlock + lane;
+            v[u] = 0.f;
+            if (j0 + u < npb && i < W.k)
+                v[u] = a.x != nullptr ? __half2float(a.x[i]) * rinv * __half2float(a.gain[i]) : __ldcg(a.vin + i);
         }
-        // digits in the codes' own (natural) order: A and B fragments are both loaded by byte
-        // position, so the MMA sees the same permutation of k on both sides
-        int qs[3];
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            xq[j * 96 + e * 32 + lane] = (int8_t)q[e];
-            qs[e] = __reduce_add_sync(0xffffffffu, q[e]);
+        for (int u = 0; u < 4; ++u) {
+            // the block's largest magnitude (non-negative floats order as their bit patterns)
+            const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v[u]))));
+            if (lane == u) am = m;
         }
-        if (lane == 0) {
-            xsc[j] = make_float4(s1, s2, s3, 0.f);
-            xsum[j] = make_int4(BIAS * qs[0], BIAS * qs[1], BIAS * qs[2], 0);
+        // lane u: the scales of block u and the inverse of the first
+        const float s1 = am / 127.0f, s2 = s1 / 254.0f, s3 = s2 / 254.0f;
+        const float i1 = am > 0.f ? 127.0f / am : 0.f;
+        if (lane < 4 && j0 + lane < npb) xsc[j0 + lane] = make_float4(s1, s2, s3, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float sc[2] = {__shfl_sync(0xffffffffu, s1, u), __shfl_sync(0xffffffffu, s2, u)};
+            const float b1 = __shfl_sync(0xffffffffu, i1, u), b2 = b1 * 254.0f;
+            const float iv[3] = {b1, b2, b2 * 254.0f};
+            if (j0 + u >= npb) break;  // (the same for the whole warp)
+            // three digits: each takes the remainder of the ones before, to within half its step, in
+            // the order in which the codes unpack (codes_f16)
+            const int at = BITS == 8 ? lane : (lane & ~3) | ((lane & 1) << 1) | ((lane >> 1) & 1);
+            float r = v[u], start = 0.f;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                const int q = (int)fminf(fmaxf(rintf(r * iv[e]), -127.f), 127.f);
+                if (e < 2) r = fmaf(-(float)q, sc[e], r);
+                xq[(j0 + u) * 96 + e * 32 + at] = __int2half_rn(q);
+                const int sum = __reduce_add_sync(0xffffffffu, q);
+                if (lane == e) start = (float)(-OFFSET * sum);
+            }
+            if (lane < 8) xst[(j0 + u) * 8 + lane] = start;
         }
     }
     __syncthreads();
     pdl_launch_dependents();
 
     // ---------------------------------------------------------------- this warp's blocks
-    float acc_a = 0.f, acc_b = 0.f;
-    auto consume = [&](const uint2 (&va)[kQUnroll], const uint2 (&vb)[kQUnroll], const __half2 (&dv)[kQUnroll], int bb) {
+    float acc[2 * MT];  // rows g, g + 8 of each row tile
+#pragma unroll
+    for (int i = 0; i < 2 * MT; ++i) acc[i] = 0.f;
+    auto consume = [&](const Batch& v) {
 #pragma unroll
         for (int u = 0; u < kQUnroll; ++u) {
-            const int b = bb + u;
-            if (b >= wb1) break;
-            const int j = b - pb0;
-            uint32_t af[4];
-            if constexpr (BITS == 8) {
-                af[0] = va[u].x;
-                af[1] = vb[u].x;
-                af[2] = va[u].y;
-                af[3] = vb[u].y;
-            } else {  // byte i of the word: code 8t + i (low nibble), 8t + 4 + i (high nibble)
-                af[0] = va[u].x & 0x0F0F0F0Fu;
-                af[1] = vb[u].x & 0x0F0F0F0Fu;
-                af[2] = (va[u].x >> 4) & 0x0F0F0F0Fu;
-                af[3] = (vb[u].x >> 4) & 0x0F0F0F0Fu;
-            }
-            uint2 bf = make_uint2(0u, 0u);
-            if (g < 3) bf = *reinterpret_cast<const uint2*>(xq + j * 96 + g * 32 + 8 * t);
-            int d[4] = {0, 0, 0, 0};
-            mma_u8s8(d, af, bf.x, bf.y);
-            // lane t = 0 holds the digit-1 and digit-2 products of rows g, g + 8; lane t = 1 digit 3
-            const int d3a = __shfl_down_sync(0xffffffffu, d[0], 1);
-            const int d3b = __shfl_down_sync(0xffffffffu, d[2], 1);
-            if (t == 0) {
-                const float4 sc = xsc[j];
-                const int4 qb = xsum[j];
-                float va_ = sc.z * (float)(d3a - qb.z);
-                va_ = fmaf(sc.y, (float)(d[1] - qb.y), va_);
-                va_ = fmaf(sc.x, (float)(d[0] - qb.x), va_);
-                float vb_ = sc.z * (float)(d3b - qb.z);
-                vb_ = fmaf(sc.y, (float)(d[3] - qb.y), vb_);
-                vb_ = fmaf(sc.x, (float)(d[2] - qb.x), vb_);
-                const float2 ds = __half22float2(dv[u]);
-                acc_a = fmaf(ds.x, va_, acc_a);
-                acc_b = fmaf(ds.y, vb_, acc_b);
+            const int j = min(cc.b + u, cc.end - 1) - pb0;  // (past the end: zero scales)
+            uint4 bf = make_uint4(0u, 0u, 0u, 0u);
+            if (g < 3) bf = *reinterpret_cast<const uint4*>(xq + j * 96 + g * 32 + 8 * t);
+            const float2 st = *reinterpret_cast<const float2*>(xst + j * 8 + 2 * t);
+            const float4 sc = xsc[j];
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                uint32_t ha[4], hb[4];
+                codes_f16<BITS>(v.q[u][m].x, v.q[u][m].y, ha);
+                codes_f16<BITS>(v.q[u][m].z, v.q[u][m].w, hb);
+                float c[4], d[4];
+                mma_f16f32(c, ha[0], hb[0], ha[1], hb[1], bf.x, bf.y, st.x, st.y, st.x, st.y);
+                mma_f16f32(d, ha[2], hb[2], ha[3], hb[3], bf.z, bf.w, c[0], c[1], c[2], c[3]);
+                // lane t = 0 holds the digit-1 and digit-2 products of its rows, lane t = 1 digit 3 (the
+                // other lanes' sums are not used)
+                const float d3a = __shfl_down_sync(0xffffffffu, d[0], 1), d3b = __shfl_down_sync(0xffffffffu, d[2], 1);
+                float va = sc.z * d3a, vb = sc.z * d3b;
+                va = fmaf(sc.y, d[1], va);
+                vb = fmaf(sc.y, d[3], vb);
+                va = fmaf(sc.x, d[0], va);
+                vb = fmaf(sc.x, d[2], vb);
+                const float2 ds = h2_to_f2(v.d[u][m]);
+                acc[2 * m] = fmaf(ds.x, va, acc[2 * m]);
+                acc[2 * m + 1] = fmaf(ds.y, vb, acc[2 * m + 1]);
             }
         }
     };
-    for (int bb = wb0; bb < wb1; bb += 2 * kQUnroll) {
-        consume(pa[0], pb[0], pd[0], bb);
-        load(pa[0], pb[0], pd[0], bb + 2 * kQUnroll);
-        if (bb + kQUnroll < wb1) {
-            consume(pa[1], pb[1], pd[1], bb + kQUnroll);
-            load(pa[1], pb[1], pd[1], bb + 3 * kQUnroll);
+    // after the last batch of a part: the part's sums of this warp's rows
+    auto advance = [&]() {
+        const int p = cc.p;
+        next(cc);
+        if (cc.p != p) {
+#pragma unroll
+            for (int i = 0; i < 2 * MT; ++i) {
+                if (t == 0) rsum[p][warp][8 * i + g] = acc[i];
+                acc[i] = 0.f;
+            }
+        }
+    };
+    __syncwarp();  // rsum is cleared
+    while (cc.p < np) {
+        consume(v0);
+        load(v0, cl);
+        next(cl);
+        advance();
+        if (cc.p < np) {
+            consume(v1);
+            load(v1, cl);
+            next(cl);
+            advance();
         }
     }
-    if (t == 0) {
-        rsum[warp][g] = acc_a;
-        rsum[warp][g + 8] = acc_b;
-    }
     __syncthreads();
-    if (tid < kQRows) rows_sum[tid] = rsum[tid >> 4][tid & 15] + rsum[4 + (tid >> 4)][tid & 15];  // halves in order
+    for (int i = tid; i < np * kQRows; i += kQThreads) {  // halves in order
+        const int p = i / kQRows, r = i % kQRows;
+        rows_sum[p][r] = rsum[p][r / kRowsW][r % kRowsW] + rsum[p][4 + r / kRowsW][r % kRowsW];
+    }
 
     // ---------------------------------------------------------------- parts of the cluster
-    if (parts > 1) cluster_sync();  // every part's row sums are in its shared memory
+    if (ranks > 1) cluster_sync();  // every part's row sums are in its CTA's shared memory
     else __syncthreads();
     float tv = 0.f;
-    const int r = tid, row = (int)blockIdx.y * kQRows + r;
-    if (part == 0 && tid < kQRows) {
-        for (int p = 0; p < parts; ++p) tv += p == 0 ? rows_sum[r] : dsmem_ld(dsmem_addr(&rows_sum[r], (uint32_t)p));
-        rows_sum[r] = tv;
+    const int r = tid, row = tile_row + r;
+    if (rank == 0 && tid < kQRows) {
+        for (int k = 0; k < ranks; ++k) {
+            const int n = (k + 1) * parts / ranks - k * parts / ranks;
+            for (int p = 0; p < n; ++p) tv += k == 0 ? rows_sum[p][r] : dsmem_ld(dsmem_addr(&rows_sum[p][r], (uint32_t)k));
+        }
     }
-    if (parts > 1) cluster_sync();  // rank 0 has read the others' sums (they may leave), and its own are final
+    __syncthreads();
+    if (rank == 0 && tid < kQRows) rows_sum[0][r] = tv;
+    if (ranks > 1) cluster_sync();  // rank 0 has read the others' sums (they may leave), and its own are final
     else __syncthreads();
-    if (part != 0 || tid >= kQRows || row >= W.rows) return;
+    if (rank != 0 || tid >= kQRows || row >= W.rows) return;
 
     // ---------------------------------------------------------------- epilogue (row pairs)
     if constexpr (EPI == kEpiPlain) {
         a.out[row] = tv;
     } else if ((r & 1) == 0 && row + 1 < W.rows) {
-        const float t_odd = rows_sum[r + 1];
+        const float t_odd = rows_sum[0][r + 1];
         if constexpr (EPI == kEpiSwiglu) {
             a.out[row >> 1] = silu(tv) * t_odd;
         } else {  // kEpiQkvRope: rows (row, row + 1) are the RoPE pair (i, i + dh / 2)
@@ -332,26 +418,38 @@ __global__ void __launch_bounds__(kQThreads) k_gemv_q(const __grid_constant__ QG
     }
 }
 
+template <int EPI, int NG, int MT>
+__global__ void __launch_bounds__(kQThreads, 3) k_gemv_q(const __grid_constant__ DecodeGroup<QGemvArgs, NG> G) {
+    int gi = 0, y = (int)blockIdx.y;  // the shard that owns this row tile
+    if constexpr (NG > 1) {
+        while (gi + 1 < G.n && y >= G.end[gi]) ++gi;
+        if (gi > 0) y -= G.end[gi - 1];
+    }
+    const QGemvArgs& a = G.a[gi];
+    if (a.w.bits == 8) gemv_q_cta<EPI, 8, MT>(a, y * 64 * MT);
+    else gemv_q_cta<EPI, 4, MT>(a, y * 64 * MT);
+}
+
 // ================================================================== device: quantizer
 //
-// One thread per block of 32 weights of a row: the fp16 scale and the biased codes of the format
+// One thread per block of 32 weights of a row: the fp16 scale and the codes of the format
 // above, packed into the kernel layout.  Every decision is the host quantizer's: IEEE fp32
 // division (amax / qmax and w / d), one rounding of the scale to fp16, round-half-even of w / d,
 // so the codes equal those of vt_quantize_rows bit for bit.
 template <int BITS>
 __global__ void k_quantize_rows(const __half* __restrict__ w, int64_t ld, int rows, int k, int nb,
-                                uint8_t* __restrict__ codes, int64_t row_bytes, __half* __restrict__ scales) {
+                                uint8_t* __restrict__ codes, __half* __restrict__ scales) {
     constexpr int QMAX = BITS == 8 ? 127 : 7, BIAS = BITS == 8 ? 128 : 8;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)rows * nb) return;
     const int r = (int)(t / nb), b = (int)(t - (int64_t)r * nb);
+    if (r >= (rows + kQTile - 1) / kQTile * kQTile) return;
     const __half* src = w + (int64_t)r * ld + (int64_t)b * kQBlock;
-    const int n = min(kQBlock, k - b * kQBlock);
+    const int n = r < rows ? min(kQBlock, k - b * kQBlock) : 0;  // (rows past the end: zeros)
     float amax = 0.f;
     for (int e = 0; e < n; ++e) amax = fmaxf(amax, fabsf(__half2float(src[e])));
     const __half d16 = __float2half_rn(amax / (float)QMAX);
     const float d = __half2float(d16);
-    scales[(int64_t)r * nb + b] = d16;
+    scales[qscale_at(r, b, nb)] = d16;
     uint32_t u[kQBlock];
 #pragma unroll
     for (int e = 0; e < kQBlock; ++e) {
@@ -362,61 +460,77 @@ __global__ void k_quantize_rows(const __half* __restrict__ w, int64_t ld, int ro
         }
         u[e] = (uint32_t)(c + BIAS);
     }
-    uint8_t* dst = codes + (int64_t)r * row_bytes + (int64_t)b * (BITS == 8 ? 32 : 16);
-    if constexpr (BITS == 8) {
-        uint32_t wd[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) wd[i] = u[4 * i] | (u[4 * i + 1] << 8) | (u[4 * i + 2] << 16) | (u[4 * i + 3] << 24);
-        reinterpret_cast<uint4*>(dst)[0] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-        reinterpret_cast<uint4*>(dst)[1] = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-    } else {
-        uint32_t wd[4];
+    for (int g = 0; g < 4; ++g) {  // positions 8g .. 8g + 7
+        uint8_t* dst = codes + qcode_at(r, b, g, nb, BITS);
+        if constexpr (BITS == 8) {
+            uint32_t wd[2];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t* v = u + 8 * g + 4 * i;
+                wd[i] = v[0] | (v[1] << 8) | (v[2] << 16) | (v[3] << 24);
+            }
+            *reinterpret_cast<uint2*>(dst) = make_uint2(wd[0], wd[1]);
+        } else {
             uint32_t v = 0;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v |= ((u[8 * g + i] & 15u) | ((u[8 * g + i + 4] & 15u) << 4)) << (8 * i);
-            wd[g] = v;
+            for (int i = 0; i < 4; ++i) v |= (u[8 * g + i] | (u[8 * g + i + 4] << 4)) << (8 * i);
+            *reinterpret_cast<uint32_t*>(dst) = v;
         }
-        *reinterpret_cast<uint4*>(dst) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
     }
 }
 
 cudaError_t launch_quantize_rows(const __half* w, int64_t ld, const QMatDev& m, cudaStream_t st) {
-    const int64_t n = (int64_t)m.rows * m.nb;
+    const int64_t n = qmat_rows(m.rows) * m.nb;
     if (n <= 0) return cudaSuccess;
     const int threads = 128;
     const unsigned blocks = (unsigned)((n + threads - 1) / threads);
     if (m.bits == 8)
-        k_quantize_rows<8><<<blocks, threads, 0, st>>>(w, ld, m.rows, m.k, m.nb, m.codes, m.row_bytes, m.scales);
+        k_quantize_rows<8><<<blocks, threads, 0, st>>>(w, ld, m.rows, m.k, m.nb, m.codes, m.scales);
     else if (m.bits == 4)
-        k_quantize_rows<4><<<blocks, threads, 0, st>>>(w, ld, m.rows, m.k, m.nb, m.codes, m.row_bytes, m.scales);
+        k_quantize_rows<4><<<blocks, threads, 0, st>>>(w, ld, m.rows, m.k, m.nb, m.codes, m.scales);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
-// Parts per row tile: enough CTAs for about 2.5 per SM, each part at least 4 blocks, at most 8
-// (the portable cluster size).
-static int gemv_q_parts(int rows, int nb) {
-    const int tiles = (rows + kQRows - 1) / kQRows;
+// Parts of a shard's blocks: enough for about 2.5 pieces of 64 rows by one part per SM, each part at
+// least 4 blocks, at most 8 (the portable cluster size).
+static int gemv_q_parts(int tiles, int nb) {
     const int want = (int)std::lround(2.5 * (g_num_sms > 0 ? g_num_sms : 148) / std::max(tiles, 1));
     return std::max(1, std::min({kQMaxParts, want, std::max(1, nb / 4)}));
 }
 
-template <int EPI>
-static cudaError_t launch_q_epi(const QGemvArgs& a, cudaStream_t st) {
-    const int parts = gemv_q_parts(a.w.rows, a.w.nb);
-    const int pb = (a.w.nb + parts - 1) / parts;
+// The n shards of `a` in one launch of 64 MT-row tiles by cluster ranks.
+template <int EPI, int NG, int MT>
+static cudaError_t launch_q_group(const QGemvArgs* a, int n, cudaStream_t st) {
+    DecodeGroup<QGemvArgs, NG> G{};
+    int tiles = 0, min_parts = kQMaxParts, max_pb = 1;
+    for (int s = 0; s < n; ++s) {
+        tiles += (a[s].w.rows + 64 * MT - 1) / (64 * MT);
+        G.a[s] = a[s];
+        G.end[s] = tiles;
+        G.a[s].parts = gemv_q_parts((a[s].w.rows + 63) / 64, a[s].w.nb);
+        min_parts = std::min(min_parts, G.a[s].parts);
+    }
+    G.n = n;
+    // CTAs per row tile: the parts of the shard, or, in a group, as many as the launch needs
+    const int ranks = n == 1 ? min_parts : std::min(min_parts, gemv_q_parts(tiles, 4 * kQMaxParts));
+    for (int s = 0; s < n; ++s)
+        for (int k = 0; k < ranks; ++k)
+            max_pb = std::max(max_pb, part_start(G.a[s].w.nb, (k + 1) * G.a[s].parts / ranks, G.a[s].parts) -
+                                          part_start(G.a[s].w.nb, k * G.a[s].parts / ranks, G.a[s].parts));
+    const size_t smem = gemv_q_smem(max_pb);
+    if (smem > 200 * 1024) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)parts, (unsigned)((a.w.rows + kQRows - 1) / kQRows));
+    cfg.gridDim = dim3((unsigned)ranks, (unsigned)tiles);
     cfg.blockDim = dim3(kQThreads);
-    cfg.dynamicSmemBytes = gemv_q_smem(pb);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int na = 0;
     attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = (unsigned)parts;
+    attr[na].val.clusterDim.x = (unsigned)ranks;
     attr[na].val.clusterDim.y = 1;
     attr[na].val.clusterDim.z = 1;
     ++na;
@@ -427,19 +541,36 @@ static cudaError_t launch_q_epi(const QGemvArgs& a, cudaStream_t st) {
     }
     cfg.attrs = attr;
     cfg.numAttrs = (unsigned)na;
-    if (a.w.bits == 8) return cudaLaunchKernelEx(&cfg, k_gemv_q<EPI, 8>, a);
-    if (a.w.bits == 4) return cudaLaunchKernelEx(&cfg, k_gemv_q<EPI, 4>, a);
-    return cudaErrorInvalidValue;
+    return cudaLaunchKernelEx(&cfg, k_gemv_q<EPI, NG, MT>, G);
 }
 
-cudaError_t launch_gemv_q(int epi, const QGemvArgs& a, cudaStream_t st) {
-    if (a.w.rows <= 0) return cudaSuccess;
-    const int parts = gemv_q_parts(a.w.rows, a.w.nb);
-    if (gemv_q_smem((a.w.nb + parts - 1) / parts) > 200 * 1024) return cudaErrorInvalidValue;
+template <int EPI>
+static cudaError_t launch_q_epi(const QGemvArgs* a, int n, cudaStream_t st) {
+    QGemvArgs sel[VT_MAX_DEVICES];
+    int m = 0, pieces = 0;
+    for (int s = 0; s < n; ++s) {
+        if (a[s].w.bits != 8 && a[s].w.bits != 4) return cudaErrorInvalidValue;
+        if (a[s].w.rows > 0) {
+            const int tiles = (a[s].w.rows + 63) / 64;
+            sel[m++] = a[s];
+            pieces += tiles * gemv_q_parts(tiles, a[s].w.nb);
+        }
+    }
+    if (m == 0) return cudaSuccess;
+    // Two row tiles a warp halve the instructions a row spends on the input, but also the CTAs: taken
+    // where 1.75 CTAs an SM are left.  A token through four 8-bit Llama-2-7B shards (5 to 9 CTAs an SM)
+    // 94 us a layer; through one such shard, which never has more than 2.5 pieces an SM, 141 us a layer
+    // with one row tile a warp against 205 with two.
+    const bool wide = 2 * pieces >= 7 * (g_num_sms > 0 ? g_num_sms : 148);
+    if (m == 1) return wide ? launch_q_group<EPI, 1, 2>(sel, m, st) : launch_q_group<EPI, 1, 1>(sel, m, st);
+    return wide ? launch_q_group<EPI, VT_MAX_DEVICES, 2>(sel, m, st) : launch_q_group<EPI, VT_MAX_DEVICES, 1>(sel, m, st);
+}
+
+cudaError_t launch_gemv_q(int epi, const QGemvArgs* a, int n, cudaStream_t st) {
     switch (epi) {
-        case kEpiPlain: return launch_q_epi<kEpiPlain>(a, st);
-        case kEpiSwiglu: return launch_q_epi<kEpiSwiglu>(a, st);
-        case kEpiQkvRope: return launch_q_epi<kEpiQkvRope>(a, st);
+        case kEpiPlain: return launch_q_epi<kEpiPlain>(a, n, st);
+        case kEpiSwiglu: return launch_q_epi<kEpiSwiglu>(a, n, st);
+        case kEpiQkvRope: return launch_q_epi<kEpiQkvRope>(a, n, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -548,9 +679,10 @@ cudaError_t launch_combine_q(const CombineQArgs& a, cudaStream_t st) {
 // One warp per block of 32 elements quantizes each shard's block as it leaves that shard and adds
 // it at once (the same codes, scales and sums as k_quantize_vec followed by k_combine_q, which the
 // tests compare with the oracle), so a block of the layer has one launch instead of one per shard
-// and the codes need no memory.  Latency bound (n * 16 KB): the launches were what it cost (four
-// launches of 10.5 + 3.3 us per block of the layer before, COMBT_US now).  The partials are
-// cleared after reading (they are accumulated into zeroed buffers).
+// and the codes need no memory.  Latency bound (n * 16 KB): the launches were what it cost.  Three
+// layers of the 8B shapes on three devices, partials at 8 bits: 670 us a token with a quantizing
+// launch per shard and a combine, 495 us with this.  The partials are cleared after reading (they
+// are accumulated into zeroed buffers).
 __global__ void __launch_bounds__(256) k_combine_token_q(const __grid_constant__ CombineTokenQArgs a) {
     pdl_wait();
     pdl_launch_dependents();
@@ -595,15 +727,18 @@ cudaError_t launch_combine_token_q(const CombineTokenQArgs& a, cudaStream_t st) 
 cudaError_t init_quant_kernels() {
     const int lim = 200 * 1024;
     cudaError_t e;
-#define VT_Q_ATTR(EPI)                                                                                            \
-    if ((e = cudaFuncSetAttribute(k_gemv_q<EPI, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) \
-        return e;                                                                                                 \
-    if ((e = cudaFuncSetAttribute(k_gemv_q<EPI, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) \
+#define VT_Q_ATTR1(EPI, NG, MT)                                                                                  \
+    if ((e = cudaFuncSetAttribute(k_gemv_q<EPI, NG, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != \
+        cudaSuccess)                                                                                             \
         return e;
+#define VT_Q_ATTR(EPI)                                                              \
+    VT_Q_ATTR1(EPI, 1, 1) VT_Q_ATTR1(EPI, 1, 2) VT_Q_ATTR1(EPI, VT_MAX_DEVICES, 1) \
+    VT_Q_ATTR1(EPI, VT_MAX_DEVICES, 2)
     VT_Q_ATTR(kEpiPlain)
     VT_Q_ATTR(kEpiSwiglu)
     VT_Q_ATTR(kEpiQkvRope)
 #undef VT_Q_ATTR
+#undef VT_Q_ATTR1
     return cudaSuccess;
 }
 

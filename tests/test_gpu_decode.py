@@ -136,6 +136,25 @@ def test_decode_uneven_and_gqa_partitions(vtlib, H, Hk, heads, cols):
                            f"H={H} Hk={Hk}")
 
 
+@pytest.mark.parametrize("H,Hk,dh,cap,L", [(19, 19, 64, 40, 39), (20, 20, 128, 256, 255), (20, 20, 64, 257, 250),
+                                           (9, 9, 64, 256, 255), (9, 9, 128, 257, 256), (12, 12, 64, 2049, 2048),
+                                           (13, 13, 64, 2049, 2040),
+                                           (32, 32, 128, 1536, 1531), (32, 32, 64, 1537, 3), (40, 40, 64, 64, 0),
+                                           (64, 32, 128, 300, 299), (80, 20, 64, 128, 65), (160, 20, 64, 96, 2)])
+def test_decode_attention_clusters_of_every_size(vtlib, H, Hk, dh, cap, L):
+    """One shard with so many KV heads that its attention runs 16, 8 or 4 CTAs a head."""
+    heads, cols = ((0, H),), ((0, 64),)
+    wl = synthetic.small("clusters", n_layers=1, d_model=64, n_heads=H, n_kv_heads=Hk, d_head=dh, d_ffn=64,
+                         head_ranges=heads, ffn_ranges=cols, kv_len=L, decode_steps=1, prompt_len=0, model_id=147)
+    w = wl.layer_weights(0)
+    kc, vc = wl.kv_fill(0, L, cap) if L > 0 else oracle.new_cache(wl, cap)
+    with build(vtlib, wl, capacity=cap) as st:
+        write_cache(vtlib, st, 0, wl, kc, vc, L, heads)
+        vtlib.vt_kv_set_length(st.kv, 0, L)
+        decode_layer_check(vtlib, st, wl, w, 0, wl.hidden(1, stream=8), L, kc, vc, heads, cols, f"Hk={Hk} cap={cap} L={L}")
+        assert vtlib.vt_kv_status(st.kv) == 0
+
+
 def test_decode_head_dim_128_gqa_4(vtlib):
     wl = synthetic.small("dh128", n_layers=1, d_model=1024, n_heads=8, n_kv_heads=2, d_head=128,
                          d_ffn=2752, head_ranges=((0, 4), (4, 8)), ffn_ranges=((0, 1376), (1376, 2752)),

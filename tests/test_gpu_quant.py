@@ -273,3 +273,50 @@ def test_precision_api_rules(vtlib):
         finally:
             vt.vt_kv_destroy(kv)
         vt.vt_partition_set_precision(st.part, (0, 1, ATTN), 8)
+
+
+@pytest.mark.parametrize("d_model,H,Hk,heads,cols,bits,comm,window", [
+    (192, 4, 4, (4,), (70,), (8,), 16, 0),                       # one shard
+    (512, 8, 2, (4, 4), (96, 210), (8,), 16, 0),                 # grouped queries, ragged columns
+    (320, 6, 6, (1, 2, 3), (3, 33, 100), (4,), 16, 5),           # 4 bits, sliding window, short rows
+    (1024, 8, 4, (2, 0, 4, 2), (500, 130, 0, 394), (8, 4, 4), 16, 0),  # mixed bits, empty shards
+    (1024, 8, 8, (2, 2, 2, 2), (256, 256, 256, 256), (4, 8), 4, 0),    # quantized partials
+    (576, 8, 8, (3, 5), (170, 171), (16, 4, 8, 4), 8, 0),        # fp16 attention shards beside quantized ones
+])
+def test_grouped_token_equals_the_shards_one_after_another(vtlib, d_model, H, Hk, heads, cols, bits, comm, window):
+    """vt_decode_token of a partition that the fused kernel does not take runs a block's shards in one
+    launch per phase; its output has the same bits as vt_decode_token_sharded, two tokens in a row
+    (FFN shards block-quantized: the fp16 FFN kernel adds its partial in arrival order)."""
+    vt = vtlib
+    n, F, L0, cap = len(heads), sum(cols), 37, 48
+    hr = tuple((sum(heads[:i]), sum(heads[:i + 1])) for i in range(n))
+    cr = tuple((sum(cols[:i]), sum(cols[:i + 1])) for i in range(n))
+    wl = synthetic.small("grouped", n_layers=2, d_model=d_model, n_heads=H, n_kv_heads=Hk, d_head=64, d_ffn=F,
+                         head_ranges=hr, ffn_ranges=cr, kv_len=L0, decode_steps=2, prompt_len=0, model_id=146)
+
+    def precision(l, d, block):
+        b = bits[(l + 2 * d + block) % len(bits)]
+        return 8 if block == FFN and b == 16 else b
+
+    from paper_2607_07046_gb300.stack import Stack
+    outs = []
+    for step in (vt.vt_decode_token, vt.vt_decode_token_sharded):
+        with Stack(shapes_of(vt, wl, max_seq=cap), wl.layer_weights, hr, cr, cap, precision=precision,
+                   windows=window or None) as st:
+            assert not vt.vt_decode_token_fused_available(st.part)[0]
+            vt.vt_partition_set_comm_bits(st.part, -1, comm)
+            for l in range(2):
+                kc, vc = wl.kv_fill(l, L0)
+                for d, r in enumerate(hr):
+                    k0, k1 = kv_range(wl, r)
+                    if k1 > k0:
+                        vt.vt_kv_write_raw(st.kv, l, d, kc[k0:k1], vc[k0:k1])
+            vt.vt_kv_set_length(st.kv, -1, L0)
+            xs = wl.hidden(2, stream=9)
+            y = torch.empty(2, d_model, dtype=torch.float16, device="cuda")
+            for t in range(2):
+                step(st.part, st.kv, dev(xs[t]), y[t])
+            outs.append(host(y).view(np.uint16))
+            assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
+    assert np.array_equal(outs[0], outs[1])
+    assert np.isfinite(outs[0].view(np.float16)).all()
