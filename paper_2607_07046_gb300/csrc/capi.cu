@@ -1627,6 +1627,14 @@ static cudaError_t attn_slices(const vt_partition* p, int l, const int* dev, int
     const int span = t.window > 0 ? std::min(t.window, kv->cap) : kv->cap;
     t.cluster = attn_cluster_size(hk, t.n, span, quantized);
     t.stages = attn_stages(span, t.cluster);
+    // One large fp16 shard: the O projection starts when attention has finished.  Its CTAs that start
+    // early take what the attention's leave of each SM, so its rows are spread unevenly, and that costs
+    // more than the early start gives: a step of 32 heads and 300 positions 40.2 us, 33.8 with the later
+    // start (24 heads 36.7 and 29.3; 12 heads of Llama-2-13B 26.7 and 25.5; 24 query heads over 6 KV
+    // heads 27.6 and 25.2).  8 heads lose 2% in a sequence of steps, 16 query heads over 4 KV heads 0.4
+    // us, and quantized shards and launches of several 1 to 2%.
+    const AttnShard& one = p->a(l, dev[0]);
+    t.early = !(n == 1 && one.bits == 16 && (hk >= 12 || (one.h1 - one.h0) * s.d_head >= 3072));
     t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)s.d_head));
     t.window = p->m->window[l];
     t.status = kv->status;

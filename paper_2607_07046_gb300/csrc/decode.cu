@@ -577,23 +577,23 @@ int g_attn_cluster = 16;  // set at init: 16 when a 16-CTA cluster can be schedu
 // CTAs per KV head, from the KV heads and shards of the launch and the positions a head may attend to
 // (capacity or window).  More CTAs shorten the slices; but a launch with more CTAs than SMs pays for a
 // second start per SM, and a larger cluster for a longer merge.  So 16 while that is one CTA an SM or
-// less, else 8; at short spans one size less.  A token through one fp16 shard, us a layer:
-//   KV heads \ span     57: 16 / 8 / 4     300: 16 / 8 / 4     1024: 16 / 8 / 4    3000: 16 / 8 / 4
-//    4 (GQA 4)       14.3 / 13.7 / 13.7  15.0 / 15.3 / 17.1  17.4 / 17.8 / 22.9  20.4 / 27.5 / 42.6
-//   12               25.1 / 24.3 / 23.7  25.2 / 24.6 / 23.6  26.1 / 24.9 / 27.8  28.8 / 32.7 / 37.0
-//   16               27.9 / 23.2 / 23.7  28.4 / 23.5 / 25.1  30.6 / 25.8 / 29.4  33.0 / 31.4 / 40.9
-//   32               47.7 / 43.8 / 38.8  48.4 / 44.4 / 40.4  51.1 / 47.3 / 44.6  59.3 / 55.1 / 57.3
-// 32 heads of four shards in one launch: 92.9 / 86.1 / 85.5, 93.3 / 86.3 / 89.2, 99.6 / 92.9 / 94.8,
-// 107.0 / 105.3 / 107.8 (8-bit weights): 4 is for one shard only.  40 heads want 8 at every span (4 is
-// above one CTA an SM too).  `fixed`: 16 whatever the launch, so that a shard's sums do not depend on
-// what runs beside it.
+// less, else 8; at short spans one size less, and one shard with so many heads that 8 are more than
+// 1.5 CTAs an SM takes 4 (four shards in one launch do not: 32 heads, 8-bit weights, us a token and
+// layer with 8 / 4 at 300 positions 86.3 / 89.2, at 1024 92.9 / 94.8).  One fp16 shard, us a layer:
+//   KV heads \ span     7: 16 / 8 / 4      300: 16 / 8 / 4     1024: 16 / 8 / 4    3000: 16 / 8 / 4
+//    2 (GQA 4)       14.0 / 13.5 / 13.4  15.0 / 15.2 / 17.3  17.4 / 17.9 / 22.9  20.6 / 27.6 / 42.8
+//   12               21.8 / 21.4 / 21.5  22.3 / 22.0 / 23.2  23.7 / 24.6 / 27.6  26.3 / 30.0 / 39.0
+//   16               25.4 / 21.5 / 21.5  26.3 / 22.1 / 23.2  28.7 / 24.5 / 27.6  31.4 / 30.1 / 39.2
+//   24               32.7 / 28.8 / 28.7  33.7 / 29.3 / 30.3  36.4 / 31.9 / 35.0  41.0 / 37.6 / 46.5
+//   32               39.8 / 35.4 / 32.4  41.2 / 36.3 / 33.8  45.2 / 40.5 / 38.5  51.0 / 51.4 / 50.7
+//   40               57.3 / 53.0 / 49.7  58.9 / 54.1 / 50.9  62.8 / 58.8 / 55.5  72.4 / 71.6 / 68.5
+// `fixed`: 16 whatever the launch, so that a shard's sums do not depend on what runs beside it.
 int attn_cluster_size(int hk, int shards, int span, bool fixed) {
     const int sms = g_num_sms > 0 ? g_num_sms : 148;
     if (fixed) return g_attn_cluster;
     if (hk * 16 <= sms) return span <= 256 ? 8 : g_attn_cluster;
     if (hk * 8 <= sms) return hk * 12 <= sms && span > 2048 ? g_attn_cluster : 8;
-    const int short_span = hk * 16 > 3 * sms ? 1536 : 256;  // 8 CTAs a head are more than 1.5 an SM
-    return shards == 1 && hk * 4 <= sms && span <= short_span ? 4 : 8;
+    return shards == 1 && hk * 16 > 3 * sms && span <= 3072 ? 4 : 8;
 }
 
 int attn_stages(int span, int csize) {
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn_decode(const __grid_const
             kn[e] = has_new ? __half2float(__ldcg(kbase + (int64_t)pnew * DH + lane * EPL + e)) : 0.f;
             vn[e] = has_new ? __half2float(__ldcg(vbase + (int64_t)pnew * DH + lane * EPL + e)) : 0.f;
         }
-        pdl_launch_dependents();
+        if (a.early) pdl_launch_dependents();
 
         float m[G], l[G], o[G][EPL];
 #pragma unroll

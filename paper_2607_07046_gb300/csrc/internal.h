@@ -81,6 +81,7 @@ struct AttnDecodeArgs {  // one layer, every shard of the launch
     int cap;
     int group;             // query heads per KV head
     int dh;
+    bool early;            // let the next kernel start while this one runs
     int cluster;           // CTAs per KV head (attn_cluster_size)
     int stages;            // K/V tiles in flight per CTA (attn_stages)
     float scale_log2;      // log2(e) / sqrt(dh)

@@ -139,7 +139,7 @@ def test_decode_uneven_and_gqa_partitions(vtlib, H, Hk, heads, cols):
 @pytest.mark.parametrize("H,Hk,dh,cap,L", [(19, 19, 64, 40, 39), (20, 20, 128, 256, 255), (20, 20, 64, 257, 250),
                                            (9, 9, 64, 256, 255), (9, 9, 128, 257, 256), (12, 12, 64, 2049, 2048),
                                            (13, 13, 64, 2049, 2040),
-                                           (32, 32, 128, 1536, 1531), (32, 32, 64, 1537, 3), (40, 40, 64, 64, 0),
+                                           (32, 32, 128, 1536, 1531), (32, 32, 64, 3073, 3), (32, 32, 64, 3072, 3000), (40, 40, 64, 64, 0),
                                            (64, 32, 128, 300, 299), (80, 20, 64, 128, 65), (160, 20, 64, 96, 2)])
 def test_decode_attention_clusters_of_every_size(vtlib, H, Hk, dh, cap, L):
     """One shard with so many KV heads that its attention runs 16, 8 or 4 CTAs a head."""
