@@ -508,7 +508,7 @@ VT_API vt_status vt_partition_set_comm_bits(vt_partition* part, int32_t device, 
  *   Otherwise (unsupported shapes, or x_out not 16-byte aligned) it runs the kernels of
  *   vt_decode_token_sharded with the shards of a block side by side: one launch per phase (and
  *   precision).  Its results have the same bits as vt_decode_token_sharded's, except that an
- *   attention launch with more KV heads may cut the cached positions into fewer slices (the sums
+ *   attention launch of several shards may cut the cached positions into fewer slices (the sums
  *   then differ in fp32 rounding; never while partials are quantized), and that fp16 FFN shards
  *   add their partial in arrival order in both.
  *   The launch can be captured in a CUDA graph.

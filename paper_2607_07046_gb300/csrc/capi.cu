@@ -1626,7 +1626,6 @@ static cudaError_t attn_slices(const vt_partition* p, int l, const int* dev, int
     for (int b : p->comm_bits) quantized |= b != 16;
     const int span = t.window > 0 ? std::min(t.window, kv->cap) : kv->cap;
     t.cluster = attn_cluster_size(hk, t.n, span, quantized);
-    t.stages = attn_stages(span, t.cluster);
     // One large fp16 shard: the O projection starts when attention has finished.  Its CTAs that start
     // early take what the attention's leave of each SM, so its rows are spread unevenly, and that costs
     // more than the early start gives: a step of 32 heads and 300 positions 40.2 us, 33.8 with the later
@@ -1635,6 +1634,7 @@ static cudaError_t attn_slices(const vt_partition* p, int l, const int* dev, int
     // us, and quantized shards and launches of several 1 to 2%.
     const AttnShard& one = p->a(l, dev[0]);
     t.early = !(n == 1 && one.bits == 16 && (hk >= 12 || (one.h1 - one.h0) * s.d_head >= 3072));
+    t.stages = attn_stages(hk, span, t.cluster, t.early);
     t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)s.d_head));
     t.window = p->m->window[l];
     t.status = kv->status;

@@ -587,18 +587,26 @@ int g_attn_cluster = 16;  // set at init: 16 when a 16-CTA cluster can be schedu
 //   24               32.7 / 28.8 / 28.7  33.7 / 29.3 / 30.3  36.4 / 31.9 / 35.0  41.0 / 37.6 / 46.5
 //   32               39.8 / 35.4 / 32.4  41.2 / 36.3 / 33.8  45.2 / 40.5 / 38.5  51.0 / 51.4 / 50.7
 //   40               57.3 / 53.0 / 49.7  58.9 / 54.1 / 50.9  62.8 / 58.8 / 55.5  72.4 / 71.6 / 68.5
+// Four shards with 8 KV heads of 4 queries between them (8 bits) want 8 also where 16 no longer hold
+// their slices in one tile: 16 / 8 at 600 positions 97.7 / 98.2, 1026 106.1 / 100.4, 3000 112.7 / 110.0.
 // `fixed`: 16 whatever the launch, so that a shard's sums do not depend on what runs beside it.
 int attn_cluster_size(int hk, int shards, int span, bool fixed) {
     const int sms = g_num_sms > 0 ? g_num_sms : 148;
     if (fixed) return g_attn_cluster;
-    if (hk * 16 <= sms) return span <= 256 ? 8 : g_attn_cluster;
+    if (hk * 16 <= sms) return span <= 256 || (shards > 1 && span > 1024 && span <= 3072) ? 8 : g_attn_cluster;
     if (hk * 8 <= sms) return hk * 12 <= sms && span > 2048 ? g_attn_cluster : 8;
     return shards == 1 && hk * 16 > 3 * sms && span <= 3072 ? 4 : 8;
 }
 
-int attn_stages(int span, int csize) {
+// Tiles of K and V in flight per CTA: those of its slice, at most 3.  Where a launch is one CTA an SM or
+// less and the next kernel may start early, slices of two tiles take 3 stages too: two CTAs of 2 stages
+// fit an SM, and the clusters were packed so (8 query heads of Llama-3-8B, 1024 / 2000 positions: 17.4 /
+// 20.5 us a step, 15.7 / 17.7 with 3; four shards in one launch, 8 bits: 110.8 -> 105.1 a layer at 2000).
+// Before a kernel that starts after the attention 3 stages lose (32 heads of 8: 29.8 -> 34.4).
+int attn_stages(int hk, int span, int csize, bool early) {
     const int per = (span + csize - 1) / csize;
     int t = (per + kAttnTilePos - 1) / kAttnTilePos;
+    if (early && t > 1 && hk * csize <= (g_num_sms > 0 ? g_num_sms : 148)) return kAttnMaxStages;
     return t < 1 ? 1 : (t > kAttnMaxStages ? kAttnMaxStages : t);
 }
 

@@ -128,7 +128,7 @@ cudaError_t launch_attn_decode(const AttnDecodeArgs& a, cudaStream_t st);
 size_t attn_decode_smem_bytes(int dh, int group, int stages);
 // hk: KV heads of the launch; span: positions that a head attends to at most (capacity or window)
 int attn_cluster_size(int hk, int shards, int span, bool fixed);
-int attn_stages(int span, int csize);
+int attn_stages(int hk, int span, int csize, bool early);
 cudaError_t launch_combine(const CombineArgs& a, cudaStream_t st);
 cudaError_t launch_ffn_decode(const FfnDecodeArgs* a, int n, cudaStream_t st);
 cudaError_t launch_transpose_f16(const __half* src, int64_t src_ld, int rows, int cols, __half* dst,
