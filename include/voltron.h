@@ -542,6 +542,11 @@ VT_API vt_status vt_token_partials_read(const vt_partition* part, int32_t block,
  * vt_partition_status with clear = 1 removes both settings and re-arms the barrier.
  * Synchronous.  VT_ERR_STATE when the partition has no fused kernel. */
 VT_API vt_status vt_token_test_barrier(vt_partition* part, int32_t cta, uint32_t spin_polls, vt_stream stream);
+/* Test hook (library plumbing) for the other kernels' waits: launches one warp that waits for a phase
+ * that nothing completes, by the wait of a CTA (`form` 0), of a thread-block cluster (1) or of the
+ * prefill attention's copies (2).  The wait gives up after about two seconds and sets
+ * VT_DEV_WAIT_TIMEOUT in the device word `status`; the stream stays usable. */
+VT_API vt_status vt_test_wait_limit(int32_t form, uint32_t* status, vt_stream stream);
 /* vt_prefill_tokens (Section 2.1, prefill phase, through the tensor-parallel layers of Section
  * 3.2.1): n prompt rows through every layer (same order as vt_decode_token), then every layer's
  * KV length advances by n.  x_in, x_out: device fp16 [n, D], may be the same.  The shards of a

@@ -1994,6 +1994,12 @@ extern "C" vt_status vt_token_test_barrier(vt_partition* p, int32_t cta, uint32_
     return ok();
 }
 
+extern "C" vt_status vt_test_wait_limit(int32_t form, uint32_t* status, vt_stream stream) {
+    if (form < 0 || form > 2 || !status) return fail(VT_ERR_INVALID_ARG, "bad vt_test_wait_limit arguments");
+    VT_CUDA(launch_wait_limit(form, status, (cudaStream_t)stream));
+    return ok();
+}
+
 // The combine of one block of the whole-token path: the plain fp32 combine, or, when some
 // device's partials travel quantized (communication scaling), the combine that quantizes each such
 // partial on its way (both clear the fp32 partials).

@@ -46,23 +46,44 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
         "r"(bytes)
         : "memory");
 }
+// One poll of a phase; it may suspend the thread for about kSuspendNs (it wakes as soon as the phase
+// completes).
+constexpr uint32_t kSuspendNs = 1000;
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
         : "memory");
     return ok != 0;
 }
-// Waits for the phase with the given parity to complete, giving up after kSpinLimit polls
-// (each poll may itself suspend the thread for a short, hardware-chosen time).  Returns false on
-// timeout; the caller records VT_DEV_WAIT_TIMEOUT and stops using the stage.
-constexpr uint32_t kSpinLimit = 1u << 24;
+// Every wait ends: it gives up once it has polled kWaitPolls times or, from kWaitMinPolls polls on,
+// kWaitNs of the global timer after it began (the time alone could be that of another process that
+// had the GPU meanwhile; the number of polls alone says nothing, since each may suspend the thread
+// for a time that the hardware chooses).  The timer is read every 64 failed polls only.
+constexpr uint32_t kWaitPolls = 1u << 24, kWaitMinPolls = 1024;
+constexpr uint64_t kWaitNs = 2000000000ull;
+struct WaitLimit {
+    uint64_t t0 = 0;
+    uint32_t polls = 0;
+    // After a failed poll: true when the wait has to give up.
+    __device__ __forceinline__ bool over() {
+        if ((++polls & 63u) != 0) return false;
+        uint64_t t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (polls == 64) t0 = t;
+        return polls >= kWaitPolls || (polls >= kWaitMinPolls && t - t0 >= kWaitNs);
+    }
+};
+// Waits for the phase with the given parity to complete.  Returns false when the wait gave up; the
+// caller records VT_DEV_WAIT_TIMEOUT and stops using the stage.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    for (uint32_t i = 0; i < kSpinLimit; ++i)
+    WaitLimit limit;
+    do {
         if (mbar_try_wait(bar, parity)) return true;
+    } while (!limit.over());
     return false;
 }
 
@@ -73,16 +94,17 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
-    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    WaitLimit limit;
+    do {
         uint32_t ok;
         asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
-            : "r"(smem_u32(bar)), "r"(parity)
+            : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
             : "memory");
         if (ok) return true;
-    }
+    } while (!limit.over());
     return false;
 }
 

@@ -987,6 +987,32 @@ __device__ __forceinline__ uint32_t fa_range_bits(int b, int e) {
     return below_e & ~((1u << b) - 1u);
 }
 
+// Test hook: one warp in each form of the kernels' waits, for a phase that nothing completes.
+__global__ void k_wait_limit(int form, uint32_t* status) {
+    __shared__ uint64_t bar;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        fence_mbar_init();
+    }
+    __syncwarp();
+    bool ok = false;
+    if (form == 0) {
+        ok = mbar_wait_warp(&bar, 0);
+    } else if (form == 1) {
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&bar, 0));
+    } else {
+        WaitLimit idle;
+        while (!(ok = __all_sync(0xffffffffu, fa_test(&bar, 0))))
+            if (__any_sync(0xffffffffu, idle.over())) break;
+    }
+    if (!ok && threadIdx.x == 0) set_status(status, VT_DEV_WAIT_TIMEOUT);
+}
+
+cudaError_t launch_wait_limit(int form, uint32_t* status, cudaStream_t st) {
+    k_wait_limit<<<1, 32, 0, st>>>(form, status);
+    return cudaGetLastError();
+}
+
 template <int DH>
 __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_constant__ FaGroup G) {
     constexpr uint32_t kQBytes = kFaRows * DH * 2, kKVBytes = kFaKeys * DH * 2, kPBytes = kFaRows * kFaKeys * 2;
@@ -1084,7 +1110,7 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
                 return j < 2 || __all_sync(0xffffffffu, fa_test(&empty[j & 1], ((j - 2) >> 1) & 1));
             };
             int jk = 0, jv = 0;
-            uint32_t idle = 0;
+            WaitLimit idle;
             bool ok = true;
             while (jk < nb || jv < nb) {
                 bool moved = false;
@@ -1097,8 +1123,8 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
                     moved = true;
                 }
                 if (moved) {
-                    idle = 0;
-                } else if (++idle > (kSpinLimit << 2) || __any_sync(0xffffffffu, *s_err)) {
+                    idle = WaitLimit();
+                } else if (__any_sync(0xffffffffu, idle.over() || *s_err)) {
                     ok = false;
                     break;
                 }

@@ -159,6 +159,7 @@ def lib() -> ctypes.CDLL:
             "vt_partition_set_comm_bits": (S, [_P, _I32, _I32]),
             "vt_token_partials_read": (S, [_P, _I32, _P]),
             "vt_token_test_barrier": (S, [_P, _I32, _U32, _P]),
+            "vt_test_wait_limit": (S, [_I32, _P, _P]),
         }
         for name, (res, args) in sig.items():
             f = getattr(L, name)
@@ -629,6 +630,12 @@ def vt_token_test_barrier(part: int, cta: int, spin_polls: int, stream=None) -> 
     """Test hook: CTA `cta` of the next fused tokens skips its first grid-barrier arrival and
     grid-barrier waits give up after `spin_polls` polls, until a status clear."""
     _check(lib().vt_token_test_barrier(part, int(cta), int(spin_polls), _stream(stream)))
+
+
+def vt_test_wait_limit(form: int, status, stream=None) -> None:
+    """Test hook: one warp waits (form 0: a CTA's wait, 1: a cluster's, 2: the prefill attention's
+    copies) for what never comes, and sets VT_DEV_WAIT_TIMEOUT in `status` when it gives up."""
+    _check(lib().vt_test_wait_limit(int(form), _ptr(status), _stream(stream)))
 
 
 def vt_prefill_tokens(part: int, kv: int, x_in, n: int, x_out, stream=None) -> None:

@@ -361,3 +361,22 @@ def test_prefill_tokens_7b_two_layers_512_rows(vtlib):
         _check_cache(vt, st, wl, 0, n, kc0, vc0, "7b")
         _check_cache(vt, st, wl, 1, n, kc1, vc1, "7b")
         assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
+
+
+@pytest.mark.parametrize("form", [0, 1, 2])
+def test_a_wait_for_what_never_comes_gives_up_after_two_seconds(vtlib, form):
+    """The waits of the kernels (a CTA's, a cluster's, the prefill attention's polls) end by time and
+    leave the context usable."""
+    vt = vtlib
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    a.record()
+    vt.vt_test_wait_limit(form, status)
+    b.record()
+    torch.cuda.synchronize()
+    assert int(status.item()) == vt.VT_DEV_WAIT_TIMEOUT
+    # the polls alone may end form 2 sooner (2^24 of them, none of which suspends)
+    assert a.elapsed_time(b) < 5000 and (form == 2 or a.elapsed_time(b) > 1900)
+    with pytest.raises(vt.VtError):
+        vt.vt_test_wait_limit(3, status)
