@@ -1871,7 +1871,7 @@ static void ffn_args(const vt_partition* p, vt_shard sh, const __half* x, int n,
 }
 
 static vt_status prefill_shard(const vt_partition* p, vt_shard sh, const __half* x, int n, vt_kv* kv,
-                               float* out, int row_offset, cudaStream_t st, bool xhat_ready = false) {
+                               float* out, int row_offset, PrefillChain& ch, bool xhat_ready = false) {
     const vt_shapes& s = p->m->s;
     if ((sh.block == VT_BLOCK_ATTN ? p->a(sh.layer, sh.device).bits : p->f(sh.layer, sh.device).bits) != 16)
         return fail(VT_ERR_STATE, "prefill runs on fp16 shards; shard (layer %d, device %d, block %d) is block-quantized",
@@ -1881,23 +1881,23 @@ static vt_status prefill_shard(const vt_partition* p, vt_shard sh, const __half*
     if (sh.block == VT_BLOCK_ATTN) {
         const AttnShard& a = p->a(sh.layer, sh.device);
         if (a.h1 == a.h0) {
-            VT_CUDA(launch_fill_zero_f32(out, (int64_t)n * D, st));
+            VT_CUDA(launch_fill_zero_f32(out, (int64_t)n * D, ch.st));
             return VT_OK;
         }
         PrefillAttnArgs t;
         attn_args(p, sh, x, n, kv, out, row_offset, xhat_ready, 0, &t);
-        vt_status r = prefill_attn_shard(t, st, &err);
+        vt_status r = prefill_attn_shard(t, ch, &err);
         if (r != VT_OK) return fail(r, "%s", err.c_str());
     } else {
         const FfnShard& f = p->f(sh.layer, sh.device);
         if (f.c1 == f.c0) {
-            VT_CUDA(launch_fill_zero_f32(out, (int64_t)n * D, st));
+            VT_CUDA(launch_fill_zero_f32(out, (int64_t)n * D, ch.st));
             return VT_OK;
         }
         if (s.d_ffn % 8 != 0) return fail(VT_ERR_SHAPE, "prefill needs d_ffn to be a multiple of 8");
         PrefillFfnArgs t;
         ffn_args(p, sh, x, n, out, xhat_ready, 0, &t);
-        vt_status r = prefill_ffn_shard(t, st, &err);
+        vt_status r = prefill_ffn_shard(t, ch, &err);
         if (r != VT_OK) return fail(r, "%s", err.c_str());
     }
     return VT_OK;
@@ -1906,7 +1906,7 @@ static vt_status prefill_shard(const vt_partition* p, vt_shard sh, const __half*
 // Every shard of one block of layer l, on `rows` rows whose normalised input is in p_xhat: the
 // shards' GEMMs run as one launch per GEMM of the block (empty shards get a zero partial).
 static vt_status prefill_block(const vt_partition* p, int l, vt_block block, const __half* x, int rows, vt_kv* kv,
-                               int row_offset, cudaStream_t st) {
+                               int row_offset, PrefillChain& ch) {
     const vt_shapes& s = p->m->s;
     const int D = s.d_model;
     PrefillAttnArgs at[VT_MAX_DEVICES];
@@ -1917,7 +1917,7 @@ static vt_status prefill_block(const vt_partition* p, int l, vt_block block, con
         const vt_shard sh{l, d, block};
         const bool empty = block == VT_BLOCK_ATTN ? p->a(l, d).h1 == p->a(l, d).h0 : p->f(l, d).c1 == p->f(l, d).c0;
         if (empty) {
-            VT_CUDA(launch_fill_zero_f32(out, (int64_t)rows * D, st));
+            VT_CUDA(launch_fill_zero_f32(out, (int64_t)rows * D, ch.st));
             continue;
         }
         if (block == VT_BLOCK_ATTN) attn_args(p, sh, x, rows, kv, out, row_offset, true, d, &at[n++]);
@@ -1926,7 +1926,7 @@ static vt_status prefill_block(const vt_partition* p, int l, vt_block block, con
     if (block == VT_BLOCK_FFN && n > 0 && s.d_ffn % 8 != 0)
         return fail(VT_ERR_SHAPE, "prefill needs d_ffn to be a multiple of 8");
     std::string err;
-    const vt_status r = block == VT_BLOCK_ATTN ? prefill_attn_group(at, n, st, &err) : prefill_ffn_group(ft, n, st, &err);
+    const vt_status r = block == VT_BLOCK_ATTN ? prefill_attn_group(at, n, ch, &err) : prefill_ffn_group(ft, n, ch, &err);
     if (r != VT_OK) return fail(r, "%s", err.c_str());
     return VT_OK;
 }
@@ -1937,7 +1937,7 @@ extern "C" vt_status vt_prefill(const vt_partition* p, vt_shard sh, const void* 
     if (!x || !out || n < 1) return fail(VT_ERR_INVALID_ARG, "x, out_partial must be set and n >= 1");
     if (!aligned16(x) || !aligned16(out)) return fail(VT_ERR_INVALID_ARG, "x and out_partial must be 16-byte aligned");
     if (n > p->m->s.max_seq) return fail(VT_ERR_INVALID_ARG, "n %d exceeds max_seq", n);
-    cudaStream_t st = (cudaStream_t)stream;
+    PrefillChain ch{(cudaStream_t)stream};
     if (sh.block == VT_BLOCK_ATTN) {
         if (!kv || kv->p != p) return fail(VT_ERR_INVALID_ARG, "an ATTN shard needs this partition's KV cache");
         if ((int64_t)kv->h_len[sh.layer] + n > kv->cap)
@@ -1948,7 +1948,7 @@ extern "C" vt_status vt_prefill(const vt_partition* p, vt_shard sh, const void* 
     for (int r0 = 0; r0 < n; r0 += kPrefillChunk) {
         const int rows = std::min(kPrefillChunk, n - r0);
         VT_TRY(prefill_shard(p, sh, static_cast<const __half*>(x) + (size_t)r0 * D, rows, kv,
-                             out + (size_t)r0 * D, r0, st));
+                             out + (size_t)r0 * D, r0, ch));
     }
     return ok();
 }
@@ -2160,6 +2160,7 @@ extern "C" vt_status vt_prefill_tokens(const vt_partition* p, vt_kv* kv, const v
     for (const FfnShard& f : p->ffn)
         if (f.bits != 16 && f.c1 > f.c0) return fail(VT_ERR_STATE, "prefill runs on fp16 shards; an FFN shard is block-quantized");
     cudaStream_t st = (cudaStream_t)stream;
+    PrefillChain ch{st};
     const int D = s.d_model, nd = p->n_dev;
     for (int r0 = 0; r0 < n; r0 += kPrefillChunk) {
         const int rows = std::min(kPrefillChunk, n - r0);
@@ -2170,19 +2171,19 @@ extern "C" vt_status vt_prefill_tokens(const vt_partition* p, vt_kv* kv, const v
         const __half* cur = static_cast<const __half*>(x_in) + (size_t)r0 * D;
         // Every shard of a block normalises the same input with the same gain: the norm runs once
         // per block, fused into the combine that produced the block's input.
-        VT_CUDA(launch_rmsnorm_rows(cur, p->m->layer[0].attn_norm, s.rms_eps, rows, D, p->p_xhat, 1, st));
+        VT_CUDA(launch_rmsnorm_rows(cur, p->m->layer[0].attn_norm, s.rms_eps, rows, D, p->p_xhat, 1, ch));
         for (int l = 0; l < s.n_layers; ++l) {
-            VT_TRY(prefill_block(p, l, VT_BLOCK_ATTN, cur, rows, kv, r0, st));
+            VT_TRY(prefill_block(p, l, VT_BLOCK_ATTN, cur, rows, kv, r0, ch));
             c.residual = cur;
             c.out = p->hbuf;
-            VT_CUDA(launch_combine_norm(c, rows, D, p->m->layer[l].ffn_norm, s.rms_eps, p->p_xhat, 0, st));
-            VT_TRY(prefill_block(p, l, VT_BLOCK_FFN, p->hbuf, rows, kv, r0, st));
+            VT_CUDA(launch_combine_norm(c, rows, D, p->m->layer[l].ffn_norm, s.rms_eps, p->p_xhat, 0, ch));
+            VT_TRY(prefill_block(p, l, VT_BLOCK_FFN, p->hbuf, rows, kv, r0, ch));
             const bool last = l == s.n_layers - 1;
             __half* dst = last ? static_cast<__half*>(x_out) + (size_t)r0 * D : p->xbuf;
             c.residual = p->hbuf;
             c.out = dst;
             VT_CUDA(launch_combine_norm(c, rows, D, last ? nullptr : p->m->layer[l + 1].attn_norm, s.rms_eps,
-                                        p->p_xhat, 1, st));
+                                        p->p_xhat, 1, ch));
             cur = dst;
         }
     }

@@ -195,17 +195,23 @@ struct PrefillFfnArgs {
     float* out;             // [n][d]
     uint32_t* status;
 };
-vt_status prefill_attn_shard(const PrefillAttnArgs& a, cudaStream_t st, std::string* err);
+// The stream of a call's prefill launches, and whether the launch ahead ran on CTA pairs, or may have
+// (that of another call is not known): the next launch then starts after it has ended.
+struct PrefillChain {
+    cudaStream_t st;
+    bool after_pair = true;
+};
+vt_status prefill_attn_shard(const PrefillAttnArgs& a, PrefillChain& ch, std::string* err);
 // the shards of one block at once (all with the same rows and normalised input): one launch per
 // GEMM of the block for every shard
-vt_status prefill_attn_group(const PrefillAttnArgs* a, int n, cudaStream_t st, std::string* err);
-vt_status prefill_ffn_group(const PrefillFfnArgs* a, int n, cudaStream_t st, std::string* err);
+vt_status prefill_attn_group(const PrefillAttnArgs* a, int n, PrefillChain& ch, std::string* err);
+vt_status prefill_ffn_group(const PrefillFfnArgs* a, int n, PrefillChain& ch, std::string* err);
 // rows x d: out = fp16(residual + sum of partials); with gain, also xhat = RMSNorm(out) * gain.
 // split != 0: xhat rows are 2d long, the fp16 value then the fp16 rounding of the remainder.
 cudaError_t launch_combine_norm(const CombineArgs& a, int rows, int d, const __half* gain, float eps, __half* xhat,
-                                int split, cudaStream_t st);
+                                int split, PrefillChain& ch);
 cudaError_t launch_rmsnorm_rows(const __half* x, const __half* gain, float eps, int rows, int d, __half* y,
-                                int split, cudaStream_t st);
+                                int split, PrefillChain& ch);
 
 // ------------------------------------------------------------------ block-quantized shard weights (quant.cu)
 // A matrix [rows][k] stored as codes of 8 or 4 bits with one fp16 scale per block of kQBlock
@@ -291,7 +297,7 @@ struct StaticAttnLayout {  // byte offsets of the vectors in the array; bytes: w
 StaticAttnLayout static_attn_layout(int hq, int hk, int dh);
 cudaError_t static_scratch_base(void** out);
 
-vt_status prefill_ffn_shard(const PrefillFfnArgs& a, cudaStream_t st, std::string* err);
+vt_status prefill_ffn_shard(const PrefillFfnArgs& a, PrefillChain& ch, std::string* err);
 
 
 // ------------------------------------------------------------------ persistent decode token (token.cu)

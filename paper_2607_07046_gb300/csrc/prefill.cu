@@ -35,16 +35,23 @@
 
 namespace vt {
 
-// Launch in the library's chain of programmatic dependent launches: a kernel's CTAs start, and set up
-// their barriers and tensor memory, while the preceding kernel's last CTAs finish.
+// Launch in the library's chain of programmatic dependent launches: a kernel's CTAs start while the
+// preceding kernel's last CTAs finish.  A launch on CTA pairs (cluster 2) has a whole kernel boundary
+// on both sides: it starts after the launch ahead has ended, as the next one does after it, and its
+// kernel releases no dependents before its CTAs have left (a launch of another call that follows).
+// In the chain, prompts on CTA pairs stopped now and then among thousands, and no cause was found.
+// Two layers of four 7B shards, 512 rows: 472 us inside the chain, 497 outside it; one 13B layer, 2048
+// rows: 1355 and 1388.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pk(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st,
+static cudaError_t launch_pk(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, PrefillChain& ch,
                              Args&&... args) {
+    const bool dependent = g_use_pdl && cluster == 1 && !ch.after_pair;
+    ch.after_pair = cluster > 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
+    cfg.stream = ch.st;
     cudaLaunchAttribute attr[2];
     int na = 0;
     if (cluster > 1) {
@@ -54,7 +61,7 @@ static cudaError_t launch_pk(void (*kern)(KArgs...), dim3 grid, int threads, siz
         attr[na].val.clusterDim.z = 1;
         ++na;
     }
-    if (g_use_pdl) {
+    if (dependent) {
         attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[na].val.programmaticStreamSerializationAllowed = 1;
         ++na;
@@ -421,12 +428,12 @@ __global__ void __launch_bounds__(1024) k_combine_norm(const __grid_constant__ C
 }
 
 cudaError_t launch_combine_norm(const CombineArgs& a, int rows, int d, const __half* gain, float eps, __half* xhat,
-                                int split, cudaStream_t st) {
+                                int split, PrefillChain& ch) {
     if (rows <= 0) return cudaSuccess;
     if (d % 8 != 0 || d > 16384) return cudaErrorInvalidValue;
     const int mc = row_mc(rows, d), t = row_threads(mc, d);
-    return mc == 1 ? launch_pk(k_combine_norm<1>, dim3(rows), t, 0, 1, st, a, d, gain, eps, xhat, split)
-                   : launch_pk(k_combine_norm<2>, dim3(rows), t, 0, 1, st, a, d, gain, eps, xhat, split);
+    return mc == 1 ? launch_pk(k_combine_norm<1>, dim3(rows), t, 0, 1, ch, a, d, gain, eps, xhat, split)
+                   : launch_pk(k_combine_norm<2>, dim3(rows), t, 0, 1, ch, a, d, gain, eps, xhat, split);
 }
 
 // ================================================================== tensor-core GEMM
@@ -677,7 +684,7 @@ __global__ void __launch_bounds__(kPThreads, 1) k_gemm_p(const __grid_constant__
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (the whole warp)
         pdl_wait();  // A was written by the preceding kernel
-        pdl_launch_dependents();
+        if constexpr (CG == 1) pdl_launch_dependents();  // (pairs: launch_pk)
         uint32_t slot = 0, phase = 0, filled = 0;  // ring position; stages filled so far
         // boxes of fewer rows do not fill the ring's copy rate anyway (48-row boxes: 31.2 us without
         // the requests, 33.1 with them; 64 rows: 32.4 and 29.3)
@@ -1556,7 +1563,7 @@ static PGemmPlan plan_pgemm(const GemmSpec* specs, int ng, int m) {
 // The grouped GEMMs of `specs` (all with m rows) as one persistent launch: one CTA (CG = 1) or
 // one CTA pair (CG = 2, 256-row tiles) per SM or SM pair, or one per tile when there are fewer.
 template <int EPI, int CG>
-static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, const PGemmPlan& plan, cudaStream_t st,
+static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, const PGemmPlan& plan, PrefillChain& ch,
                                      std::string* err) {
     PGemmGroup G{};
     G.n_groups = ng;
@@ -1591,7 +1598,7 @@ static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, const
     }
     G.total_tiles = acc;
     const size_t smem = 1024 + (size_t)G.stages * pgemm_stage_bytes(G.am, G.bn / CG, G.kts, G.ab) + kPBarBytes + kPEpiBytes;
-    const cudaError_t e = launch_pk(k_gemm_p<EPI, CG>, dim3((unsigned)(CG * std::min(acc, slots))), kPThreads, smem, CG, st, G);
+    const cudaError_t e = launch_pk(k_gemm_p<EPI, CG>, dim3((unsigned)(CG * std::min(acc, slots))), kPThreads, smem, CG, ch, G);
     if (e != cudaSuccess) {
         *err = std::string("persistent GEMM launch failed: ") + cudaGetErrorString(e);
         return VT_ERR_CUDA;
@@ -1601,29 +1608,29 @@ static vt_status run_gemm_persistent(const GemmSpec* specs, int ng, int m, const
 
 // Launches the GEMMs of `specs` (all with m rows) kGemmGroups at a time.
 template <int EPI>
-static vt_status run_gemm_group(const GemmSpec* specs, int n_specs, int m, cudaStream_t st, std::string* err) {
+static vt_status run_gemm_group(const GemmSpec* specs, int n_specs, int m, PrefillChain& ch, std::string* err) {
     for (int g0 = 0; g0 < n_specs; g0 += kGemmGroups) {
         const int ng = std::min(kGemmGroups, n_specs - g0);
         const PGemmPlan plan = plan_pgemm(specs + g0, ng, m);
-        const vt_status r = plan.cg == 2 ? run_gemm_persistent<EPI, 2>(specs + g0, ng, m, plan, st, err)
-                                         : run_gemm_persistent<EPI, 1>(specs + g0, ng, m, plan, st, err);
+        const vt_status r = plan.cg == 2 ? run_gemm_persistent<EPI, 2>(specs + g0, ng, m, plan, ch, err)
+                                         : run_gemm_persistent<EPI, 1>(specs + g0, ng, m, plan, ch, err);
         if (r != VT_OK) return r;
     }
     return VT_OK;
 }
 
 cudaError_t launch_rmsnorm_rows(const __half* x, const __half* gain, float eps, int rows, int d, __half* y,
-                                int split, cudaStream_t st) {
+                                int split, PrefillChain& ch) {
     if (rows <= 0) return cudaSuccess;
     if (d % 8 != 0 || d > 16384) return cudaErrorInvalidValue;
     const int mc = row_mc(rows, d), t = row_threads(mc, d);
-    return mc == 1 ? launch_pk(k_rmsnorm_rows<1>, dim3(rows), t, 0, 1, st, x, gain, eps, d, y, split)
-                   : launch_pk(k_rmsnorm_rows<2>, dim3(rows), t, 0, 1, st, x, gain, eps, d, y, split);
+    return mc == 1 ? launch_pk(k_rmsnorm_rows<1>, dim3(rows), t, 0, 1, ch, x, gain, eps, d, y, split)
+                   : launch_pk(k_rmsnorm_rows<2>, dim3(rows), t, 0, 1, ch, x, gain, eps, d, y, split);
 }
 
 static vt_status run_rmsnorm(const __half* x, const __half* gain, float eps, int n, int d, __half* y, int split,
-                             cudaStream_t st, std::string* err) {
-    const cudaError_t e = launch_rmsnorm_rows(x, gain, eps, n, d, y, split, st);
+                             PrefillChain& ch, std::string* err) {
+    const cudaError_t e = launch_rmsnorm_rows(x, gain, eps, n, d, y, split, ch);
     if (e != cudaSuccess) {
         *err = std::string("RMSNorm launch failed: ") + cudaGetErrorString(e);
         return VT_ERR_CUDA;
@@ -1658,7 +1665,7 @@ static GemmSpec o_spec(const PrefillAttnArgs& a) {
 }
 
 // Causal attention of every shard of an ATTN block on tcgen05: one launch per kFaGroups shards.
-static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, cudaStream_t st, std::string* err) {
+static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, PrefillChain& ch, std::string* err) {
     for (int g0 = 0; g0 < n; g0 += kFaGroups) {
         const int ng = std::min(kFaGroups, n - g0);
         FaGroup G{};
@@ -1687,8 +1694,8 @@ static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, cudaStre
         G.n_groups = ng;
         if (heads < 1 || as[0].n < 1) continue;
         const dim3 grid(heads, (as[0].n + kFaRows - 1) / kFaRows);
-        const cudaError_t e = as[0].dh == 128 ? launch_pk(k_prefill_attn_tc<128>, grid, kFaThreads, fa_smem<128>(), 1, st, G)
-                                              : launch_pk(k_prefill_attn_tc<64>, grid, kFaThreads, fa_smem<64>(), 1, st, G);
+        const cudaError_t e = as[0].dh == 128 ? launch_pk(k_prefill_attn_tc<128>, grid, kFaThreads, fa_smem<128>(), 1, ch, G)
+                                              : launch_pk(k_prefill_attn_tc<64>, grid, kFaThreads, fa_smem<64>(), 1, ch, G);
         if (e != cudaSuccess) {
             *err = std::string("prefill attention launch failed: ") + cudaGetErrorString(e);
             return VT_ERR_CUDA;
@@ -1698,38 +1705,38 @@ static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, cudaStre
 }
 
 // Causal attention of every shard of an ATTN block (all with the same rows).
-static vt_status prefill_attention(const PrefillAttnArgs* as, int n, cudaStream_t st, std::string* err) {
-    return prefill_attention_tc(as, n, st, err);
+static vt_status prefill_attention(const PrefillAttnArgs* as, int n, PrefillChain& ch, std::string* err) {
+    return prefill_attention_tc(as, n, ch, err);
 }
 
-vt_status prefill_attn_shard(const PrefillAttnArgs& a, cudaStream_t st, std::string* err) {
-    return prefill_attn_group(&a, 1, st, err);
+vt_status prefill_attn_shard(const PrefillAttnArgs& a, PrefillChain& ch, std::string* err) {
+    return prefill_attn_group(&a, 1, ch, err);
 }
 
 // The shards of one ATTN block: one QKV launch for all of them, their attention, one O launch.
 // Every shard has its own q, attention and output buffers; they share the normalised input.
-vt_status prefill_attn_group(const PrefillAttnArgs* a, int n, cudaStream_t st, std::string* err) {
+vt_status prefill_attn_group(const PrefillAttnArgs* a, int n, PrefillChain& ch, std::string* err) {
     if (n < 1) return VT_OK;
     vt_status r;
-    if (!a[0].xhat_ready && (r = run_rmsnorm(a[0].x, a[0].gain, a[0].eps, a[0].n, a[0].d, a[0].xhat, 1, st, err)) != VT_OK)
+    if (!a[0].xhat_ready && (r = run_rmsnorm(a[0].x, a[0].gain, a[0].eps, a[0].n, a[0].d, a[0].xhat, 1, ch, err)) != VT_OK)
         return r;
     GemmSpec specs[VT_MAX_DEVICES];
     for (int i = 0; i < n; ++i) specs[i] = qkv_spec(a[i]);
-    if ((r = run_gemm_group<kGemmQkv>(specs, n, a[0].n, st, err)) != VT_OK) return r;
-    if ((r = prefill_attention(a, n, st, err)) != VT_OK) return r;
+    if ((r = run_gemm_group<kGemmQkv>(specs, n, a[0].n, ch, err)) != VT_OK) return r;
+    if ((r = prefill_attention(a, n, ch, err)) != VT_OK) return r;
     for (int i = 0; i < n; ++i) specs[i] = o_spec(a[i]);
-    return run_gemm_group<kGemmF32>(specs, n, a[0].n, st, err);
+    return run_gemm_group<kGemmF32>(specs, n, a[0].n, ch, err);
 }
 
-vt_status prefill_ffn_shard(const PrefillFfnArgs& a, cudaStream_t st, std::string* err) {
-    return prefill_ffn_group(&a, 1, st, err);
+vt_status prefill_ffn_shard(const PrefillFfnArgs& a, PrefillChain& ch, std::string* err) {
+    return prefill_ffn_group(&a, 1, ch, err);
 }
 
 // The shards of one FFN block: one gate/up (+ SwiGLU) launch and one down launch for all of them.
-vt_status prefill_ffn_group(const PrefillFfnArgs* a, int n, cudaStream_t st, std::string* err) {
+vt_status prefill_ffn_group(const PrefillFfnArgs* a, int n, PrefillChain& ch, std::string* err) {
     if (n < 1) return VT_OK;
     vt_status r;
-    if (!a[0].xhat_ready && (r = run_rmsnorm(a[0].x, a[0].gain, a[0].eps, a[0].n, a[0].d, a[0].xhat, 0, st, err)) != VT_OK)
+    if (!a[0].xhat_ready && (r = run_rmsnorm(a[0].x, a[0].gain, a[0].eps, a[0].n, a[0].d, a[0].xhat, 0, ch, err)) != VT_OK)
         return r;
     GemmSpec specs[VT_MAX_DEVICES];
     for (int i = 0; i < n; ++i) {
@@ -1740,7 +1747,7 @@ vt_status prefill_ffn_group(const PrefillFfnArgs* a, int n, cudaStream_t st, std
         g.status = a[i].status;
         specs[i] = GemmSpec{a[i].xhat, a[i].d, a[i].wgu, a[i].d, 2 * a[i].c, a[i].d, g};
     }
-    if ((r = run_gemm_group<kGemmSwiglu>(specs, n, a[0].n, st, err)) != VT_OK) return r;
+    if ((r = run_gemm_group<kGemmSwiglu>(specs, n, a[0].n, ch, err)) != VT_OK) return r;
     for (int i = 0; i < n; ++i) {
         GemmArgs o{};
         o.c = a[i].out;
@@ -1749,7 +1756,7 @@ vt_status prefill_ffn_group(const PrefillFfnArgs* a, int n, cudaStream_t st, std
         // K runs over the shifted columns [0, ushift + c) of U and the same columns of Wd from wd
         specs[i] = GemmSpec{a[i].u, a[i].ldu, a[i].wd, a[i].wd_ld, a[i].d, a[i].ushift + a[i].c, o};
     }
-    return run_gemm_group<kGemmF32>(specs, n, a[0].n, st, err);
+    return run_gemm_group<kGemmF32>(specs, n, a[0].n, ch, err);
 }
 
 }  // namespace vt

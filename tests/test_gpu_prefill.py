@@ -380,3 +380,34 @@ def test_a_wait_for_what_never_comes_gives_up_after_two_seconds(vtlib, form):
     assert a.elapsed_time(b) < 5000 and (form == 2 or a.elapsed_time(b) > 1900)
     with pytest.raises(vt.VtError):
         vt.vt_test_wait_limit(3, status)
+
+
+def test_thousands_of_prompts_in_a_row(vtlib):
+    """Prompts without a synchronisation between them: the first chunk (1024 rows) runs on CTA pairs, the
+    second (76) on single CTAs; the down projections give a pair three or four tiles of a K that is not
+    in whole k-tiles.  No wait gives up, and the last prompt has the bits of the first."""
+    vt = vtlib
+    rows, L0 = 1100, 37
+    heads, cols = ((0, 2), (2, 4)), ((0, 203), (203, 416))
+    wl = synthetic.small("many", n_layers=1, d_model=7424, n_heads=4, n_kv_heads=4, d_head=128, d_ffn=416,
+                         head_ranges=heads, ffn_ranges=cols, kv_len=L0, decode_steps=0, prompt_len=rows, model_id=149)
+    x = dev(wl.hidden(rows, stream=13))
+    out = [torch.empty_like(x), torch.empty_like(x)]
+    with build(vt, wl, rows + L0) as st:
+        kc, vc = wl.kv_fill(0, L0)
+        for d, (h0, h1) in enumerate(heads):
+            vt.vt_kv_write_raw(st.kv, 0, d, kc[h0:h1], vc[h0:h1])
+        vt.vt_kv_set_length(st.kv, -1, L0)
+
+        def prompts(n, y):
+            for _ in range(n):
+                vt.vt_prefill_tokens(st.part, st.kv, x, rows, y)
+                vt.vt_kv_advance(st.kv, -1, -rows)
+            torch.cuda.synchronize()
+            assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
+
+        prompts(1, out[0])
+        for _ in range(6):  # (the status words are looked at now and then)
+            prompts(500, out[1])
+        assert torch.equal(out[0].view(torch.int16), out[1].view(torch.int16))
+        assert torch.isfinite(out[0].float()).all()
