@@ -35,8 +35,8 @@
 
 namespace vt {
 
-// Launch in the library's chain of programmatic dependent launches: a kernel's CTAs start while the
-// preceding kernel's last CTAs finish.  A launch on CTA pairs (cluster 2) has a whole kernel boundary
+// Launch in the library's chain of programmatic dependent launches: a kernel's CTAs start, and set up
+// their barriers, while the preceding kernel's last CTAs finish.  A launch on CTA pairs (cluster 2) has a whole kernel boundary
 // on both sides: it starts after the launch ahead has ended, as the next one does after it, and its
 // kernel releases no dependents before its CTAs have left (a launch of another call that follows).
 // In the chain, prompts on CTA pairs stopped now and then among thousands, and no cause was found.
@@ -658,6 +658,9 @@ __global__ void __launch_bounds__(kPThreads, 1) k_gemm_p(const __grid_constant__
         s_err = 0;
         fence_mbar_init();
     }
+    // A, the lengths and what the outputs overwrite belong to the preceding kernels.  Tensor memory is
+    // taken after them too: its allocation waits, without a limit, for a kernel that holds it.
+    pdl_wait();
     if (warp == 1) {
         if constexpr (CG == 2) {
             tc::tmem_alloc_pair(tmem_slot, kPTmemCols);
@@ -683,7 +686,6 @@ __global__ void __launch_bounds__(kPThreads, 1) k_gemm_p(const __grid_constant__
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (the whole warp)
-        pdl_wait();  // A was written by the preceding kernel
         if constexpr (CG == 1) pdl_launch_dependents();  // (pairs: launch_pk)
         uint32_t slot = 0, phase = 0, filled = 0;  // ring position; stages filled so far
         // boxes of fewer rows do not fill the ring's copy rate anyway (48-row boxes: 31.2 us without
@@ -883,6 +885,7 @@ __global__ void __launch_bounds__(kPThreads, 1) k_gemm_p(const __grid_constant__
         if constexpr (CG == 2) tc::tmem_dealloc_pair(tmem, kPTmemCols);
         else tc::tmem_dealloc(tmem, kPTmemCols);
     }
+    if constexpr (CG == 2) cluster_sync();  // both halves of the pair's tensor memory are given back
 }
 
 // am: rows of an A box; bn_cta: rows of the B tile one CTA holds (the tile width, or half of it for
@@ -1070,6 +1073,7 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
         *s_err = 0;
         fence_mbar_init();
     }
+    pdl_wait();  // q and the cache rows were written by the preceding kernel, which may hold tensor memory
     if (warp == 1) {
         tc::tmem_alloc(tmem_slot, 512);
         tc::tmem_relinquish();
@@ -1079,7 +1083,6 @@ __global__ void __launch_bounds__(kFaThreads, 1) k_prefill_attn_tc(const __grid_
     tc::fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    pdl_wait();  // q and the cache rows were written by the preceding kernel
     pdl_launch_dependents();
     // Q does not depend on the KV length: its load goes out first
     if (warp == 0 && r0 < a.n) {

@@ -382,15 +382,9 @@ def test_a_wait_for_what_never_comes_gives_up_after_two_seconds(vtlib, form):
         vt.vt_test_wait_limit(3, status)
 
 
-def test_thousands_of_prompts_in_a_row(vtlib):
-    """Prompts without a synchronisation between them: the first chunk (1024 rows) runs on CTA pairs, the
-    second (76) on single CTAs; the down projections give a pair three or four tiles of a K that is not
-    in whole k-tiles.  No wait gives up, and the last prompt has the bits of the first."""
-    vt = vtlib
-    rows, L0 = 1100, 37
-    heads, cols = ((0, 2), (2, 4)), ((0, 203), (203, 416))
-    wl = synthetic.small("many", n_layers=1, d_model=7424, n_heads=4, n_kv_heads=4, d_head=128, d_ffn=416,
-                         head_ranges=heads, ffn_ranges=cols, kv_len=L0, decode_steps=0, prompt_len=rows, model_id=149)
+def _prompts_in_a_row(vt, wl, heads, rows, L0, n):
+    """n prompts without a synchronisation between them, but for a look at the status words now and
+    then: no wait gives up, and the last prompt has the bits of the first."""
     x = dev(wl.hidden(rows, stream=13))
     out = [torch.empty_like(x), torch.empty_like(x)]
     with build(vt, wl, rows + L0) as st:
@@ -407,7 +401,26 @@ def test_thousands_of_prompts_in_a_row(vtlib):
             assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
 
         prompts(1, out[0])
-        for _ in range(6):  # (the status words are looked at now and then)
+        for _ in range(n // 500):
             prompts(500, out[1])
         assert torch.equal(out[0].view(torch.int16), out[1].view(torch.int16))
         assert torch.isfinite(out[0].float()).all()
+
+
+def test_thousands_of_prompts_in_a_row(vtlib):
+    """The first chunk (1024 rows) runs on CTA pairs, the second (76) on single CTAs; the down
+    projections give a pair three or four tiles of a K that is not in whole k-tiles."""
+    heads, cols = ((0, 2), (2, 4)), ((0, 203), (203, 416))
+    wl = synthetic.small("many", n_layers=1, d_model=7424, n_heads=4, n_kv_heads=4, d_head=128, d_ffn=416,
+                         head_ranges=heads, ffn_ranges=cols, kv_len=37, decode_steps=0, prompt_len=1100, model_id=149)
+    _prompts_in_a_row(vtlib, wl, heads, 1100, 37, 3000)
+
+
+@pytest.mark.parametrize("dh,rows", [(64, 5), (64, 128), (128, 77)])
+def test_thousands_of_short_prompts_in_a_row(vtlib, dh, rows):
+    """Single CTAs only, every launch in the dependent chain: GEMMs so small that two of their CTAs, or
+    one and an attention CTA, fit an SM and ask for the whole tensor memory."""
+    heads, cols = ((0, 3), (3, 8)), ((0, 203), (203, 416))
+    wl = synthetic.small("short", n_layers=1, d_model=512, n_heads=8, n_kv_heads=8, d_head=dh, d_ffn=416,
+                         head_ranges=heads, ffn_ranges=cols, kv_len=200, decode_steps=0, prompt_len=rows, model_id=150)
+    _prompts_in_a_row(vtlib, wl, heads, rows, 200, 3000)
