@@ -140,8 +140,7 @@ bool token_plan(const TokArgs& a, int max_hq, TokPlan* plan, std::string* why) {
     slot = std::max<int64_t>(slot, 2 * std::max<int64_t>(table, o_rows * o_spr));
     slot = std::max<int64_t>(slot, a.d);  // the FFN phase stages a D-vector there for its bulk reduction
     if (slot > 16384) return no("too much per-CTA work for the partial-sum slots");
-    // the attention's warp states, with 4 query heads per KV head also their split queries and scales
-    const int uni = std::max(max_hq * a.dh, kTokWarps * a.group * (a.dh + 2) + (a.group == 4 ? a.group * (a.dh + 1) : 0));
+    const int uni = std::max(max_hq * a.dh, kTokWarps * a.group * (a.dh + 2));
     int stages = kTokMaxStages;
     while (stages >= kTokMinStages && token_smem(a, stages, uni, (int)slot) > g_tok_dyn_max[vi]) --stages;
     if (stages < kTokMinStages) return no("not enough shared memory");

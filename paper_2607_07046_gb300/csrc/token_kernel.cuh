@@ -662,229 +662,6 @@ __device__ __forceinline__ Ring attn_slice(const TokArgs& a, const TokShardPtrs*
     return ring;
 }
 
-// Online-softmax attention of one KV head over positions [t0, t1) (EPL = dh / 32 elements per
-// lane, G query heads per KV head), then the warps' states merged into one slice state.
-// The ring state goes in and comes back by value.
-//
-// With 4 query heads per KV head.  What bounds it is instructions (a stage of 64 positions arrives
-// in about 1400 cycles; four heads on the CUDA cores took 11 us for what is read in 2.5), so a warp
-// takes 8 positions at a time and the scores of all G heads come from the tensor cores: MMA rows are
-// the query heads, split into fp16 hi and lo halves of q scaled by the power of two of the head's
-// largest value (an error of 2^-22 of that value, whatever its size), columns the 8 positions.  A
-// lane's share of a K row is whole 16-byte chunks, the k order following the chunks (the queries are
-// laid out the same way); rows of odd positions fetch the two chunks of a pair in the other order, so
-// that the 8 lanes of a shared-memory phase hit 8 different bank groups.  The weights stay fp32 and
-// are passed through shared memory to the sums over V.  Llama-3-8B shapes, 4096 positions, a token
-// of 4 layers: 411 us, 426 with attn_slice; at 46 positions both take 110.  With one query
-// head per KV head the scores are a quarter of that work, and attn_slice is as fast.
-template <int EPL, int G>
-__device__ __forceinline__ Ring attn_slice_mma(const TokArgs& a, const TokShardPtrs* sp, Ring ring, int j, int t0, int t1,
-                                        int seg, int pnew, float* wst, int tid, int warp, int lane) {
-    bool live = ring.live;
-    constexpr int DH = EPL * 32;
-    constexpr int NP = DH / 64;  // pairs of 16-byte chunks of a K row per lane
-    const int s = shard_of_kv(a, j), jl = j - a.kv0[s];
-    const __half* kb = sp[s].kc + (int64_t)jl * a.cap * DH;
-    const __half* vb = sp[s].vc + (int64_t)jl * a.cap * DH;
-    constexpr int np_stage = kTokStageBytes / (4 * DH);
-    static_assert(np_stage % 8 == 0, "a batch of 8 positions stays within its stage");
-    const int old_end = pnew >= 0 ? min(t1, pnew) : t1;
-    const bool has_new = pnew >= t0 && pnew < t1;
-
-    // the queries, scaled and split: warp w < G takes head w; rows g < G hold the hi halves, the next G
-    // the lo halves, and behind them the heads' scales
-    __half* qs = reinterpret_cast<__half*>(wst + 2 * kTokWarps * G + kTokWarps * G * DH);
-    float* qscale = reinterpret_cast<float*>(qs + 2 * G * DH);
-    if (warp < G) {
-        const float* qh = a.q_all + (size_t)(j * G + warp) * DH + lane * EPL;
-        float q[EPL], mx = 0.f;
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) q[e] = __ldcg(qh + e);
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) mx = fmaxf(mx, fabsf(q[e]));
-        mx = warp_max(mx);
-        const int ex = min(max((__float_as_int(mx) >> 23) & 255, 1), 253);
-        const float inv = __int_as_float((254 - ex) << 23);  // 2^(127 - ex)
-        uint32_t* dst = reinterpret_cast<uint32_t*>(qs + warp * DH) + lane * (EPL / 2);
-#pragma unroll
-        for (int e = 0; e < EPL; e += 2) {
-            uint32_t hi, lo;
-            split2(q[e] * inv, q[e + 1] * inv, hi, lo);
-            dst[e / 2] = hi;
-            dst[G * DH / 2 + e / 2] = lo;
-        }
-        if (lane == 0) qscale[warp] = __int_as_float(ex << 23) * a.scale_log2;  // 2^(ex - 127) log2(e) / sqrt(dh)
-    }
-    consumer_bar(1, kTokConsumers);
-    // lane (g, t): MMA row g is head g % G, hi or lo; columns 2t and 2t + 1 are positions
-    const int g = lane >> 2, t = lane & 3, hd = g & (G - 1);
-    const bool odd = g & 1;
-    uint4 qa[NP][2];
-#pragma unroll
-    for (int i = 0; i < NP; ++i)
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-            qa[i][c] = *reinterpret_cast<const uint4*>(qs + (g & (2 * G - 1)) * DH + (i * 8 + c * 4 + t) * 8);
-    const float scale = qscale[hd];
-    float m = -INFINITY, l = 0.f;  // of this lane's head; l: over this lane's positions
-    float o[G][EPL];
-#pragma unroll
-    for (int h = 0; h < G; ++h)
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) o[h][e] = 0.f;
-    // the warp's weights [8 positions][G] and rescales [G], in its part of the states written below
-    float* pw = wst + 2 * kTokWarps * G + warp * G * DH;
-    auto load_lane = [&](const __half* row, float (&dst)[EPL]) {
-        if constexpr (EPL == 4) {
-            const uint2 u = *reinterpret_cast<const uint2*>(row + lane * 4);
-            const float2 f0 = h2_to_f2(u.x), f1 = h2_to_f2(u.y);
-            dst[0] = f0.x; dst[1] = f0.y; dst[2] = f1.x; dst[3] = f1.y;
-        } else {
-            const float2 f0 = h2_to_f2(*reinterpret_cast<const uint32_t*>(row + lane * 2));
-            dst[0] = f0.x; dst[1] = f0.y;
-        }
-    };
-    auto load_heads = [&](const float* src, float (&dst)[G]) {
-        if constexpr (G == 4) {
-            const float4 u = *reinterpret_cast<const float4*>(src);
-            dst[0] = u.x; dst[1] = u.y; dst[2] = u.z; dst[3] = u.w;
-        } else {
-#pragma unroll
-            for (int h = 0; h < G; ++h) dst[h] = src[h];
-        }
-    };
-    for (int tp = t0; tp < old_end; tp += np_stage) {
-        const int n = min(np_stage, old_end - tp);
-        const uint8_t* st = ring_acquire(ring, live, a);
-        if (!st) continue;
-        const __half* kt = reinterpret_cast<const __half*>(st);
-        const __half* vt = reinterpret_cast<const __half*>(st + kTokStageBytes / 2);
-        for (int b0 = warp * 8; b0 < n; b0 += kTokWarps * 8) {
-            // rows past n hold whatever the stage held: their columns are masked below
-            const uint4* kr = reinterpret_cast<const uint4*>(kt + (b0 + g) * DH);
-            float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int i = 0; i < NP; ++i) {
-                const uint4 u = kr[i * 8 + t + (odd ? 4 : 0)], v = kr[i * 8 + t + (odd ? 0 : 4)];
-                mma16816(d0, qa[i][0].x, 0u, qa[i][0].y, 0u, odd ? v.x : u.x, odd ? v.y : u.y);
-                mma16816(d1, qa[i][0].z, 0u, qa[i][0].w, 0u, odd ? v.z : u.z, odd ? v.w : u.w);
-                mma16816(d0, qa[i][1].x, 0u, qa[i][1].y, 0u, odd ? u.x : v.x, odd ? u.y : v.y);
-                mma16816(d1, qa[i][1].z, 0u, qa[i][1].w, 0u, odd ? u.z : v.z, odd ? u.w : v.w);
-            }
-            float sc[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float own = d0[i] + d1[i], other = __shfl_xor_sync(0xffffffffu, own, 4 * G);
-                const float hi = (g & G) ? other : own, lo = (g & G) ? own : other;
-                // an infinite K: the hi half alone has the sign
-                sc[i] = (fabsf(hi) < INFINITY ? hi + lo : hi) * scale;
-                if (b0 + 2 * t + i >= n) sc[i] = -INFINITY;
-            }
-            float mb = fmaxf(sc[0], sc[1]);
-            mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 1));
-            mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 2));
-            mb = fmaxf(mb, m);
-            const float corr = exp2f(m - mb);
-            const float p0 = b0 + 2 * t < n ? exp2f(sc[0] - mb) : 0.f;
-            const float p1 = b0 + 2 * t + 1 < n ? exp2f(sc[1] - mb) : 0.f;
-            l = l * corr + (p0 + p1);
-            const bool rescale = __any_sync(0xffffffffu, m != mb);
-            m = mb;
-            if (g < G) {
-                pw[2 * t * G + g] = p0;
-                pw[(2 * t + 1) * G + g] = p1;
-                if (t == 0) pw[8 * G + g] = corr;
-            }
-            __syncwarp();
-            if (rescale) {
-                float cf[G];
-                load_heads(pw + 8 * G, cf);
-#pragma unroll
-                for (int h = 0; h < G; ++h)
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) o[h][e] *= cf[h];
-            }
-#pragma unroll 4
-            for (int i = 0; i < 8; ++i) {
-                if (b0 + i >= n) break;
-                float vv[EPL], ph[G];
-                load_lane(vt + (b0 + i) * DH, vv);
-                load_heads(pw + i * G, ph);
-#pragma unroll
-                for (int h = 0; h < G; ++h)
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) o[h][e] = fmaf(ph[h], vv[e], o[h][e]);
-            }
-            __syncwarp();  // the weights are read before the next batch's are written
-        }
-        ring_release(ring, lane);
-    }
-    if (has_new && warp == 0 && live) {
-        // the token's own K/V row, appended by the QKV phase of this launch: read through L2
-        float kn[EPL], vn[EPL];
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) {
-            kn[e] = __half2float(__ldcg(kb + (int64_t)pnew * DH + lane * EPL + e));
-            vn[e] = __half2float(__ldcg(vb + (int64_t)pnew * DH + lane * EPL + e));
-        }
-#pragma unroll
-        for (int h = 0; h < G; ++h) {
-            float sc = 0.f;
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) sc = fmaf(__ldcg(a.q_all + (j * G + h) * DH + lane * EPL + e), kn[e], sc);
-            sc = warp_sum(sc) * a.scale_log2;
-            const float mh = __shfl_sync(0xffffffffu, m, 4 * h);
-            const float mn = fmaxf(mh, sc);
-            const float corr = exp2f(mh - mn);
-            const float w = exp2f(sc - mn);
-            if (hd == h) {
-                l = l * corr + (t == 0 ? w : 0.f);
-                m = mn;
-            }
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) o[h][e] = fmaf(o[h][e], corr, w * vn[e]);
-        }
-    }
-    l += __shfl_xor_sync(0xffffffffu, l, 1);
-    l += __shfl_xor_sync(0xffffffffu, l, 2);
-    // per-warp states -> one slice state (warps merged in fixed order)
-    float* wm = wst;                          // [warps][G]
-    float* wl = wm + kTokWarps * G;           // [warps][G]
-    float* wo = wl + kTokWarps * G;           // [warps][G][DH]
-    if (g < G && t == 0) {
-        wm[warp * G + g] = m;
-        wl[warp * G + g] = l;
-    }
-#pragma unroll
-    for (int h = 0; h < G; ++h)
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) wo[(warp * G + h) * DH + lane * EPL + e] = o[h][e];
-    consumer_bar(1, kTokConsumers);
-    float* out = a.states + ((size_t)(blockIdx.x * kTokMaxSeg + seg) * G) * (DH + 4);
-    for (int idx = tid; idx < G * DH; idx += kTokConsumers) {
-        const int h = idx / DH, d = idx - h * DH;
-        float M = -INFINITY;
-        for (int w = 0; w < kTokWarps; ++w) M = fmaxf(M, wm[w * G + h]);
-        float L = 0.f, O = 0.f;
-        if (M != -INFINITY) {
-            for (int w = 0; w < kTokWarps; ++w) {
-                const float f = exp2f(wm[w * G + h] - M);
-                L += wl[w * G + h] * f;
-                O += wo[(w * G + h) * DH + d] * f;
-            }
-        }
-        float* so = out + (size_t)h * (DH + 4);
-        __stcg(so + 4 + d, O);
-        if (d == 0) {
-            __stcg(so, M);
-            __stcg(so + 1, L);
-        }
-    }
-    consumer_bar(1, kTokConsumers);  // the warp states are reused by the next slice
-    ring.live = live;
-    return ring;
-}
-
 // The attention output of shard s (K = its query heads x dh), merged from the slice states with
 // log-sum-exp weights: each thread takes 4 consecutive elements of one query head and issues the
 // loads of 8 slices together (heads cut into more slices take further batches of 8); the result
@@ -1214,10 +991,7 @@ __global__ void __launch_bounds__(kTokThreads, 1) k_decode_token(const __grid_co
         // sliding window: the layer attends to positions [t_lo, n_pos); slices are cut from those
         const int t_lo = window_start(n_pos, a.layer[l].window), n_att = n_pos - t_lo;
         for_kv_pieces(a, n_att, c, NC, [&](int j, int t0, int t1, int seg) {
-            if constexpr (G == 4)
-                ring = attn_slice_mma<dh / 32, G>(a, sp, ring, j, t_lo + t0, t_lo + t1, seg, pnew, uni, tid, warp, lane);
-            else
-                ring = attn_slice<dh / 32, G>(a, sp, ring, j, t_lo + t0, t_lo + t1, seg, pnew, uni, tid, warp, lane);
+            ring = attn_slice<dh / 32, G>(a, sp, ring, j, t_lo + t0, t_lo + t1, seg, pnew, uni, tid, warp, lane);
         });
         live = ring.live;
         // Slice table of every KV head for the O phase: the state offset of each CTA slice of the

@@ -332,3 +332,34 @@ def test_fused_token_four_query_heads_per_kv_head(vtlib, monkeypatch, L0, q_scal
     r = _one_layer_token_with_small_residual(vtlib, wl, 0, L0)
     x, got_out, got_attn, got_ffn, h_ref, xn_ref, ap, fp = r
     _check_partials(wl, got_out, got_attn, got_ffn, x, h_ref, xn_ref, ap, fp, f"L0={L0} q*{q_scale}")
+
+
+def test_fused_token_outlying_query_dimensions(vtlib, monkeypatch):
+    """Four query heads per KV head whose rotated queries have two dimensions about 2^22 times the others,
+    where the keys are zero: the scores come from the small ones alone, which fp32 queries hold in
+    full.  (Two fp16 halves scaled by a head's largest value, here about 2^18, are off by up to 2^-8
+    in every element; times keys of 5 in 126 dimensions over sqrt(128): 1e-2 in a score.)"""
+    wl = synthetic.small("outlier", n_layers=1, d_model=1024, n_heads=4, n_kv_heads=1, d_head=128, d_ffn=1408,
+                         head_ranges=((0, 4),), ffn_ranges=((0, 1408),), kv_len=700, decode_steps=1, prompt_len=0,
+                         model_id=151)
+    weights, fill = type(wl).layer_weights, type(wl).kv_fill
+
+    def scaled_weights(self, layer):
+        w = dict(weights(self, layer))
+        w["wq"], w["wk"] = w["wq"] / np.float16(8), w["wk"] * np.float16(8)
+        for i in (0, 64):  # one RoPE pair
+            w["wq"][i::128] = (w["wq"][i::128].astype(np.float32) * 2.0 ** 22).astype(np.float16)
+            w["wk"][i::128] = 0
+        return w
+
+    def zeroed_fill(self, layer, n_pos, cap=None):
+        k, v = fill(self, layer, n_pos, cap)
+        k = k * np.float16(8)
+        k[..., [0, 64]] = 0
+        return k, v
+
+    monkeypatch.setattr(type(wl), "layer_weights", scaled_weights)
+    monkeypatch.setattr(type(wl), "kv_fill", zeroed_fill)
+    r = _one_layer_token_with_small_residual(vtlib, wl, 0, 700)
+    x, got_out, got_attn, got_ffn, h_ref, xn_ref, ap, fp = r
+    _check_partials(wl, got_out, got_attn, got_ffn, x, h_ref, xn_ref, ap, fp, "outlying dimensions")
