@@ -1624,6 +1624,7 @@ static cudaError_t attn_slices(const vt_partition* p, int l, const int* dev, int
     // tie, so their tokens have the same bits shard by shard and grouped.
     bool quantized = false;
     for (int b : p->comm_bits) quantized |= b != 16;
+    t.window = p->m->window[l];
     const int span = t.window > 0 ? std::min(t.window, kv->cap) : kv->cap;
     t.cluster = attn_cluster_size(hk, t.n, span, quantized);
     // One large fp16 shard: the O projection starts when attention has finished.  Its CTAs that start
@@ -1636,7 +1637,6 @@ static cudaError_t attn_slices(const vt_partition* p, int l, const int* dev, int
     t.early = !(n == 1 && one.bits == 16 && (hk >= 12 || (one.h1 - one.h0) * s.d_head >= 3072));
     t.stages = attn_stages(hk, span, t.cluster, t.early);
     t.scale_log2 = (float)(1.4426950408889634 / sqrt((double)s.d_head));
-    t.window = p->m->window[l];
     t.status = kv->status;
     return launch_attn_decode(t, st);
 }

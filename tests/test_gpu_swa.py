@@ -73,6 +73,29 @@ def test_decode_step_window(vtlib, L, W):
         assert vt.vt_kv_status(st.kv) == 0
 
 
+@pytest.mark.parametrize("H,W", [(2, 40), (2, 256), (2, 257), (10, 1024), (10, 2049), (32, 100), (32, 3072)])
+def test_decode_step_window_bits_do_not_depend_on_the_capacity(vtlib, H, W):
+    """How a windowed layer's attention is cut follows the window, not the cache behind it: the step in
+    a cache just large enough and in one of 7000 positions gives the same bits."""
+    vt = vtlib
+    L = W + 30
+    wl = synthetic.small("swa-cap", n_layers=1, d_model=256, n_heads=H, n_kv_heads=H, d_head=64, d_ffn=64,
+                         head_ranges=((0, H),), ffn_ranges=((0, 64),), kv_len=L, decode_steps=1, prompt_len=0, model_id=152)
+    x = wl.hidden(1, stream=211)
+    got = []
+    for cap in (L + 1, 7000):
+        kc, vc = wl.kv_fill(0, L, cap)
+        with stack(vt, wl, cap, W) as st:
+            fill(vt, st, 0, wl, kc, vc, L)
+            part = torch.empty(wl.d_model, dtype=torch.float32, device="cuda")
+            vt.vt_decode_step(st.part, (0, 0, ATTN), dev(x.reshape(-1)), st.kv, part)
+            got.append(host(part))
+            assert vt.vt_kv_status(st.kv) == 0
+    assert np.array_equal(got[0].view(np.uint32), got[1].view(np.uint32))
+    _, ap = oracle.tp_attention(wl, wl.layer_weights(0), x, L, kc, vc, window=W)
+    assert_close(got[0], ap[0], f"H={H} W={W}")
+
+
 def test_static_step_window(vtlib):
     """The static-scratch step honours the window like vt_decode_step (GQA group 4, dh 128)."""
     vt = vtlib
