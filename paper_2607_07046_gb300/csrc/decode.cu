@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <utility>
 
+#include "deal.h"
 #include "device.cuh"
 #include "internal.h"
 
@@ -85,21 +86,6 @@ static int gemv_cpl(int k) {
         }
     }
     return best;
-}
-
-// Deals `ctas` CTAs out to n shards by their bytes: shard s gets end[s] - end[s - 1], at least enough
-// for its units at `per` units a CTA, at most one per unit.  Returns the launch's CTAs.
-static int deal_ctas(const double* bytes, const int* units, int per, int n, int ctas, int* end) {
-    double tot = 0;
-    for (int s = 0; s < n; ++s) tot += bytes[s];
-    int acc = 0;
-    for (int s = 0; s < n; ++s) {
-        int g = n == 1 ? ctas : (int)(ctas * bytes[s] / tot + 0.5);
-        g = std::min(std::max({g, (units[s] + per - 1) / per, 1}), units[s]);
-        acc += g;
-        end[s] = acc;
-    }
-    return acc;
 }
 
 // The shard of CTA `x` of the launch, and the CTA's number and the CTAs within that shard.
