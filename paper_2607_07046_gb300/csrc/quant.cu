@@ -203,7 +203,8 @@ __device__ __forceinline__ void gemv_q_cta(const QGemvArgs& a, int tile_row) {
     constexpr uint32_t kCode = BITS == 8 ? 512 : 256;  // bytes of a row tile's block
     const uint8_t* const codes = W.codes + lane * (kCode / 32);
     const __half* const scales = W.scales + 2 * g;
-    uint32_t first[MT];  // block 0 of the row tile (32-bit indices: a matrix has at most 2^28 codes)
+    // block 0 of the row tile, in row tiles x blocks (rows * k / 512: at most 3 * 2^19 under the shape limits)
+    uint32_t first[MT];
 #pragma unroll
     for (int m = 0; m < MT; ++m) first[m] = (uint32_t)min(tile0 + m, tiles - 1) * (uint32_t)nb;
     struct Batch {
@@ -559,8 +560,10 @@ static cudaError_t launch_q_epi(const QGemvArgs* a, int n, cudaStream_t st) {
     if (m == 0) return cudaSuccess;
     // Two row tiles a warp halve the instructions a row spends on the input, but also the CTAs: taken
     // where 1.75 CTAs an SM are left.  A token through four 8-bit Llama-2-7B shards (5 to 9 CTAs an SM)
-    // 94 us a layer; through one such shard, which never has more than 2.5 pieces an SM, 141 us a layer
-    // with one row tile a warp against 205 with two.
+    // 94 us a layer; through one such shard (at most 2.5 pieces an SM) 141 us a layer with one row tile a
+    // warp against 205 with two.  A shard alone has 3.5 pieces from 34000 rows on, which only QKV can
+    // have: an ATTN step of 96 heads and 4096 columns, 8 bits, 76 us with two row tiles and 92 with one.
+    // (With two, the compiler spills 56 to 88 bytes a thread at the 80 registers that three CTAs leave.)
     const bool wide = 2 * pieces >= 7 * (g_num_sms > 0 ? g_num_sms : 148);
     if (m == 1) return wide ? launch_q_group<EPI, 1, 2>(sel, m, st) : launch_q_group<EPI, 1, 1>(sel, m, st);
     return wide ? launch_q_group<EPI, VT_MAX_DEVICES, 2>(sel, m, st) : launch_q_group<EPI, VT_MAX_DEVICES, 1>(sel, m, st);

@@ -320,3 +320,52 @@ def test_grouped_token_equals_the_shards_one_after_another(vtlib, d_model, H, Hk
             assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
     assert np.array_equal(outs[0], outs[1])
     assert np.isfinite(outs[0].view(np.float16)).all()
+
+
+@pytest.mark.parametrize("bits", [(8,), (4,), (8, 4, 4)])
+def test_grouped_token_with_two_row_tiles_a_warp(vtlib, bits):
+    """Launches of so many pieces (3.5 an SM or more) that a warp takes two row tiles: one layer of 8B
+    shapes on four shards, D = 4160 and 2 x 3587 or 2 x 3590 gate/up rows leaving the last CTA with half
+    its rows or with one row tile, and parts that its CTAs share unevenly (three of gate/up on two).
+    The token has the bits of the shards one after another (one row tile a warp, fewer than 3.5
+    pieces each) and the oracle's values.  (At most 256 attended positions of 8 KV heads: the
+    attention is cut the same way in both.)"""
+    vt = vtlib
+    heads, cols, L0, cap = (8, 8, 8, 8), (3587, 3580, 3590, 3579), 21, 32
+    hr = tuple((sum(heads[:i]), sum(heads[:i + 1])) for i in range(4))
+    cr = tuple((sum(cols[:i]), sum(cols[:i + 1])) for i in range(4))
+    wl = synthetic.small("wide", n_layers=1, d_model=4160, n_heads=32, n_kv_heads=8, d_head=128, d_ffn=sum(cols),
+                         head_ranges=hr, ffn_ranges=cr, kv_len=L0, decode_steps=1, prompt_len=0, model_id=153)
+    prec = {b: [bits[(2 * d + b) % len(bits)] for d in range(4)] for b in (ATTN, FFN)}
+    x = wl.hidden(1, stream=17)
+    outs = []
+    for step in (vt.vt_decode_token, vt.vt_decode_token_sharded):
+        kc, vc = wl.kv_fill(0, L0, cap)
+        with stack(vt, wl, cap, precision=lambda l, d, b: prec[b][d]) as st:
+            for d, r in enumerate(hr):
+                k0, k1 = kv_range(wl, r)
+                vt.vt_kv_write_raw(st.kv, 0, d, kc[k0:k1, :L0], vc[k0:k1, :L0])
+            vt.vt_kv_set_length(st.kv, -1, L0)
+            y = torch.empty(wl.d_model, dtype=torch.float16, device="cuda")
+            step(st.part, st.kv, dev(x.reshape(-1)), y)
+            outs.append(host(y))
+            assert vt.vt_kv_status(st.kv) == 0 and vt.vt_partition_status(st.part) == 0
+    assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
+    _, ref, _, _ = oracle.tp_layer_mixed(wl, wl.layer_weights(0), x, L0, kc, vc, prec[ATTN], prec[FFN])
+    assert_close(outs[0], ref.reshape(-1), f"two row tiles a warp, {bits}")
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+def test_one_shard_with_two_row_tiles_a_warp(vtlib, bits):
+    """One shard of 179 heads: its 34368 QKV rows are 537 pieces, and the last CTA has half its rows."""
+    vt = vtlib
+    L, cap = 9, 16
+    wl = synthetic.small("lone", n_layers=1, d_model=192, n_heads=179, n_kv_heads=179, d_head=64, d_ffn=70,
+                         head_ranges=((0, 179),), ffn_ranges=((0, 70),), kv_len=L, decode_steps=1, prompt_len=0, model_id=154)
+    w = wl.layer_weights(0)
+    kc, vc = wl.kv_fill(0, L, cap)
+    with stack(vt, wl, cap, precision=lambda l, d, b: bits) as st:
+        vt.vt_kv_write_raw(st.kv, 0, 0, kc[:, :L], vc[:, :L])
+        vt.vt_kv_set_length(st.kv, 0, L)
+        _shard_checks(vt, st, wl, w, 0, wl.hidden(1, stream=18), L, kc, vc, [bits], [bits], f"179 heads, {bits} bits")
+        assert vt.vt_kv_status(st.kv) == 0
