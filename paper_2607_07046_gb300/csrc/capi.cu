@@ -1543,10 +1543,11 @@ extern "C" vt_status vt_kv_write_raw(vt_kv* kv, int32_t l, int32_t d, int32_t n_
 
 // ================================================================== shard compute
 
-// QKV projection of ATTN shard (l, d) with RoPE and the K/V append at the layer's length: the
 // One phase of a block of layer l: the block-quantized shards of `dev` (n devices, none empty) in one
-// launch, the fp16 ones in another, whose input is then at least two launches old: it streams
-// beside the first.  Both kinds of arguments are filled in from the same description of the phase.
+// launch, the fp16 ones in another.  The quantized launch releases its dependents only after its own
+// wait, so the phase's input is complete when the fp16 one starts: it reads it at once (`indep`) and
+// streams beside the first.  Both kinds of arguments are filled in from the same description of the
+// phase.
 struct DecodePhase {
     GemvArgs g[VT_MAX_DEVICES];
     QGemvArgs q[VT_MAX_DEVICES];

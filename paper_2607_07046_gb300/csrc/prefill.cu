@@ -208,8 +208,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// The wait with the loaded registers as operands, so that no use of them is scheduled before it.
+// The wait for the loads, with the loaded registers as operands: no use of them is scheduled before it.
 __device__ __forceinline__ void tmem_ld_wait_on(uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
@@ -1667,8 +1666,9 @@ static GemmSpec o_spec(const PrefillAttnArgs& a) {
     return GemmSpec{a.attn, K, a.wo, K, a.d, K, o};
 }
 
-// Causal attention of every shard of an ATTN block on tcgen05: one launch per kFaGroups shards.
-static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, PrefillChain& ch, std::string* err) {
+// Causal attention of every shard of an ATTN block (all with the same rows): one launch per kFaGroups
+// shards.
+static vt_status prefill_attention(const PrefillAttnArgs* as, int n, PrefillChain& ch, std::string* err) {
     for (int g0 = 0; g0 < n; g0 += kFaGroups) {
         const int ng = std::min(kFaGroups, n - g0);
         FaGroup G{};
@@ -1705,11 +1705,6 @@ static vt_status prefill_attention_tc(const PrefillAttnArgs* as, int n, PrefillC
         }
     }
     return VT_OK;
-}
-
-// Causal attention of every shard of an ATTN block (all with the same rows).
-static vt_status prefill_attention(const PrefillAttnArgs* as, int n, PrefillChain& ch, std::string* err) {
-    return prefill_attention_tc(as, n, ch, err);
 }
 
 vt_status prefill_attn_shard(const PrefillAttnArgs& a, PrefillChain& ch, std::string* err) {

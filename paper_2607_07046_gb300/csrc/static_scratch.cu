@@ -26,10 +26,11 @@ static size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 StaticAttnLayout static_attn_layout(int hq, int hk, int dh) {
     StaticAttnLayout L{};
-    L.q = round256((size_t)kStaticMaxKvHeads * 4);
-    L.attn = L.q + round256((size_t)hq * dh * 4);
-    // the call's published limit: room for 16 slice states (max, sum, weighted V) per KV head
-    const size_t end = L.attn + round256((size_t)hq * dh * 4);
+    L.q = 0;
+    L.attn = round256((size_t)hq * dh * 4);
+    // the call's published limit: 256 bytes and 16 slice states (max, sum, weighted V) per KV head more
+    // than the two vectors take
+    const size_t end = 256 + 2 * L.attn;
     const size_t group = (size_t)(hk > 0 ? hq / hk : 1), states = (size_t)hk * kStaticSplits * group;
     L.bytes = end + round256(states * 2 * 4) + round256(states * (size_t)dh * 4);
     return L;
