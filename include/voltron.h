@@ -510,7 +510,9 @@ VT_API vt_status vt_partition_set_comm_bits(vt_partition* part, int32_t device, 
  *   precision).  Its results have the same bits as vt_decode_token_sharded's, except that an
  *   attention launch of several shards may cut the cached positions into fewer slices (the sums
  *   then differ in fp32 rounding; never while partials are quantized), and that fp16 FFN shards
- *   add their partial in arrival order in both.
+ *   add their partial in arrival order in both.  How many slices an attention launch takes follows
+ *   from its KV heads and from the layer's window or the capacity of the cache, so a cache of
+ *   another capacity may give another fp32 rounding.
  *   The launch can be captured in a CUDA graph.
  */
 VT_API vt_status vt_decode_token(const vt_partition* part, vt_kv* kv, const void* x_in, void* x_out,
